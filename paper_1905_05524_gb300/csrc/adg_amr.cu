@@ -372,41 +372,47 @@ __device__ __forceinline__ Phys leaf_phys(const Phys& P0, const double* geo, int
 }
 
 // ------------------------------------------------------------------ kernels
-template <int N, int CPB>
-__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
-k_predictor_amr(const double* __restrict__ u, double* __restrict__ rvol, double* __restrict__ trace, int cells,
-                double dt, const Basis B, const Phys P0, const double* __restrict__ geo,
-                const double* __restrict__ bgl) {
-    constexpr int n = N + 1, n2 = n * n;
+// FP64 predictor on the leaves [first, end): all of them, or one level's with
+// its own dt (local time stepping; REC adds the per-time-node face traces).
+// Leaves are ordered by level, so a block meets few changes of cell size.
+template <int N, bool REC>
+__global__ void __launch_bounds__(FxCfg<N>::threads, FxCfg<N>::resident)
+k_predictor_amr(const double* __restrict__ u, double* __restrict__ rvol, double* __restrict__ trace, int first, int end,
+                double dt, const Basis B, const Phys P0, const double* __restrict__ geo, const int* __restrict__ nbr,
+                const double* __restrict__ bgl, double* __restrict__ ttrace) {
+    using C = FxCfg<N>;
     extern __shared__ double sm[];
-    const int cl = threadIdx.x / n2;
-    const int j = (threadIdx.x - cl * n2) / n;
-    const int cell_raw = blockIdx.x * CPB + cl;
-    const bool active = cell_raw < cells;
-    const int cell = active ? cell_raw : cells - 1;
-    const Phys P = leaf_phys(P0, geo, cell, N);
-    predictor_fp64_body<N, CPB>(u, rvol, trace, cell, active, dt, B, P, geo[cell * 4], geo[cell * 4 + 1],
-                                bgl[((size_t)cell * n + j) * 2], bgl[((size_t)cell * n + j) * 2 + 1], sm);
+    const int cl = threadIdx.x / C::tpc, tid = threadIdx.x - cl * C::tpc;
+    const int j = min(tid, C::n3 - 1) % C::n2 / C::n;
+    Limbs* K = reinterpret_cast<Limbs*>(sm + (size_t)C::cpb * C::words(false));
+    fx_time_table<N>(K, B);
+    FxRows<N> O;
+    Phys P;
+    P.hx = P.hy = 0.0;
+    for (int c0 = first + blockIdx.x * C::cpb; c0 < end; c0 += gridDim.x * C::cpb) {
+        const bool active = c0 + cl < end;
+        const int cell = active ? c0 + cl : end - 1;
+        const double4 ge = *reinterpret_cast<const double4*>(geo + (size_t)cell * 4);
+        if (ge.z != P.hx || ge.w != P.hy) {
+            P = leaf_phys(P0, geo, cell, N);
+            O.make(B, fx_tab<N, false>(sm, cl), tid, P.inv_hx, P.inv_hy);
+        }
+        unsigned gmask = 0;
+#pragma unroll
+        for (int f = 0; f < 4; ++f) gmask |= nbr[((size_t)cell * 4 + f) * kNbrInts] == NB_WALL ? 1u << f : 0u;
+        predictor_fp64_body<N, false, REC>(u, rvol, trace, cell, active, tid, dt, B, P, O, K, ge.x, ge.y,
+                                           bgl[((size_t)cell * C::n + j) * 2], bgl[((size_t)cell * C::n + j) * 2 + 1],
+                                           gmask, sm + (size_t)cl * C::words(false), 0.0, ttrace);
+    }
 }
 
-// Local time stepping: the FP64 predictor on the leaf range [first, end) (one
-// level) with dt of that level; REC adds the per-time-node face traces.
-template <int N, int CPB, bool REC>
-__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
-k_predictor_amr_lts(const double* __restrict__ u, double* __restrict__ rvol, double* __restrict__ trace, int first,
-                    int end, double dt, const Basis B, const Phys P0, const double* __restrict__ geo,
-                    const double* __restrict__ bgl, double* __restrict__ ttrace) {
-    constexpr int n = N + 1, n2 = n * n;
-    extern __shared__ double sm[];
-    const int cl = threadIdx.x / n2;
-    const int j = (threadIdx.x - cl * n2) / n;
-    const int cell_raw = first + blockIdx.x * CPB + cl;
-    const bool active = cell_raw < end;
-    const int cell = active ? cell_raw : end - 1;
-    const Phys P = leaf_phys(P0, geo, cell, N);
-    predictor_fp64_body<N, CPB, false, REC>(u, rvol, trace, cell, active, dt, B, P, geo[cell * 4], geo[cell * 4 + 1],
-                                            bgl[((size_t)cell * n + j) * 2], bgl[((size_t)cell * n + j) * 2 + 1],
-                                            sm, 0.0, ttrace);
+template <int N, bool REC>
+static cudaError_t launch_predictor_amr(adg_mesh* m, int first, int end, double dt, cudaStream_t s) {
+    using C = FxCfg<N>;
+    static_assert(C::smem(false) <= 48 * 1024, "within the default shared-memory limit");
+    k_predictor_amr<N, REC><<<fx_grid((end - first + C::cpb - 1) / C::cpb, C::resident), C::threads, C::smem(false), s>>>(
+        m->u, m->rvol, m->trace, first, end, dt, m->B, m->P, m->geo, m->nbr, m->bgl, REC ? m->lts_ttrace : nullptr);
+    return cudaGetLastError();
 }
 
 // Mixed-precision predictor of the adaptive mesh: the Picard iteration of
@@ -1033,7 +1039,6 @@ struct AmrCfg {
     static constexpr int n = N + 1;
     static constexpr int cpb = tv_cpb(N);
     static constexpr int threads = cpb * n * n;
-    static constexpr size_t smem_pred = (size_t)cpb * 3 * n * 4 * n * n * sizeof(double);
 };
 
 #define AMR_DISPATCH(FN, ...)                     \
@@ -1059,7 +1064,6 @@ constexpr int amr_mixed_cpb() {
 
 template <int N>
 static int pred_n(adg_mesh* m, double dt, cudaStream_t s) {
-    using C = AmrCfg<N>;
     if (m->d.precision == ADG_PREC_MIXED) {
         constexpr int CM = amr_mixed_cpb<N>();
         auto km = k_predictor_amr_mixed<N, CM>;
@@ -1071,11 +1075,7 @@ static int pred_n(adg_mesh* m, double dt, cudaStream_t s) {
         ADG_CK(cudaGetLastError(), "amr mixed predictor launch");
         return ADG_OK;
     }
-    auto kern = k_predictor_amr<N, C::cpb>;
-    ADG_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_pred), "amr pred");
-    kern<<<(m->cells + C::cpb - 1) / C::cpb, C::threads, C::smem_pred, s>>>(m->u, m->rvol, m->trace, m->cells, dt,
-                                                                             m->B, m->P, m->geo, m->bgl);
-    ADG_CK(cudaGetLastError(), "amr predictor launch");
+    ADG_CK((launch_predictor_amr<N, false>(m, 0, m->cells, dt, s)), "amr predictor launch");
     return ADG_OK;
 }
 int amr_predictor(adg_mesh* m, double dt, void* stream) { AMR_DISPATCH(pred_n, m, dt, (cudaStream_t)stream) }
@@ -1161,18 +1161,9 @@ static int lts_level_n(LtsRun& R, int l, double t, int kstep) {
     (void)t;
     if (end > first) {
         const int blocks = (end - first + C::cpb - 1) / C::cpb;
-        if (finer) {
-            auto k = k_predictor_amr_lts<N, C::cpb, true>;
-            ADG_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_pred), "lts pred");
-            k<<<blocks, C::threads, C::smem_pred, R.s>>>(m->u, m->rvol, m->trace, first, end, dtl, m->B, m->P, m->geo,
-                                                          m->bgl, m->lts_ttrace);
-        } else {
-            auto k = k_predictor_amr_lts<N, C::cpb, false>;
-            ADG_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_pred), "lts pred");
-            k<<<blocks, C::threads, C::smem_pred, R.s>>>(m->u, m->rvol, m->trace, first, end, dtl, m->B, m->P, m->geo,
-                                                          m->bgl, nullptr);
-        }
-        ADG_CK(cudaGetLastError(), "lts predictor launch");
+        ADG_CK((finer ? launch_predictor_amr<N, true>(m, first, end, dtl, R.s)
+                      : launch_predictor_amr<N, false>(m, first, end, dtl, R.s)),
+               "lts predictor launch");
     }
     if (finer) {
         const size_t per_leaf = (size_t)4 * 3 * 4 * m->n;

@@ -143,7 +143,32 @@ bool adg::build_basis(int N, adg::Basis& B) {
         B.Kw1[l] = s;
     }
     for (int p = 0; p < n; ++p)
-        for (int i = 0; i < n; ++i) B.Vx[p][i] = B.w[p] * B.D[p][i] / B.w[i];
+        for (int i = 0; i < n; ++i) {
+            B.Vx[p][i] = B.w[p] * B.D[p][i] / B.w[i];
+            B.dphi0[i] += B.phi0[p] * B.D[p][i];
+            B.dphi1[i] += B.phi1[p] * B.D[p][i];
+        }
+    for (int i = 0; i < n; ++i) {
+        double row = 0.0;
+        for (int j = 0; j < n; ++j) {
+            row += std::fabs(B.D[i][j]);
+            B.Dmax = std::fmax(B.Dmax, std::fabs(B.D[i][j]));
+        }
+        B.Drow = std::fmax(B.Drow, row * (1.0 + 1e-9));
+    }
+    double big = 0.0;
+    for (int l = 0; l < n; ++l)
+        for (int k = 0; k < n; ++k) big = std::fmax(big, std::fabs(B.Kw[l][k]));
+    int e = 0;
+    std::frexp(big, &e);  // |Kw| < 2^e
+    B.KwE = e + 1022;
+    for (int l = 0; l < n; ++l)
+        for (int k = 0; k < n; ++k) {
+            const long long m = std::llrint(std::ldexp(B.Kw[l][k], 58 - e));
+            const long long h = (m + (1ll << 28)) >> 29;
+            B.KwH[l][k] = (int)h;
+            B.KwL[l][k] = (int)(m - h * (1ll << 29));
+        }
     return true;
 }
 

@@ -15,12 +15,11 @@
 // on its 4 faces (neighbour traces, or a slip-wall ghost, Eq. 10) and the
 // FP64 update u += dt (rvol - lift(F*)).
 //
-// Thread mapping: CPB cells per block, one thread per spatial node (j, i) of
-// a cell; each thread loops over the n time nodes of its node column, so the
-// time contraction of the Picard update stays in registers.  The space-time
-// tensor of a cell (q, F, G: 3 x n^3 x 4 doubles) lives in shared memory.
-// FP64 arithmetic is the binding resource on this part, so the first sweep
-// (whose iterate is constant in time) evaluates the fluxes once, not n times.
+// Thread mapping: adg_fp64_body.cuh (predictor, one thread per space-time
+// node); the corrector runs one thread per spatial node, CPB cells per block.
+// FP64 arithmetic is the binding resource on this part, so the predictor's
+// contractions run on the integer pipe (adg_fixed.cuh) and its first sweep,
+// whose iterate is constant in time, evaluates the fluxes once, not n times.
 #include <cuda_runtime.h>
 
 #include "adg_internal.h"
@@ -36,25 +35,37 @@ struct Fp64Cfg {
     // cells per block: enough threads per block for small degrees
     static constexpr int cpb = tv_cpb(N);
     static constexpr int threads = cpb * n * n;
-    static constexpr size_t smem_pred = (size_t)cpb * 3 * n * 4 * n * n * sizeof(double);
 };
 
-template <int N, int CPB, bool TSRC>
-__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
+// Boundary sides of cell (ix, iy) as a face mask (E, W, N, S).
+__device__ __forceinline__ unsigned edge_faces(int ix, int iy, const Phys& P) {
+    unsigned m = 0;
+    if (P.bc_x != ADG_BC_PERIODIC) m |= (ix == P.nx - 1 ? 1u : 0u) | (ix == 0 ? 2u : 0u);
+    if (P.bc_y != ADG_BC_PERIODIC) m |= (iy == P.ny - 1 ? 4u : 0u) | (iy == 0 ? 8u : 0u);
+    return m;
+}
+
+template <int N, bool TSRC>
+__global__ void __launch_bounds__(FxCfg<N>::threads, FxCfg<N>::resident)
 k_predictor_fp64(const double* __restrict__ u, double* __restrict__ rvol,
                  double* __restrict__ trace, int cells, double dt, double t,
                  const Basis B, const Phys P, const Background bg) {
-    constexpr int n = N + 1, n2 = n * n;
+    using C = FxCfg<N>;
     extern __shared__ double sm[];
-    const int cl = threadIdx.x / n2;
-    const int j = (threadIdx.x - cl * n2) / n;
-    const int cell_raw = blockIdx.x * CPB + cl;
-    const bool active = cell_raw < cells;
-    const int cell = active ? cell_raw : cells - 1;
-    const int ix = cell % P.nx, iy = cell / P.nx;
-    predictor_fp64_body<N, CPB, TSRC>(u, rvol, trace, cell, active, dt, B, P, P.x0 + ix * P.hx,
-                                      P.y0 + iy * P.hy, bg.pbar_node[iy * n + j], bg.rhobar_node[iy * n + j],
-                                      sm, t);
+    const int cl = threadIdx.x / C::tpc, tid = threadIdx.x - cl * C::tpc;
+    const int j = min(tid, C::n3 - 1) % C::n2 / C::n;
+    Limbs* K = reinterpret_cast<Limbs*>(sm + (size_t)C::cpb * C::words(TSRC));
+    fx_time_table<N>(K, B);
+    FxRows<N> O;
+    O.make(B, fx_tab<N, TSRC>(sm, cl), tid, P.inv_hx, P.inv_hy);
+    for (int c0 = blockIdx.x * C::cpb; c0 < cells; c0 += gridDim.x * C::cpb) {
+        const bool active = c0 + cl < cells;
+        const int cell = active ? c0 + cl : cells - 1;
+        const int ix = cell % P.nx, iy = cell / P.nx;
+        predictor_fp64_body<N, TSRC>(u, rvol, trace, cell, active, tid, dt, B, P, O, K, P.x0 + ix * P.hx,
+                                     P.y0 + iy * P.hy, bg.pbar_node[iy * C::n + j], bg.rhobar_node[iy * C::n + j],
+                                     edge_faces(ix, iy, P), sm + (size_t)cl * C::words(TSRC), t);
+    }
 }
 
 // Slip-wall ghost of face f (0 E, 1 W, 2 N, 3 S) from the interior trace
@@ -271,25 +282,33 @@ k_corrector_fp64(double* __restrict__ u, const double* __restrict__ rvol,
 
 // Batched persistent FP64 kernels over uniform instances (tile = instance,
 // first cell; tile t goes to block t mod grid): the per-mesh bodies.
-template <int N, int CPB>
-__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
+template <int N>
+__global__ void __launch_bounds__(FxCfg<N>::threads, FxCfg<N>::resident)
 k_predictor_batch_fp64(const Fp64Inst* __restrict__ insts, const BatchTile* __restrict__ tiles, int ntiles,
                        const Basis B) {
-    constexpr int n = N + 1, n2 = n * n;
+    using C = FxCfg<N>;
     extern __shared__ double sm[];
-    const int cl = threadIdx.x / n2;
-    const int j = (threadIdx.x - cl * n2) / n;
-    for (int tt = blockIdx.x; tt < ntiles; tt += gridDim.x) {
+    const int cl = threadIdx.x / C::tpc, tid = threadIdx.x - cl * C::tpc;
+    const int j = min(tid, C::n3 - 1) % C::n2 / C::n;
+    Limbs* K = reinterpret_cast<Limbs*>(sm + (size_t)C::cpb * C::words(false));
+    fx_time_table<N>(K, B);
+    FxRows<N> O;
+    Phys P;
+    for (int tt = blockIdx.x, last = -1; tt < ntiles; tt += gridDim.x) {
         const BatchTile tl = tiles[tt];
         const Fp64Inst& I = insts[tl.inst];
-        const Phys P = I.P;
+        if (tl.inst != last) {
+            P = I.P;
+            O.make(B, fx_tab<N, false>(sm, cl), tid, P.inv_hx, P.inv_hy);
+            last = tl.inst;
+        }
         const int cell_raw = tl.c0 + cl;
         const bool active = cell_raw < I.cells;
         const int cell = active ? cell_raw : I.cells - 1;
         const int ix = cell % P.nx, iy = cell / P.nx;
-        predictor_fp64_body<N, CPB>(I.u, I.rvol, I.trace, cell, active, I.dt, B, P, P.x0 + ix * P.hx,
-                                    P.y0 + iy * P.hy, I.bg.pbar_node[iy * n + j], I.bg.rhobar_node[iy * n + j], sm);
-        __syncthreads();
+        predictor_fp64_body<N>(I.u, I.rvol, I.trace, cell, active, tid, I.dt, B, P, O, K, P.x0 + ix * P.hx,
+                               P.y0 + iy * P.hy, I.bg.pbar_node[iy * C::n + j], I.bg.rhobar_node[iy * C::n + j],
+                               edge_faces(ix, iy, P), sm + (size_t)cl * C::words(false));
     }
 }
 
@@ -311,18 +330,16 @@ template <int N>
 static int batch_fp64_n(int phase, const Fp64Inst* insts, const BatchTile* tiles, int ntiles, const Basis& B,
                         int* cpb_out, int* blocks_io, cudaStream_t s) {
     using C = Fp64Cfg<N>;
-    if (cpb_out) *cpb_out = C::cpb;
+    using F = FxCfg<N>;
+    if (cpb_out) *cpb_out = phase == 0 ? F::cpb : C::cpb;
     if (!tiles) {  // query: smem limit and persistent grid (not during capture)
         int per_sm = 0, dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cudaError_t e;
         if (phase == 0) {
-            e = cudaFuncSetAttribute(k_predictor_batch_fp64<N, C::cpb>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)C::smem_pred);
-            if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_predictor_batch_fp64<N, C::cpb>,
-                                                                  C::threads, C::smem_pred);
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_predictor_batch_fp64<N>, F::threads,
+                                                              F::smem(false));
         } else {
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_corrector_batch_fp64<N, C::cpb>, C::threads,
                                                               0);
@@ -332,7 +349,7 @@ static int batch_fp64_n(int phase, const Fp64Inst* insts, const BatchTile* tiles
         return 0;
     }
     if (phase == 0)
-        k_predictor_batch_fp64<N, C::cpb><<<*blocks_io, C::threads, C::smem_pred, s>>>(insts, tiles, ntiles, B);
+        k_predictor_batch_fp64<N><<<*blocks_io, F::threads, F::smem(false), s>>>(insts, tiles, ntiles, B);
     else
         k_corrector_batch_fp64<N, C::cpb><<<*blocks_io, C::threads, 0, s>>>(insts, tiles, ntiles, B);
     return (int)cudaGetLastError();
@@ -353,18 +370,27 @@ int launch_batch_fp64(int N, int phase, const Fp64Inst* insts, const BatchTile* 
     return (int)cudaErrorInvalidValue;
 }
 
+template <int N, bool TSRC>
+static int launch_pred_src(const double* u, double* rvol, double* trace, int cells, double dt, double t, const Basis& B,
+                           const Phys& P, const Background& bg, cudaStream_t s) {
+    using C = FxCfg<N>;
+    static_assert(C::smem(TSRC) <= 48 * 1024 || N == 7, "within the default shared-memory limit");
+    auto kern = k_predictor_fp64<N, TSRC>;
+    if (C::smem(TSRC) > 48 * 1024) {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem(TSRC));
+        if (e != cudaSuccess) return (int)e;
+    }
+    kern<<<fx_grid((cells + C::cpb - 1) / C::cpb, C::resident), C::threads, C::smem(TSRC), s>>>(u, rvol, trace, cells, dt,
+                                                                                           t, B, P, bg);
+    return (int)cudaGetLastError();
+}
+
 template <int N>
 static int launch_pred(const double* u, double* rvol, double* trace, int cells, double dt,
                        double t, const Basis& B, const Phys& P, const Background& bg,
                        cudaStream_t s) {
-    using C = Fp64Cfg<N>;
-    auto kern = P.source == ADG_SRC_PAPER ? k_predictor_fp64<N, C::cpb, true> : k_predictor_fp64<N, C::cpb, false>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)C::smem_pred);
-    if (e != cudaSuccess) return (int)e;
-    const int blocks = (cells + C::cpb - 1) / C::cpb;
-    kern<<<blocks, C::threads, C::smem_pred, s>>>(u, rvol, trace, cells, dt, t, B, P, bg);
-    return (int)cudaGetLastError();
+    return P.source == ADG_SRC_PAPER ? launch_pred_src<N, true>(u, rvol, trace, cells, dt, t, B, P, bg, s)
+                                     : launch_pred_src<N, false>(u, rvol, trace, cells, dt, t, B, P, bg, s);
 }
 
 template <int N>

@@ -25,6 +25,11 @@ struct Basis {
     double Vx[kMaxN][kMaxN];  // Vx[p][i] = w_p D[p][i] / w_i (weak volume term)
     double lift0[kMaxN];      // phi_i(0) / w_i
     double lift1[kMaxN];      // phi_i(1) / w_i
+    double dphi0[kMaxN];      // phi_j'(0)
+    double dphi1[kMaxN];      // phi_j'(1)
+    // Kw in fixed point (adg_fixed.cuh): Kw = (KwH 2^29 + KwL) 2^(KwE - 1080)
+    int KwH[kMaxN][kMaxN], KwL[kMaxN][kMaxN], KwE;
+    double Dmax, Drow;        // largest |D[i][j]|; an upper bound of the rows' sums of |D|
 };
 
 // Physical and mesh constants of one mesh.
