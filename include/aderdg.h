@@ -284,7 +284,7 @@ int adg_check_finite(adg_mesh* m, void* stream);
  * captures the graph again.
  * adg_batch_create times the predictor's candidates on the batch -- three
  * tile sizes of the node-per-thread body and, for batches of uniform
- * instances at degrees 3 and 5, the node-pair body (two nodes per thread) --
+ * instances at degrees 3, 5 and 7, the node-pair body (two nodes per thread) --
  * and keeps the fastest, cached per (degree, precision, SM count, size class,
  * number of candidates, adaptive or not) in memory and in a JSON file:
  * $ADG_TUNE_CACHE if set (an empty value keeps the cache in memory only),
@@ -318,7 +318,7 @@ int adg_batch_step(adg_batch* b, const double* dt, int nsteps, void* stream);
 int adg_batch_info(const adg_batch* b, int* info, int n);
 /* Pins the predictor's candidate (0, 1 or 2: half, default and double the
  * per-mesh node-per-thread cells per block; 3: the node-pair body with its
- * per-mesh cells per block at degrees 3 and 5 in a batch without adaptive
+ * per-mesh cells per block at degrees 3, 5 and 7 in a batch without adaptive
  * instances, candidate 1 otherwise) instead of the timed choice, e.g. to
  * reproduce a run or to test every candidate.  Synchronises the device
  * (the previous tile list may be in use by a launched step), rebuilds the

@@ -424,14 +424,14 @@ static cudaError_t launch_predictor_amr(adg_mesh* m, int first, int end, double 
 // the node's row, which does not vary along x; y-faces: the FP64
 // extrapolation of the leaf's nodal background) with the Rusanov speed in
 // FP32 -- so the FP64 corrector with its hanging faces runs unchanged.
-// Shared memory of the mixed adaptive predictor per leaf: q', F and G as
-// float2 pairs of time slices, padded to a bank offset of 16 (mod 32 floats)
+// Shared memory of the mixed adaptive predictor per leaf: q' (4), F and G (3
+// each: the mass fluxes are momenta) as float2 pairs of time slices, padded to a bank offset of 16 (mod 32 floats)
 // between neighbouring leaves.
 template <int N>
 struct AmrMixCfg {
     static constexpr int n = N + 1;
     static constexpr int npair = (n + 1) / 2;
-    static constexpr int raw = 3 * npair * 4 * n * n * 2;
+    static constexpr int raw = npair * 10 * n * n * 2;
     static constexpr int stride = raw + ((16 - raw % 32) + 32) % 32;
 };
 
@@ -446,6 +446,7 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
                                                          double* __restrict__ trace, int cells, int c0, float dt,
                                                          const BasisF& B, const PhysF& P,
                                                          const double* __restrict__ geo,
+                                                         const int* __restrict__ nbr,
                                                          const double* __restrict__ mb64,
                                                          const float* __restrict__ mbf, float* smf) {
     constexpr int n = N + 1, n2 = n * n, SL = 4 * n2;
@@ -458,7 +459,11 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
     constexpr int NPAIR = AmrMixCfg<N>::npair, PS = 4 * n2;  // slice pairs, pair stride (float2)
     float2* Q2 = reinterpret_cast<float2*>(smf + (size_t)cl * AmrMixCfg<N>::stride);  // [h][v][j][i]
     float2* F2 = Q2 + NPAIR * PS;                                                      // [h][v][j][i]
-    float2* G2 = F2 + NPAIR * PS;                                                      // [h][v][j][i]
+    constexpr int FS = 3 * n2;                                                         // pair stride of F, G
+    float2* G2 = F2 + NPAIR * FS;                                                      // [h][v - 1][j][i]
+    unsigned wf = 0;  // wall faces: grad q-bar is read there only
+#pragma unroll
+    for (int f = 0; f < 4; ++f) wf |= nbr[((size_t)cell * 4 + f) * kNbrInts] == NB_WALL ? 1u << f : 0u;
     const double hx = geo[cell * 4 + 2], hy = geo[cell * 4 + 3], yorg = geo[cell * 4 + 1];
     const float inv_hx = (float)(1.0 / hx), inv_hy = (float)(1.0 / hy);
     const float z = (float)(yorg + (double)B.xi[j] * hy);
@@ -528,12 +533,14 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
     };
     auto store_flux_pair = [&](int h, const FluxF2& f) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            F2[h * PS + v * n2 + node] = f.F[v];
-            G2[h * PS + v * n2 + node] = f.G[v];
+        for (int v = 1; v < 4; ++v) {
+            F2[h * FS + (v - 1) * n2 + node] = f.F[v];
+            G2[h * FS + (v - 1) * n2 + node] = f.G[v];
         }
     };
-    auto divergence = [&](int h, int v) { return add2(xdot(F2 + h * PS + v * n2), ydot(G2 + h * PS + v * n2)); };
+    auto divergence = [&](int h, int v) {
+        return add2(xdot(F2 + h * FS + (v - 1) * n2), ydot(G2 + h * FS + (v - 1) * n2));
+    };
     auto store_q_pair = [&](int g, int v, float a, float b) {
         Q2[g * PS + v * n2 + node] = make_float2(a, 2 * g + 1 < n ? b : a);
     };
@@ -546,7 +553,7 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
         __syncthreads();
         float R0[4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) R0[v] = (v == 2 ? f.S2.x : 0.f) - divergence(0, v).x;
+        for (int v = 0; v < 4; ++v) R0[v] = (v == 2 ? f.S2.x : 0.f) - (v == 0 ? add2(gx[1], gy[2]) : divergence(0, v)).x;
 #pragma unroll
         for (int g = 0; g < NPAIR; ++g) {
             const int l1 = 2 * g + 1 < n ? 2 * g + 1 : 2 * g;
@@ -558,7 +565,7 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
     }
 #pragma unroll 1
     for (int r = 1; r < n; ++r) {
-        float2 S2h[NPAIR];
+        float2 S2h[NPAIR], M2h[NPAIR];
 #pragma unroll
         for (int h = 0; h < NPAIR; ++h) {
             float2 q[4], gx[4], gy[4];
@@ -566,13 +573,14 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
             eval_pair(h, q, gx, gy, f);
             store_flux_pair(h, f);
             S2h[h] = f.S2;
+            M2h[h] = add2(gx[1], gy[2]);
         }
         __syncthreads();
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             float2 R2[NPAIR];  // slices 2h, 2h+1 of variable v
 #pragma unroll
-            for (int h = 0; h < NPAIR; ++h) R2[h] = fma2(bc2(-1.f), divergence(h, v), v == 2 ? S2h[h] : bc2(0.f));
+            for (int h = 0; h < NPAIR; ++h) R2[h] = fma2(bc2(-1.f), v == 0 ? M2h[h] : divergence(h, v), v == 2 ? S2h[h] : bc2(0.f));
 #pragma unroll
             for (int g = 0; g < NPAIR; ++g) {
                 const int l0 = 2 * g, l1 = 2 * g + 1 < n ? 2 * g + 1 : 2 * g;
@@ -601,10 +609,17 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             qb[v] = fmaf(w1, q[v].y, fmaf(w0, q[v].x, qb[v]));
-            Fb[v] = fmaf(w1, f.F[v].y, fmaf(w0, f.F[v].x, Fb[v]));
-            Gb[v] = fmaf(w1, f.G[v].y, fmaf(w0, f.G[v].x, Gb[v]));
-            qxb[v] = fmaf(w1, gx[v].y, fmaf(w0, gx[v].x, qxb[v]));
-            qyb[v] = fmaf(w1, gy[v].y, fmaf(w0, gy[v].x, qyb[v]));  // full y-gradient (background included)
+            if (v > 0) {
+                Fb[v] = fmaf(w1, f.F[v].y, fmaf(w0, f.F[v].x, Fb[v]));
+                Gb[v] = fmaf(w1, f.G[v].y, fmaf(w0, f.G[v].x, Gb[v]));
+            }
+        }
+        if (wf) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                qxb[v] = fmaf(w1, gx[v].y, fmaf(w0, gx[v].x, qxb[v]));
+                qyb[v] = fmaf(w1, gy[v].y, fmaf(w0, gy[v].x, qyb[v]));  // full y-gradient (background included)
+            }
         }
         Sz = fmaf(w1, f.S2.y, fmaf(w0, f.S2.x, Sz));
     }
@@ -616,10 +631,12 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
         A[0 * SL + v * n2 + node] = qb[v];
-        A[1 * SL + v * n2 + node] = Fb[v];
-        A[2 * SL + v * n2 + node] = Gb[v];
-        A[3 * SL + v * n2 + node] = qxb[v];
-        A[4 * SL + v * n2 + node] = qyb[v];
+        A[1 * SL + v * n2 + node] = v == 0 ? qb[1] : Fb[v];
+        A[2 * SL + v * n2 + node] = v == 0 ? qb[2] : Gb[v];
+        if (wf) {
+            A[3 * SL + v * n2 + node] = qxb[v];
+            A[4 * SL + v * n2 + node] = qyb[v];
+        }
     }
     __syncthreads();
     if (active) {
@@ -640,9 +657,11 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
         const int f = idx / n, m = idx - f * n;
         const bool xface = f < 2;
         const float* phi = (f == 0 || f == 2) ? B.phi1 : B.phi0;
+        const bool wall = wf >> f & 1u;
         float rec[kTraceComps];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
+            if (c >= 2 && !wall) continue;
             const int slot = c == 0 ? 0 : c == 1 ? (xface ? 1 : 2) : (c == 2 ? 3 : 4);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
@@ -680,7 +699,8 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
         if (active) {
             double* tr = trace + ((size_t)cell * 4 + f) * kTraceComps * n;
 #pragma unroll
-            for (int c = 0; c < 16; ++c) tr[c * n + m] = f32_to_f64(rec[c]);
+            for (int c = 0; c < 16; ++c)
+                if (c < 8 || wall) tr[c * n + m] = f32_to_f64(rec[c]);
             tr[0 * n + m] = brho + f32_to_f64(rec[0]);
             tr[3 * n + m] = bE + f32_to_f64(rec[3]);
             tr[16 * n + m] = f32_to_f64(sp);
@@ -692,9 +712,9 @@ template <int N, int CPB>
 __global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
 k_predictor_amr_mixed(const double* __restrict__ u, double* __restrict__ rvol, double* __restrict__ trace, int cells,
                       float dt, const BasisF B, const PhysF P, const double* __restrict__ geo,
-                      const double* __restrict__ mb64, const float* __restrict__ mbf) {
+                      const int* __restrict__ nbr, const double* __restrict__ mb64, const float* __restrict__ mbf) {
     extern __shared__ float smf[];
-    predictor_amr_mixed_body<N, CPB>(u, rvol, trace, cells, blockIdx.x * CPB, dt, B, P, geo, mb64, mbf, smf);
+    predictor_amr_mixed_body<N, CPB>(u, rvol, trace, cells, blockIdx.x * CPB, dt, B, P, geo, nbr, mb64, mbf, smf);
 }
 
 // face data (q-bar and normal flux) of record `rec` of a coarse face evaluated
@@ -781,7 +801,8 @@ __device__ __forceinline__ void corrector_amr_body(double* __restrict__ u, const
         } else {
             double rec[kTraceComps];
 #pragma unroll
-            for (int c = 0; c < kTraceComps; ++c) rec[c] = own[c * n + m];
+            for (int c = 0; c < kTraceComps; ++c)
+                if (c < 8 || c == 16 || type == NB_WALL) rec[c] = own[c * n + m];
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 qo[v] = rec[v];
@@ -1070,8 +1091,8 @@ static int pred_n(adg_mesh* m, double dt, cudaStream_t s) {
         const size_t smem = (size_t)CM * AmrMixCfg<N>::stride * sizeof(float);
         ADG_CK(cudaFuncSetAttribute(km, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "amr pred mixed");
         km<<<(m->cells + CM - 1) / CM, CM * (N + 1) * (N + 1), smem, s>>>(m->u, m->rvol, m->trace, m->cells,
-                                                                          (float)dt, m->Bf, m->Pf, m->geo, m->mbl64,
-                                                                          m->mblf);
+                                                                          (float)dt, m->Bf, m->Pf, m->geo, m->nbr,
+                                                                          m->mbl64, m->mblf);
         ADG_CK(cudaGetLastError(), "amr mixed predictor launch");
         return ADG_OK;
     }
@@ -1299,8 +1320,8 @@ k_predictor_batch(const MixedInst* __restrict__ insts, const AmrInst* __restrict
         } else {
             const AmrInst& I = ainsts[-tl.inst - 1];
             const PhysF P = I.Pf;
-            predictor_amr_mixed_body<N, CPB>(I.u, I.rvol, I.trace, I.cells, tl.c0, I.dtf, B, P, I.geo, I.mb64,
-                                             I.mbf, smf);
+            predictor_amr_mixed_body<N, CPB>(I.u, I.rvol, I.trace, I.cells, tl.c0, I.dtf, B, P, I.geo, I.nbr,
+                                             I.mb64, I.mbf, smf);
         }
         __syncthreads();
     }
@@ -1327,7 +1348,7 @@ k_corrector_batch(const MixedInst* __restrict__ insts, const AmrInst* __restrict
 }
 
 // Node-pair predictor over the tiles of uniform instances (candidate 3 of a
-// batch without adaptive instances at N = 3, 5): the per-mesh node-pair body,
+// batch without adaptive instances at N = 3, 5, 7): the per-mesh node-pair body,
 // two nodes per thread, MixCfg2's cells per tile.
 template <int N, int CPB>
 __global__ void __launch_bounds__(CPB*(N + 1) * (N + 1) / 2, (MixCfg2<N, CPB>::minb))
@@ -1424,7 +1445,7 @@ static int batch_n(int cand, int phase, const MixedInst* insts, const AmrInst* a
         ADG_BATCH_CASE(1)
         ADG_BATCH_CASE(2)
         case 3:  // the node-pair predictor where it exists, else candidate 1
-            if constexpr (N == 3 || N == 5)
+            if constexpr (N == 3 || N == 5 || N == 7)
                 if (!amr && phase == 0) return batch_x2<N>(insts, tiles, ntiles, Bf, cpb_out, blocks_out, s);
             return amr ? batch_nka<N, 1, true>(phase, insts, ainsts, tiles, ntiles, Bf, B, O, cpb_out, blocks_out, s)
                        : batch_nka<N, 1, false>(phase, insts, ainsts, tiles, ntiles, Bf, B, O, cpb_out, blocks_out, s);

@@ -202,7 +202,8 @@ __device__ __forceinline__ void corrector_fp64_body(double* __restrict__ u, cons
         const double* own = trace + ((size_t)cell * 4 + f) * TR;
         double rec[kTraceComps];
 #pragma unroll
-        for (int c = 0; c < kTraceComps; ++c) rec[c] = own[c * n + m];
+        for (int c = 0; c < kTraceComps; ++c)
+            if (c < 8 || c == 16 || wall || noslip) rec[c] = own[c * n + m];
         double qo[4] = {rec[0], rec[1], rec[2], rec[3]};
         double fo[4] = {rec[4], rec[5], rec[6], rec[7]};
         const double so = rec[16];

@@ -72,7 +72,9 @@ constexpr int pred_cpb() {
 template <int N>
 static int launch_pred_mixed(const double* u, float* rvol, float* trace, int cells, float dt,
                              const BasisF& B, const PhysF& P, const MixedBg& bg, cudaStream_t s) {
-    if constexpr (N == 3 || N == 5) {  // node pairs (measured slower at N = 7: 232 registers, 8 warps per SM)
+    // node pairs where a row has an even number of nodes: 2124 against 2405 us
+    // per 243x243 launch at N = 7 (N = 1 has rows of one pair)
+    if constexpr (N == 3 || N == 5 || N == 7) {
         using C2 = MixCfg2<N>;
         auto kern = k_predictor_mixed_x2<N, C2::cpb>;
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C2::smem_pred);

@@ -27,7 +27,7 @@ struct MixCfg {
     // favours 8, which measured 2% slower, so 16 stays there and elsewhere
     static constexpr int np = n + (n & 1);
     static constexpr int npair = (n + 1) / 2;
-    static constexpr int raw = 3 * npair * 4 * n * n * 2;
+    static constexpr int raw = npair * 10 * n * n * 2;  // q' (4), F (3), G (3): the mass fluxes are momenta
     static constexpr int bank_off = cpb != cpb_default ? 16 : N == 2 ? 8 : N == 4 ? 18 : 16;
     static constexpr int stride = raw + ((bank_off - raw % 32) + 32) % 32;
     static constexpr size_t smem_pred = (size_t)cpb * stride * sizeof(float);
@@ -41,12 +41,22 @@ struct MixCfg {
     static constexpr int minb = (N == 5 && cpb == 4) ? 4 : (N == 4 && cpb == 5) ? 4 : (N == 3 && cpb == 8) ? 5 : (N == 2 && cpb == 16) ? 4 : (N == 6 && cpb == 2) ? 4 : (N == 7 && cpb == 2) ? 4 : (N == 6 && cpb == 3) ? 3 : (N == 6 && cpb == 5) ? 2 : 1;
 };
 
+// Slip-wall sides of cell (ix, iy) as a face mask (E, W, N, S).
+__device__ __forceinline__ unsigned wall_faces(int ix, int iy, const PhysF& P) {
+    unsigned m = 0;
+    if (P.bc_x == ADG_BC_WALL) m |= (ix == P.nx - 1 ? 1u : 0u) | (ix == 0 ? 2u : 0u);
+    if (P.bc_y == ADG_BC_WALL) m |= (iy == P.ny - 1 ? 4u : 0u) | (iy == 0 ? 8u : 0u);
+    return m;
+}
+
 // Predictor body for the tile of CPB cells starting at cell c0 (one thread per
 // spatial node); shared by the per-mesh kernel and the batched persistent one.
 //
 // Shared-memory layout per cell: the iterate q' and the fluxes F and G, each
 // row-major [h][v][j][i] of float2 holding time slices (2h, 2h+1) -- the
-// pairs the packed FP32x2 flux evaluation works on.  One 8-byte load then
+// pairs the packed FP32x2 flux evaluation works on (F and G without the mass
+// fluxes: F[0] = rho u and G[0] = rho v, whose derivatives the gradients of
+// the iterate already hold).  One 8-byte load then
 // serves both slices of a contraction term: x-contractions walk a row (the
 // lanes of one row read the same entry, a broadcast), y-contractions a column
 // (the lanes of one column likewise), with no transposed copies.  For odd n
@@ -68,7 +78,8 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
     constexpr int NPAIR = MixCfg<N, CPB>::npair, PS = 4 * n2;  // slice pairs, pair stride (float2)
     float2* Q2 = reinterpret_cast<float2*>(smf + (size_t)cl * MixCfg<N, CPB>::stride);  // [h][v][j][i]
     float2* F2 = Q2 + NPAIR * PS;                                                       // [h][v][j][i]
-    float2* G2 = F2 + NPAIR * PS;                                                       // [h][v][j][i]
+    constexpr int FS = 3 * n2;                                                          // pair stride of F, G
+    float2* G2 = F2 + NPAIR * FS;                                                       // [h][v - 1][j][i]
     const int ix = cell % P.nx, iy = cell / P.nx;
     const int row = iy * n + j;
     const float x = node_coord_f(P.x0, ix, B.xi[i], P.hx);
@@ -142,13 +153,15 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
     };
     auto store_flux_pair = [&](int h, const FluxF2& f) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            F2[h * PS + v * n2 + node] = f.F[v];
-            G2[h * PS + v * n2 + node] = f.G[v];
+        for (int v = 1; v < 4; ++v) {
+            F2[h * FS + (v - 1) * n2 + node] = f.F[v];
+            G2[h * FS + (v - 1) * n2 + node] = f.G[v];
         }
     };
-    // dF/dx + dG/dy of slice pair h at this node
-    auto divergence = [&](int h, int v) { return add2(xdot(F2 + h * PS + v * n2), ydot(G2 + h * PS + v * n2)); };
+    // dF/dx + dG/dy of slice pair h at this node, v >= 1 (v = 0: gx[1] + gy[2], the same sums)
+    auto divergence = [&](int h, int v) {
+        return add2(xdot(F2 + h * FS + (v - 1) * n2), ydot(G2 + h * FS + (v - 1) * n2));
+    };
     // slices 2g, 2g+1 of variable v (for odd n the slot past the last slice
     // repeats it)
     auto store_q_pair = [&](int g, int v, float a, float b) {
@@ -163,7 +176,8 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
         __syncthreads();
         float R0[4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) R0[v] = (v == 2 ? f.S2.x : 0.f) + Sm[v] - divergence(0, v).x;
+        for (int v = 0; v < 4; ++v)
+            R0[v] = (v == 2 ? f.S2.x : 0.f) + Sm[v] - (v == 0 ? add2(gx[1], gy[2]) : divergence(0, v)).x;
 #pragma unroll
         for (int g = 0; g < NPAIR; ++g) {
             const int l1 = 2 * g + 1 < n ? 2 * g + 1 : 2 * g;
@@ -174,11 +188,11 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
         __syncthreads();
     }
     // sweeps 2..n on the slice pairs; the residual is contracted in time one
-    // variable at a time, so only the z-momentum source of each pair stays
-    // live across the barrier
+    // variable at a time, so only two scalars of each pair stay live across the
+    // barrier
 #pragma unroll 1
     for (int r = 1; r < n; ++r) {
-        float2 S2h[NPAIR];
+        float2 S2h[NPAIR], M2h[NPAIR];  // of each pair: the z-momentum source, the divergence of the mass flux
 #pragma unroll
         for (int h = 0; h < NPAIR; ++h) {
             float2 q[4], gx[4], gy[4];
@@ -186,6 +200,7 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
             eval_pair(h, q, gx, gy, f);
             store_flux_pair(h, f);
             S2h[h] = f.S2;
+            M2h[h] = add2(gx[1], gy[2]);
         }
         __syncthreads();
 #pragma unroll
@@ -195,7 +210,7 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
             for (int h = 0; h < NPAIR; ++h) {
                 R2[h] = bc2(Sm[v]);
                 if (v == 2) R2[h] = add2(R2[h], S2h[h]);
-                R2[h] = fma2(bc2(-1.f), divergence(h, v), R2[h]);
+                R2[h] = fma2(bc2(-1.f), v == 0 ? M2h[h] : divergence(h, v), R2[h]);
             }
 #pragma unroll
             for (int g = 0; g < NPAIR; ++g) {
@@ -216,6 +231,7 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
     // final evaluation on the converged iterate and the time averages
     // (scalar accumulators: half the registers of packed ones, at the
     // register peak of the kernel)
+    const unsigned wf = wall_faces(ix, iy, P);  // grad q-bar is read on walls only
     float qb[4], Fb[4], Gb[4], Sb[4], qxb[4], qyb[4], Sz = 0.f;
 #pragma unroll
     for (int v = 0; v < 4; ++v) qb[v] = Fb[v] = Gb[v] = qxb[v] = qyb[v] = 0.f;
@@ -228,10 +244,17 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             qb[v] = fmaf(w1, q[v].y, fmaf(w0, q[v].x, qb[v]));
-            Fb[v] = fmaf(w1, f.F[v].y, fmaf(w0, f.F[v].x, Fb[v]));
-            Gb[v] = fmaf(w1, f.G[v].y, fmaf(w0, f.G[v].x, Gb[v]));
-            qxb[v] = fmaf(w1, gx[v].y, fmaf(w0, gx[v].x, qxb[v]));
-            qyb[v] = fmaf(w1, gy[v].y, fmaf(w0, gy[v].x, qyb[v]));  // full y-gradient (background included)
+            if (v > 0) {
+                Fb[v] = fmaf(w1, f.F[v].y, fmaf(w0, f.F[v].x, Fb[v]));
+                Gb[v] = fmaf(w1, f.G[v].y, fmaf(w0, f.G[v].x, Gb[v]));
+            }
+        }
+        if (wf) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                qxb[v] = fmaf(w1, gx[v].y, fmaf(w0, gx[v].x, qxb[v]));
+                qyb[v] = fmaf(w1, gy[v].y, fmaf(w0, gy[v].x, qyb[v]));  // full y-gradient (background included)
+            }
         }
         Sz = fmaf(w1, f.S2.y, fmaf(w0, f.S2.x, Sz));
     }
@@ -245,10 +268,12 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
         A[0 * SLP + v * RS + rm] = qb[v];
-        A[1 * SLP + v * RS + rm] = Fb[v];
-        A[2 * SLP + v * RS + rm] = Gb[v];
-        A[3 * SLP + v * RS + rm] = qxb[v];
-        A[4 * SLP + v * RS + rm] = qyb[v];
+        A[1 * SLP + v * RS + rm] = v == 0 ? qb[1] : Fb[v];
+        A[2 * SLP + v * RS + rm] = v == 0 ? qb[2] : Gb[v];
+        if (wf) {
+            A[3 * SLP + v * RS + rm] = qxb[v];
+            A[4 * SLP + v * RS + rm] = qyb[v];
+        }
     }
     __syncthreads();
     if (active) {
@@ -268,9 +293,11 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
         const int f = idx / n, m = idx - f * n;
         const bool xface = f < 2;
         const float* phi = (f == 0 || f == 2) ? B.phi1 : B.phi0;
+        const bool wall = wf >> f & 1u;  // the gradients go to wall faces alone
         float rec[kTraceComps];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
+            if (c >= 2 && !wall) continue;
             const int slot = c == 0 ? 0 : c == 1 ? (xface ? 1 : 2) : (c == 2 ? 3 : 4);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
@@ -299,7 +326,8 @@ __device__ __forceinline__ void predictor_mixed_body(const double* __restrict__ 
         if (active) {
             float* tr = trace + ((size_t)cell * 4 + f) * kTraceComps * n;
 #pragma unroll
-            for (int c = 0; c < kTraceComps; ++c) tr[c * n + m] = rec[c];
+            for (int c = 0; c < kTraceComps; ++c)
+                if (c < 8 || c == 16 || wall) tr[c * n + m] = rec[c];
         }
     }
 }
@@ -395,12 +423,12 @@ __device__ __forceinline__ void corrector_mixed_body(double* __restrict__ u, con
     for (int idx = node; idx < 4 * n; idx += n2) {
         const int f = idx / n, m = idx - f * n;
         const bool xface = f < 2;
-        const bool wall = xface ? (P.bc_x == ADG_BC_WALL && ((f == 0 && ix == P.nx - 1) || (f == 1 && ix == 0)))
-                                : (P.bc_y == ADG_BC_WALL && ((f == 2 && iy == P.ny - 1) || (f == 3 && iy == 0)));
+        const bool wall = wall_faces(ix, iy, P) >> f & 1u;
         const float* own = trace + ((size_t)cell * 4 + f) * TR;
         float rec[kTraceComps];
 #pragma unroll
-        for (int c = 0; c < kTraceComps; ++c) rec[c] = own[c * n + m];
+        for (int c = 0; c < kTraceComps; ++c)
+            if (c < 8 || c == 16 || wall) rec[c] = own[c * n + m];
         float qo[4] = {rec[0], rec[1], rec[2], rec[3]};
         float fo[4] = {rec[4], rec[5], rec[6], rec[7]};
         const float so = rec[16];

@@ -7,6 +7,7 @@
 
 #include "adg_convert.cuh"
 #include "adg_internal.h"
+#include "adg_mixed_body.cuh"
 #include "adg_mixed_point.cuh"
 
 namespace adg {
@@ -32,18 +33,22 @@ struct MixCfg2 {
     // measured at N = 5: 7 cells per block (126 threads, three resident blocks) took 101.7 us on the
     // 81x81 warm bubble against 105.2 (6 cells), 102.5 (5), and 0.791 against 0.834 ms per step on
     // the 243x243 sweep mesh; 4, 8, 10 cells were slower still (0.132, 0.123, 0.113 ms)
-    static constexpr int cpb_default = N == 3 ? 16 : N == 5 ? 7 : 4;
+    // N = 7 (255 registers, four blocks): 2124 us per 243x243 launch with 2 cells, 2152 with 4, 2244 with 1
+    static constexpr int cpb_default = N == 3 ? 16 : N == 5 ? 7 : N == 7 ? 2 : 4;
     static constexpr int cpb = CPB_ ? CPB_ : cpb_default;
     static constexpr int threads = cpb * tpc;
     static constexpr int npair = n / 2;
-    static constexpr int raw = 3 * npair * 4 * n * n * 2;             // q', F, G as float2 pairs
+    // row stride in float2: rows of 8 would put the 16-byte row loads of four
+    // rows on the same banks (4446 against 2152 us per 243x243 launch at N = 7)
+    static constexpr int rq = n == 8 ? 10 : n;
+    static constexpr int raw = npair * 10 * n * rq * 2;               // q' (4), F (3), G (3) as float2 pairs
     static constexpr int bank_off = 16;                                // floats, mod 32, between cells
     static constexpr int stride = raw + ((bank_off - raw % 32) + 32) % 32;  // a multiple of 4 floats
     static constexpr size_t smem_pred = (size_t)cpb * stride * sizeof(float);
-    // three resident blocks asked of the register allocator: at N = 3 taking the pair's
-    // own iterate from its row loads otherwise grows the kernel to 218 registers (two
-    // blocks, 0.175 ms per 243x243 step); capped it keeps 167 (0.157 ms)
-    static constexpr int minb = (N == 5 || N == 3) ? 3 : 1;
+    // resident blocks asked of the register allocator: four at N = 3 (128
+    // registers, 111.3 us per 243x243 launch; three 113.1), three at N = 5
+    // (642 us; four spill, 645), four at N = 7
+    static constexpr int minb = N == 5 ? 3 : N == 3 || N == 7 ? 4 : 1;
 };
 
 template <int N, int CPB>
@@ -54,7 +59,7 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
     using C = MixCfg2<N, CPB>;
     constexpr int n = N + 1, n2 = n * n, SL = 4 * n2, TPC = C::tpc;
     constexpr int NP = n, RS = n * NP, SLP = 4 * RS;  // time-average rows (even n: no padding)
-    constexpr int NPAIR = C::npair, PS = 4 * n2;      // slice pairs, pair stride (float2)
+    constexpr int NPAIR = C::npair, RQ = C::rq, PL = n * RQ, PS = 4 * PL;  // slice pairs, row, plane and pair strides (float2)
     const int cl = threadIdx.x / TPC;
     const int loc = threadIdx.x - cl * TPC;
     // column-pair-major: the lanes of one column pair are adjacent, so a
@@ -63,12 +68,14 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
     // runs of 8-byte or 8 of 16-byte accesses in one)
     const int ip = loc / n, j = loc - ip * n, i0 = 2 * ip;
     const int nd0 = j * n + i0;  // first node of the pair; the second is nd0 + 1
+    const int ns0 = j * RQ + i0;  // its place in a plane of the slice-pair arrays
     const int cell_raw = c0 + cl;
     const bool active = cell_raw < cells;
     const int cell = active ? cell_raw : cells - 1;
     float2* Q2 = reinterpret_cast<float2*>(smf + (size_t)cl * C::stride);  // [h][v][j][i]
     float2* F2 = Q2 + NPAIR * PS;
-    float2* G2 = F2 + NPAIR * PS;
+    constexpr int FS = 3 * PL;            // F and G hold v = 1..3: the mass fluxes are momenta
+    float2* G2 = F2 + NPAIR * FS;
     // float4 = the float2 pairs of nodes (a, b) and (a, b+1), b even
     auto ld4 = [](const float2* S, int idx) { return *reinterpret_cast<const float4*>(S + idx); };
     auto st4 = [](float2* S, int idx, float2 a, float2 b) {
@@ -90,7 +97,7 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
         up[a][3] = f64_to_f32(uc[3 * n2 + nd0 + a] - Eb64);
     }
 #pragma unroll
-    for (int v = 0; v < 4; ++v) st4(Q2, v * n2 + nd0, bc2(up[0][v]), bc2(up[1][v]));
+    for (int v = 0; v < 4; ++v) st4(Q2, v * PL + ns0, bc2(up[0][v]), bc2(up[1][v]));
     float Sm[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
     if (P.source == ADG_SRC_STEADY) {
 #pragma unroll
@@ -108,7 +115,7 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
     }
     // x-contractions of row j for both nodes: one 16-byte load per two terms
     auto xdot2 = [&](const float2* S, float2& s0, float2& s1) {
-        const float2* r = S + j * n;
+        const float2* r = S + j * RQ;
         float4 a = ld4(r, 0);
         s0 = fma2(bc2(dI0[1]), make_float2(a.z, a.w), mul2(bc2(dI0[0]), make_float2(a.x, a.y)));
         s1 = fma2(bc2(dI1[1]), make_float2(a.z, a.w), mul2(bc2(dI1[0]), make_float2(a.x, a.y)));
@@ -122,7 +129,7 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
     // the same, also returning the pair's own values, which the row loads
     // include (the load at p = i0), so the iterate needs no load of its own
     auto xdot2_own = [&](const float2* S, float2& s0, float2& s1, float2& q0, float2& q1) {
-        const float2* r = S + j * n;
+        const float2* r = S + j * RQ;
         float4 a = ld4(r, 0);
         float4 own = a;
         s0 = fma2(bc2(dI0[1]), make_float2(a.z, a.w), mul2(bc2(dI0[0]), make_float2(a.x, a.y)));
@@ -144,17 +151,17 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
         s1 = mul2(bc2(dJ[0]), make_float2(a.z, a.w));
 #pragma unroll
         for (int p = 1; p < n; ++p) {
-            a = ld4(S, p * n + i0);
+            a = ld4(S, p * RQ + i0);
             s0 = fma2(bc2(dJ[p]), make_float2(a.x, a.y), s0);
             s1 = fma2(bc2(dJ[p]), make_float2(a.z, a.w), s1);
         }
     };
-    // both slices of pair h at both nodes; fluxes of node a in f[a]
-    auto eval_pair = [&](int h, FluxF2 f[2]) {
+    // both slices of pair h at both nodes; fluxes of node a in f[a], divergence of its mass flux in md[a]
+    auto eval_pair = [&](int h, FluxF2 f[2], float2 md[2]) {
         float2 q[2][4], gx[2][4], gy[2][4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const float2* S = Q2 + h * PS + v * n2;
+            const float2* S = Q2 + h * PS + v * PL;
             xdot2_own(S, gx[0][v], gx[1][v], q[0][v], q[1][v]);
             ydot2(S, gy[0][v], gy[1][v]);
         }
@@ -163,34 +170,36 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
             gy[a][0] = add2(gy[a][0], bc2(dzr));
             gy[a][3] = add2(gy[a][3], bc2(dzE));
             ns_flux_pert2(q[a], gx[a], gy[a], z, rb, Eb, pb, P, f[a]);
+            md[a] = add2(gx[a][1], gy[a][2]);
         }
     };
     auto store_flux_pair = [&](int h, const FluxF2 f[2]) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            st4(F2, h * PS + v * n2 + nd0, f[0].F[v], f[1].F[v]);
-            st4(G2, h * PS + v * n2 + nd0, f[0].G[v], f[1].G[v]);
+        for (int v = 1; v < 4; ++v) {
+            st4(F2, h * FS + (v - 1) * PL + ns0, f[0].F[v], f[1].F[v]);
+            st4(G2, h * FS + (v - 1) * PL + ns0, f[0].G[v], f[1].G[v]);
         }
     };
-    // dF/dx + dG/dy of slice pair h at both nodes
+    // dF/dx + dG/dy of slice pair h at both nodes, v >= 1
     auto divergence2 = [&](int h, int v, float2& d0, float2& d1) {
         float2 x0, x1, y0, y1;
-        xdot2(F2 + h * PS + v * n2, x0, x1);
-        ydot2(G2 + h * PS + v * n2, y0, y1);
+        xdot2(F2 + h * FS + (v - 1) * PL, x0, x1);
+        ydot2(G2 + h * FS + (v - 1) * PL, y0, y1);
         d0 = add2(x0, y0);
         d1 = add2(x1, y1);
     };
 
     {  // sweep 1: iterate constant in time (both slices of pair 0 hold it)
         FluxF2 f[2];
-        eval_pair(0, f);
+        float2 md[2];
+        eval_pair(0, f, md);
         store_flux_pair(0, f);
         __syncthreads();
         float R0[2][4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            float2 d0, d1;
-            divergence2(0, v, d0, d1);
+            float2 d0 = md[0], d1 = md[1];
+            if (v > 0) divergence2(0, v, d0, d1);
             R0[0][v] = (v == 2 ? f[0].S2.x : 0.f) + Sm[0][v] - d0.x;
             R0[1][v] = (v == 2 ? f[1].S2.x : 0.f) + Sm[1][v] - d1.x;
         }
@@ -203,7 +212,7 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
                 for (int b = 0; b < 2; ++b)
                     a[b] = make_float2(fmaf(dt, B.Kw1[2 * g] * R0[b][v], up[b][v]),
                                        fmaf(dt, B.Kw1[2 * g + 1] * R0[b][v], up[b][v]));
-                st4(Q2, g * PS + v * n2 + nd0, a[0], a[1]);
+                st4(Q2, g * PS + v * PL + ns0, a[0], a[1]);
             }
         }
         __syncthreads();
@@ -211,12 +220,15 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
     // sweeps 2..n on the slice pairs, the residual contracted in time one variable at a time
 #pragma unroll 1
     for (int r = 1; r < n; ++r) {
-        float2 S2h[2][NPAIR];
+        float2 S2h[2][NPAIR], M2h[2][NPAIR];
 #pragma unroll
         for (int h = 0; h < NPAIR; ++h) {
             FluxF2 f[2];
-            eval_pair(h, f);
+            float2 md[2];
+            eval_pair(h, f, md);
             store_flux_pair(h, f);
+            M2h[0][h] = md[0];
+            M2h[1][h] = md[1];
             S2h[0][h] = f[0].S2;
             S2h[1][h] = f[1].S2;
         }
@@ -226,8 +238,8 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
             float2 R2[2][NPAIR];
 #pragma unroll
             for (int h = 0; h < NPAIR; ++h) {
-                float2 d[2];
-                divergence2(h, v, d[0], d[1]);
+                float2 d[2] = {M2h[0][h], M2h[1][h]};
+                if (v > 0) divergence2(h, v, d[0], d[1]);
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
                     R2[b][h] = bc2(Sm[b][v]);
@@ -250,13 +262,14 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
                     }
                     o[b] = make_float2(fmaf(dt, a0.x + a0.y, up[b][v]), fmaf(dt, a1.x + a1.y, up[b][v]));
                 }
-                st4(Q2, g * PS + v * n2 + nd0, o[0], o[1]);
+                st4(Q2, g * PS + v * PL + ns0, o[0], o[1]);
             }
         }
         __syncthreads();
     }
 
     // final evaluation on the converged iterate and the time averages
+    const unsigned wf = wall_faces(ix, iy, P);  // grad q-bar is read on walls only
     float qb[2][4], Fb[2][4], Gb[2][4], qxb[2][4], qyb[2][4], Sz[2] = {0.f, 0.f};
 #pragma unroll
     for (int b = 0; b < 2; ++b)
@@ -267,7 +280,7 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
         float2 q[2][4], gx[2][4], gy[2][4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            const float2* S = Q2 + h * PS + v * n2;
+            const float2* S = Q2 + h * PS + v * PL;
             xdot2_own(S, gx[0][v], gx[1][v], q[0][v], q[1][v]);
             ydot2(S, gy[0][v], gy[1][v]);
         }
@@ -281,10 +294,17 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 qb[b][v] = fmaf(w1, q[b][v].y, fmaf(w0, q[b][v].x, qb[b][v]));
-                Fb[b][v] = fmaf(w1, f.F[v].y, fmaf(w0, f.F[v].x, Fb[b][v]));
-                Gb[b][v] = fmaf(w1, f.G[v].y, fmaf(w0, f.G[v].x, Gb[b][v]));
-                qxb[b][v] = fmaf(w1, gx[b][v].y, fmaf(w0, gx[b][v].x, qxb[b][v]));
-                qyb[b][v] = fmaf(w1, gy[b][v].y, fmaf(w0, gy[b][v].x, qyb[b][v]));
+                if (v > 0) {
+                    Fb[b][v] = fmaf(w1, f.F[v].y, fmaf(w0, f.F[v].x, Fb[b][v]));
+                    Gb[b][v] = fmaf(w1, f.G[v].y, fmaf(w0, f.G[v].x, Gb[b][v]));
+                }
+            }
+            if (wf) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    qxb[b][v] = fmaf(w1, gx[b][v].y, fmaf(w0, gx[b][v].x, qxb[b][v]));
+                    qyb[b][v] = fmaf(w1, gy[b][v].y, fmaf(w0, gy[b][v].x, qyb[b][v]));
+                }
             }
             Sz[b] = fmaf(w1, f.S2.y, fmaf(w0, f.S2.x, Sz[b]));
         }
@@ -297,10 +317,12 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
 #pragma unroll
     for (int v = 0; v < 4; ++v) {
         st2(A + 0 * SLP + v * RS + rm, qb[0][v], qb[1][v]);
-        st2(A + 1 * SLP + v * RS + rm, Fb[0][v], Fb[1][v]);
-        st2(A + 2 * SLP + v * RS + rm, Gb[0][v], Gb[1][v]);
-        st2(A + 3 * SLP + v * RS + rm, qxb[0][v], qxb[1][v]);
-        st2(A + 4 * SLP + v * RS + rm, qyb[0][v], qyb[1][v]);
+        st2(A + 1 * SLP + v * RS + rm, v == 0 ? qb[0][1] : Fb[0][v], v == 0 ? qb[1][1] : Fb[1][v]);
+        st2(A + 2 * SLP + v * RS + rm, v == 0 ? qb[0][2] : Gb[0][v], v == 0 ? qb[1][2] : Gb[1][v]);
+        if (wf) {
+            st2(A + 3 * SLP + v * RS + rm, qxb[0][v], qxb[1][v]);
+            st2(A + 4 * SLP + v * RS + rm, qyb[0][v], qyb[1][v]);
+        }
     }
     __syncthreads();
     if (active) {
@@ -327,9 +349,11 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
         const int f = idx / n, m = idx - f * n;
         const bool xface = f < 2;
         const float* phi = (f == 0 || f == 2) ? B.phi1 : B.phi0;
+        const bool wall = wf >> f & 1u;  // the gradients go to wall faces alone
         float rec[kTraceComps];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
+            if (c >= 2 && !wall) continue;
             const int slot = c == 0 ? 0 : c == 1 ? (xface ? 1 : 2) : (c == 2 ? 3 : 4);
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
@@ -357,7 +381,8 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
         if (active) {
             float* tr = trace + ((size_t)cell * 4 + f) * kTraceComps * n;
 #pragma unroll
-            for (int c = 0; c < kTraceComps; ++c) tr[c * n + m] = rec[c];
+            for (int c = 0; c < kTraceComps; ++c)
+                if (c < 8 || c == 16 || wall) tr[c * n + m] = rec[c];
         }
     }
 }
