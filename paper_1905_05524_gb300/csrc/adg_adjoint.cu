@@ -14,26 +14,35 @@
 //      into shared memory, then run the predictor backwards: face
 //      extrapolation and wave speed, weak volume residual, time averages and
 //      final evaluation, and the n sweeps, each through the hand-written
-//      reverse of the point-wise flux (ns_flux_adj).
+//      reverse of the point-wise flux (ns_flux5_adj).  One thread per
+//      space-time node, contractions on the integer pipe, as the forward
+//      predictor (adg_fp64_body.cuh, adg_fixed.cuh).
 //
 // Non-smooth points take one-sided derivatives: max(s_L, s_R) differentiates
 // into s_L on ties, |v.n| into sign(v.n) (0 at 0).
 #include <cuda_runtime.h>
 
+#include "adg_fp64_body.cuh"
 #include "adg_internal.h"
 #include "adg_physics.cuh"
 
 namespace adg {
 
+// Predictor adjoint: the thread layout of the forward predictor (FxCfg: one
+// thread per space-time node), its contractions on the integer pipe.
 template <int N>
 struct AdjCfg {
-    static constexpr int n = N + 1;
-    static constexpr int cpb = N <= 2 ? 4 : N <= 4 ? 2 : 1;
-    static constexpr int threads = cpb * n * n;
-    static constexpr int SL = 4 * n * n;
-    // iterates q^(1..n) (n slices each) + q^(0) (one slice) + QB, RB, QXB, QYB
-    static constexpr int per_cell = (n * n + 1) * SL + 4 * n * SL;
-    static constexpr size_t smem = (size_t)cpb * per_cell * sizeof(double);
+    using F = FxCfg<N>;
+    static constexpr int n = F::n, n2 = F::n2, n3 = F::n3;
+    static constexpr int cpb = F::cpb, tpc = F::tpc, threads = F::threads;
+    static constexpr int resident = N == 5 ? 2 : 4;  // blocks per SM asked of the register allocator
+    // per cell, in 8-byte words: the limbs of the iterates q^(0) (one time
+    // slice) and q^(1..n); a work area (fluxes and residual forward; adjoints
+    // of q, of the residual and of the gradients backward); u; D/h and -dt D/h;
+    // the adjoints of the face records; iterate exponents and group magnitudes
+    static constexpr int work = 8 * n3 > 20 * n2 ? 8 * n3 : 20 * n2;
+    static constexpr int words = 4 * n2 + 4 * n * n3 + work + 4 * n2 + 4 * n2 + 64 * n + 2 * (n + 1) + 4;
+    static constexpr size_t smem = ((size_t)cpb * words + n2 + n) * 8;
 };
 
 // ------------------------------------------------------------------ corrector
@@ -175,373 +184,458 @@ k_corrector_adj_fp64(const double* __restrict__ lam, const double* __restrict__ 
 }
 
 // ------------------------------------------------------------------ predictor
-template <int N, int CPB>
-__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
+// Adjoint of ns_flux5: given the adjoints of the fluxes (Fb, Gb; F[2] and G[1]
+// are one value) and of the z-momentum source (Sb2), adds the adjoints of the
+// state and its gradients.  Written line by line against ns_flux5.
+__device__ __forceinline__ void ns_flux5_adj(const double q[4], const double gx[4], const double gy[4], double g, double gz,
+                                             double gm1, double mu, double mu23, double kR, const double Fb[4],
+                                             const double Gb[4], double Sb2, double qb[4], double gxb[4], double gyb[4]) {
+    const double rho = q[0], mx = q[1], my = q[2], E = q[3];
+    const double r = fx_rcp(rho);
+    const double u = mx * r, v = my * r;
+    const double p = gm1 * fma(-0.5, fma(my, v, mx * u), fma(-gz, rho, E));
+    const double Ep = E + p, eR = E * r;
+    const double ux = fma(-u, gx[0], gx[1]), uy = fma(-u, gy[0], gy[1]);
+    const double vx = fma(-v, gx[0], gx[2]), vy = fma(-v, gy[0], gy[2]);
+    const double hx = fma(-v, vx, fma(-u, ux, fma(-eR, gx[0], gx[3])));
+    const double hy = fma(-g, rho, fma(-v, vy, fma(-u, uy, fma(-eR, gy[0], gy[3]))));
+    const double m23 = mu23 * r, kr = kR * r, A = -mu * r;
+    const double X = fma(-2.0, ux, vy), Y = fma(-2.0, vy, ux), Z = uy + vx;
+    const double sxx = m23 * X, syy = m23 * Y, sxy = A * Z;
+    // fluxes
+    const double a1 = Fb[1], a3 = Fb[3], b2 = Gb[2], b3 = Gb[3], xb = Fb[2] + Gb[1];
+    const double sxxb = fma(a3, u, a1), syyb = fma(b3, v, b2), sxyb = fma(b3, u, fma(a3, v, xb));
+    const double Epb = fma(b3, v, a3 * u), pb = gm1 * (Epb + (a1 + b2));
+    const double ke = -0.5 * pb;
+    double mxb = fma(u, ke, fma(a1, u, Fb[0])), myb = fma(v, ke, fma(b2, v, fma(xb, u, Gb[0])));
+    double ub = fma(mx, ke, fma(b3, sxy, fma(a3, Ep + sxx, fma(xb, my, a1 * mx))));
+    double vb = fma(my, ke, fma(a3, sxy, fma(b3, Ep + syy, b2 * my)));
+    // heat flux, stresses
+    const double hxb = -kr * a3, hyb = -kr * b3;
+    const double t1 = m23 * sxxb, t2 = m23 * syyb, t3 = A * sxyb;
+    const double uxb = fma(-u, hxb, fma(-2.0, t1, t2)), vyb = fma(-v, hyb, fma(-2.0, t2, t1));
+    const double uyb = fma(-u, hyb, t3), vxb = fma(-v, hxb, t3);
+    ub -= fma(gy[0], uyb, fma(gx[0], uxb, fma(uy, hyb, ux * hxb)));
+    vb -= fma(gy[0], vyb, fma(gx[0], vxb, fma(vy, hyb, vx * hxb)));
+    const double eRb = -fma(gy[0], hyb, gx[0] * hxb);
+    double rb = fma(mu23, fma(syyb, Y, sxxb * X), -mu * (sxyb * Z));
+    rb = fma(-kR, fma(hy, b3, hx * a3), rb);
+    rb = fma(my, vb, fma(mx, ub, fma(E, eRb, rb)));
+    qb[0] += fma(-r, r * rb, fma(-gz, pb, -g * (hyb + Sb2)));
+    qb[1] += fma(r, ub, mxb);
+    qb[2] += fma(r, vb, myb);
+    qb[3] += fma(r, eRb, Epb + pb);
+    gxb[0] -= fma(v, vxb, fma(u, uxb, eR * hxb));
+    gyb[0] -= fma(v, vyb, fma(u, uyb, eR * hyb));
+    gxb[1] += uxb;
+    gyb[1] += uyb;
+    gxb[2] += vxb;
+    gyb[2] += vyb;
+    gxb[3] += hxb;
+    gyb[3] += hyb;
+}
+
+// One cell per group of tpc threads (all groups of the block in step).  The
+// iterates of the forward sweeps stay in shared memory as limbs, from which
+// the reverse sweeps form the gradients and the node's own state again.
+template <int N>
+__global__ void __launch_bounds__(AdjCfg<N>::threads, AdjCfg<N>::resident)
 k_predictor_adj_fp64(const double* __restrict__ u, const double* __restrict__ lam,
                      const double* __restrict__ trace, const double* __restrict__ trace_bar,
                      double* __restrict__ lam_out, int cells, double dt, const Basis B, const Phys P,
                      const Background bg) {
-    constexpr int n = N + 1, n2 = n * n, SL = 4 * n2, TR = kTraceComps * n;
+    using C = AdjCfg<N>;
+    constexpr int n = C::n, n2 = C::n2, n3 = C::n3, SL = 4 * n2, TR = kTraceComps * n;
     extern __shared__ double sm[];
-    const int cl = threadIdx.x / n2;
-    const int node = threadIdx.x - cl * n2;
-    const int j = node / n, i = node - j * n;
-    const int cell_raw = blockIdx.x * CPB + cl;
+    const int cl = threadIdx.x / C::tpc, tid = threadIdx.x - cl * C::tpc;
+    const bool on = tid < n3;
+    const int id = on ? tid : n3 - 1;
+    const int k = id / n2, node = id - k * n2, j = node / n, i = node - j * n;
+    double* base = sm + (size_t)cl * C::words;
+    Limbs* U0 = reinterpret_cast<Limbs*>(base);  // q^(0) [4][n2]
+    Limbs* IT = U0 + 4 * n2;                     // q^(r) at IT + (r - 1) 4 n3, [4][n][n2]
+    double* Wd = base + 4 * n2 + 4 * n * n3;
+    Limbs* W = reinterpret_cast<Limbs*>(Wd);
+    double* US = Wd + C::work;                            // u [4][n2]
+    Limbs* DT = reinterpret_cast<Limbs*>(US + 4 * n2);    // D/hx, D/hy [n][n]
+    Limbs* DM = DT + 2 * n2;                              // -dt D/hx, -dt D/hy
+    double* FR = US + 8 * n2;                             // adjoints of the face records [4][16][n]
+    int* EX = reinterpret_cast<int*>(FR + 64 * n);        // exponents of the iterates [n + 1][3 (+1)]
+    uint32_t* mx = reinterpret_cast<uint32_t*>(EX + 4 * (n + 1));
+    Limbs* K = reinterpret_cast<Limbs*>(sm + (size_t)C::cpb * C::words);  // [n][n], then the row sums [n]
+    fx_time_table<N>(K, B);
+    for (int a = threadIdx.x; a < n; a += blockDim.x) K[n2 + a] = fx_split_centred(fx_from(B.Kw1[a], B.KwE + 3));
+    const double hmax = B.Dmax * fmax(P.inv_hx, P.inv_hy);
+    const int ed = fx_exp(fx_mag(hmax)), em = fx_exp(fx_mag(hmax * dt));
+    const int sh = (int)(fx_mag(B.Drow * (P.inv_hx + P.inv_hy)) >> 20) - ed + 1;
+    for (int a = tid; a < n2; a += C::tpc) {
+        const double dx = B.D[a / n][a % n] * P.inv_hx, dy = B.D[a / n][a % n] * P.inv_hy;
+        DT[a] = fx_split_centred(fx_from(dx, ed));
+        DT[n2 + a] = fx_split_centred(fx_from(dy, ed));
+        DM[a] = fx_split_centred(fx_from(-dt * dx, em));
+        DM[n2 + a] = fx_split_centred(fx_from(-dt * dy, em));
+    }
+    const int cell_raw = blockIdx.x * C::cpb + cl;
     const bool active = cell_raw < cells;
     const int cell = active ? cell_raw : cells - 1;
-    double* IT = sm + (size_t)cl * AdjCfg<N>::per_cell;  // q^(r) at IT + ((r-1) n + k) SL, r = 1..n
-    double* U0 = IT + n * n * SL;                        // q^(0) = u (one slice)
-    double* QB = U0 + SL;
-    double* RB = QB + n * SL;
-    double* QXB = RB + n * SL;
-    double* QYB = QXB + n * SL;
     const int ix = cell % P.nx, iy = cell / P.nx;
-    const double x = P.x0 + (ix + B.xi[i]) * P.hx;
-    const double z = P.y0 + (iy + B.xi[j]) * P.hy;
-    const double pbar = bg.pbar_node[iy * n + j];
-    const double rhobar = bg.rhobar_node[iy * n + j];
+    const double x = P.x0 + (ix + B.xi[i]) * P.hx, z = P.y0 + (iy + B.xi[j]) * P.hy;
+    const double pbar = bg.pbar_node[iy * n + j], rhobar = bg.rhobar_node[iy * n + j];
+    const double g = P.gravity ? P.g : 0.0, gz = g * z;
+    const double mu23 = (2.0 / 3.0) * P.mu, kR = P.gm1 * P.kappa * P.invR;
+    const bool has_src = P.source == ADG_SRC_STEADY;
     double Sm[4] = {0.0, 0.0, 0.0, 0.0};
-    if (P.source == ADG_SRC_STEADY) steady_source(x, z, P, Sm);
-    auto iter = [&](int r, int k) -> double* { return r == 0 ? U0 : IT + ((r - 1) * n + k) * SL; };
+    if (has_src) steady_source(x, z, P, Sm);
 
-    double uu[4];
-    const double* uc = u + (size_t)cell * SL;
+    auto push = [&](int slot, uint32_t m) {
+        if constexpr (C::tpc >= 32) {
+            m = __reduce_max_sync(0xffffffffu, m);
+            if ((threadIdx.x & 31) == 0) atomicMax(mx + slot, m);
+        } else {
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        uu[v] = uc[v * n2 + node];
-        U0[v * n2 + node] = uu[v];
-    }
-    __syncthreads();
-
-    auto grads = [&](const double* Qk, double q[4], double qx[4], double qy[4]) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            const double* Qv = Qk + v * n2;
-            q[v] = Qv[node];
-            double sx = 0.0, sy = 0.0;
-#pragma unroll
-            for (int p = 0; p < n; ++p) {
-                sx += B.D[i][p] * Qv[j * n + p];
-                sy += B.D[j][p] * Qv[p * n + i];
-            }
-            qx[v] = sx * P.inv_hx;
-            qy[v] = sy * P.inv_hy;
+            for (int o = 1; o < C::tpc; o *= 2) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (tid == 0) mx[slot] = max(mx[slot], m);
         }
     };
-    // F, G of slice k go to RB / QXB as scratch during the forward recompute
-    auto divergence = [&](const double* Fk, const double* Gk, int v) {
-        double sx = 0.0, sy = 0.0;
+    auto smag = [&](double S) {
+        const uint32_t h = fx_mag(S);
+        const int e = (int)(h >> 20) - ed + 1023 - sh;
+        return h >= 0x7ff00000u ? h : (h < 0x100000u || e <= 0) ? 0u : (uint32_t)e << 20;
+    };
+    auto gv = [](int v) { return v == 0 ? 0 : v == 3 ? 2 : 1; };
+    // gradients at this node from the limbs of an iterate's time slice (plane stride ps)
+    auto gradients = [&](const Limbs* Qk, int ps, const int* eq, double gx[4], double gy[4], long long& R0) {
+        FxSum a[4], b[4];
 #pragma unroll
         for (int p = 0; p < n; ++p) {
-            sx += B.D[i][p] * Fk[v * n2 + j * n + p];
-            sy += B.D[j][p] * Gk[v * n2 + p * n + i];
+            const Limbs d = DT[i * n + p];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) a[v].add(d, Qk[v * ps + j * n + p]);
         }
-        return -(sx * P.inv_hx + sy * P.inv_hy);
+        R0 = a[1].value();
+#pragma unroll
+        for (int v = 0; v < 4; ++v) gx[v] = fx_to(a[v].value(), eq[gv(v)] + ed - 2102);
+#pragma unroll
+        for (int p = 0; p < n; ++p) {
+            const Limbs d = DT[n2 + j * n + p];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) b[v].add(d, Qk[v * ps + p * n + i]);
+        }
+        R0 += b[2].value();
+#pragma unroll
+        for (int v = 0; v < 4; ++v) gy[v] = fx_to(b[v].value(), eq[gv(v)] + ed - 2102);
     };
 
     // ---------------- forward recompute of the iterates (as k_predictor_fp64)
-    {
-        double q[4], qx[4], qy[4];
-        Flux4 f;
-        grads(U0, q, qx, qy);
-        ns_flux(q, qx, qy, z, pbar, rhobar, P, f);
+    double q[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) q[v] = u[(size_t)cell * SL + v * n2 + node];
+    if (tid < 8) mx[tid] = 0;
+    __syncthreads();
+    auto push_q = [&]() {
+        push(0, fx_mag(q[0]));
+        push(1, max(max(fx_mag(q[1]), fx_mag(q[2])), has_src ? smag(Sm[0]) : 0u));
+        push(2, fx_mag(q[3]));
+    };
+    push_q();
+    __syncthreads();
+    if (tid < 3) EX[tid] = fx_exp(mx[tid]);
+    if (on && k == 0) {
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            RB[v * n2 + node] = f.F[v];
-            QXB[v * n2 + node] = f.G[v];
+            U0[v * n2 + node] = fx_limbs(q[v], fx_exp(mx[gv(v)]));
+            US[v * n2 + node] = q[v];
         }
-        __syncthreads();
-        double R0[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) R0[v] = f.S[v] + Sm[v] + divergence(RB, QXB, v);
-#pragma unroll
-        for (int l = 0; l < n; ++l) {
-#pragma unroll
-            for (int v = 0; v < 4; ++v) iter(1, l)[v * n2 + node] = uu[v] + dt * (B.Kw1[l] * R0[v]);
-        }
-        __syncthreads();
     }
+    __syncthreads();
+    if (tid < 3) mx[tid] = 0;
 #pragma unroll 1
-    for (int r = 2; r <= n; ++r) {
-        double R[n][4];
+    for (int r = 0; r < n; ++r) {
+        const int ks = r == 0 ? 0 : k, ps = r == 0 ? n2 : n3;
+        const Limbs* Qk = r == 0 ? U0 : IT + (r - 1) * 4 * n3 + k * n2;
+        int eq[3];
 #pragma unroll
-        for (int k = 0; k < n; ++k) {
-            double q[4], qx[4], qy[4];
-            Flux4 f;
-            grads(iter(r - 1, k), q, qx, qy);
-            ns_flux(q, qx, qy, z, pbar, rhobar, P, f);
+        for (int a = 0; a < 3; ++a) eq[a] = EX[4 * r + a];
+        double gx[4], gy[4];
+        long long R0;
+        gradients(Qk, ps, eq, gx, gy, R0);
+        FxFlux f{0.0, 0.0, 0.0, 0.0, 0.0};
+        if (r > 0 || k == 0) f = ns_flux5(q, gx, gy, g, gz, pbar, P.gm1, P.mu, mu23, kR);
+        double S2 = Sm[2];
+        if (P.gravity) S2 = fma(-g, q[0] - rhobar, S2);
+        uint32_t m3 = max(max(max(fx_mag(f.f1), fx_mag(f.xy)), fx_mag(f.g2)), smag(S2)), m4 = max(fx_mag(f.f3), fx_mag(f.g3));
+        if (has_src) {
+            m3 = max(m3, smag(Sm[1]));
+            m4 = max(m4, smag(Sm[3]));
+        }
+        push(3, m3);
+        push(4, m4);
+        __syncthreads();
+        const int EF[2] = {fx_exp(mx[3]), fx_exp(mx[4])};
+        if (on && (r > 0 || k == 0)) {
+            Limbs* Fk = W + k * n2 + node;
+            Fk[0] = fx_limbs(f.f1, EF[0]);
+            Fk[n3] = fx_limbs(f.xy, EF[0]);
+            Fk[2 * n3] = fx_limbs(f.f3, EF[1]);
+            Fk[3 * n3] = fx_limbs(f.g2, EF[0]);
+            Fk[4 * n3] = fx_limbs(f.g3, EF[1]);
+        }
+        __syncthreads();
+        if (tid < 2) mx[3 + tid] = 0;
+        const int ER[3] = {eq[1] + ed - 1022 + sh, EF[0] + ed - 1022 + sh, EF[1] + ed - 1022 + sh};
+        Limbs* Rn = IT + r * 4 * n3;  // the next iterate's place holds the residual first
+        {
+            FxSum a[3];
+            const Limbs* Fx = W + ks * n2 + j * n;
+            const Limbs* Gy = W + ks * n2 + i;
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                RB[k * SL + v * n2 + node] = f.F[v];
-                QXB[k * SL + v * n2 + node] = f.G[v];
-                R[k][v] = f.S[v] + Sm[v];
+            for (int p = 0; p < n; ++p) {
+                const Limbs d = DT[i * n + p];
+#pragma unroll
+                for (int v = 0; v < 3; ++v) a[v].add(d, Fx[v * n3 + p]);
+            }
+#pragma unroll
+            for (int p = 0; p < n; ++p) {
+                const Limbs d = DT[n2 + j * n + p];
+                a[0].add(d, Gy[n3 + p * n]);
+                a[1].add(d, Gy[3 * n3 + p * n]);
+                a[2].add(d, Gy[4 * n3 + p * n]);
+            }
+            long long R[4];
+            R[0] = -(R0 >> sh);
+#pragma unroll
+            for (int v = 0; v < 3; ++v) R[v + 1] = -(a[v].value() >> sh);
+            if (has_src) {
+                R[0] += fx_from(Sm[0], ER[0]);
+                R[1] += fx_from(Sm[1], ER[1]);
+                R[3] += fx_from(Sm[3], ER[2]);
+            }
+            if (has_src || P.gravity) R[2] += fx_from(S2, ER[1]);
+            if (on) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) Rn[(v * n + k) * n2 + node] = fx_split(R[v]);
             }
         }
         __syncthreads();
+        {
+            FxSum a[4];
 #pragma unroll
-        for (int k = 0; k < n; ++k) {
+            for (int kk = 0; kk < n; ++kk) {
+                const Limbs d = K[k * n + kk];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) R[k][v] += divergence(RB + k * SL, QXB + k * SL, v);
-        }
-#pragma unroll
-        for (int l = 0; l < n; ++l) {
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                double acc = 0.0;
-#pragma unroll
-                for (int k = 0; k < n; ++k) acc += B.Kw[l][k] * R[k][v];
-                iter(r, l)[v * n2 + node] = uu[v] + dt * acc;
+                for (int v = 0; v < 4; ++v) a[v].add(d, Rn[(v * n + kk) * n2 + node]);
             }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) q[v] = fma(dt, fx_to(a[v].value(), ER[gv(v)] + B.KwE - 2102), US[v * n2 + node]);
+        }
+        push_q();
+        __syncthreads();
+        if (tid < 3) EX[4 * (r + 1) + tid] = fx_exp(mx[tid]);
+        if (on) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) Rn[(v * n + k) * n2 + node] = fx_limbs(q[v], fx_exp(mx[gv(v)]));
         }
         __syncthreads();
+        if (tid < 3) mx[tid] = 0;
     }
 
     // ---------------- reverse of the epilogue
-    // time-averaged face data of the forward (for the wave-speed adjoint)
-    const double* tr = trace + (size_t)cell * 4 * TR;
-    const double* tb = trace_bar + (size_t)cell * 4 * TR;
-    // adjoint of the face records incl. the wave speed, per face node
-    auto face_rec_bar = [&](int f, int m, double out[16]) {
-        const double* rb = tb + f * TR;
-        const double* rf = tr + f * TR;
+    // adjoints of the face records, the wave speed's folded into those of q
+    for (int o = tid; o < 4 * n; o += C::tpc) {
+        const int f = o / n, m = o - f * n;
+        const double* rb = trace_bar + ((size_t)cell * 4 + f) * TR;
+        const double* rf = trace + ((size_t)cell * 4 + f) * TR;
+        double out[4];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) out[c] = rb[c * n + m];
+        for (int c = 0; c < 4; ++c) out[c] = rb[c * n + m];
         const double sb = rb[16 * n + m];
         if (sb != 0.0) {
-            double qf[4] = {rf[0 * n + m], rf[1 * n + m], rf[2 * n + m], rf[3 * n + m]};
+            const double qf[4] = {rf[m], rf[n + m], rf[2 * n + m], rf[3 * n + m]};
             const bool xface = f < 2;
             const double zf = xface ? P.y0 + (iy + B.xi[m]) * P.hy : P.y0 + (iy + (f == 2 ? 1 : 0)) * P.hy;
             wave_speed_adj(qf, zf, xface, P, sb, out);
         }
-    };
-    // slot adjoints at this node: qbar, Fbar, Gbar, qxbar, qybar
-    double Aq[4] = {0, 0, 0, 0}, AF[4] = {0, 0, 0, 0}, AG[4] = {0, 0, 0, 0}, Ax[4] = {0, 0, 0, 0},
-           Ay[4] = {0, 0, 0, 0};
-    {
-        double e[16];
-        face_rec_bar(0, j, e);  // east: phi1[i]
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            Aq[v] += B.phi1[i] * e[v];
-            AF[v] += B.phi1[i] * e[4 + v];
-            Ax[v] += B.phi1[i] * e[8 + v];
-            Ay[v] += B.phi1[i] * e[12 + v];
-        }
-        face_rec_bar(1, j, e);  // west: phi0[i]
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            Aq[v] += B.phi0[i] * e[v];
-            AF[v] += B.phi0[i] * e[4 + v];
-            Ax[v] += B.phi0[i] * e[8 + v];
-            Ay[v] += B.phi0[i] * e[12 + v];
-        }
-        face_rec_bar(2, i, e);  // north: phi1[j]
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            Aq[v] += B.phi1[j] * e[v];
-            AG[v] += B.phi1[j] * e[4 + v];
-            Ax[v] += B.phi1[j] * e[8 + v];
-            Ay[v] += B.phi1[j] * e[12 + v];
-        }
-        face_rec_bar(3, i, e);  // south: phi0[j]
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            Aq[v] += B.phi0[j] * e[v];
-            AG[v] += B.phi0[j] * e[4 + v];
-            Ax[v] += B.phi0[j] * e[8 + v];
-            Ay[v] += B.phi0[j] * e[12 + v];
-        }
+        for (int c = 0; c < 16; ++c) FR[(f * 16 + c) * n + m] = c < 4 ? out[c] : rb[c * n + m];
     }
-    // weak volume residual: rvol_bar = dt lam'
+    __syncthreads();
+    // adjoints of the time averages at a node: qbar, Fbar, Gbar, qxbar, qybar [5][4][n2], from the faces and
+    // the weak volume residual (rvol_bar = dt lam')
     const double* lc = lam + (size_t)cell * SL;
-    double Sbar_b[4];
+    if (on)
+        for (int v = k; v < 4; v += n) {
+            auto fr = [&](int f, int c) { return FR[(f * 16 + c + v) * n + (f < 2 ? j : i)]; };
+            const double pe = B.phi1[i], pw = B.phi0[i], pn = B.phi1[j], ps = B.phi0[j];
+            auto all = [&](int c) { return fma(ps, fr(3, c), fma(pn, fr(2, c), fma(pw, fr(1, c), pe * fr(0, c)))); };
+            double sx = 0.0, sy = 0.0;
 #pragma unroll
-    for (int v = 0; v < 4; ++v) {
-        double sx = 0.0, sy = 0.0;
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-            sx += B.Vx[i][p] * lc[v * n2 + j * n + p];
-            sy += B.Vx[j][p] * lc[v * n2 + p * n + i];
+            for (int p = 0; p < n; ++p) {
+                sx = fma(B.Vx[i][p], lc[v * n2 + j * n + p], sx);
+                sy = fma(B.Vx[j][p], lc[v * n2 + p * n + i], sy);
+            }
+            Wd[v * n2 + node] = all(0);
+            Wd[(4 + v) * n2 + node] = fma(dt * P.inv_hx, sx, fma(pw, fr(1, 4), pe * fr(0, 4)));
+            Wd[(8 + v) * n2 + node] = fma(dt * P.inv_hy, sy, fma(ps, fr(3, 4), pn * fr(2, 4)));
+            Wd[(12 + v) * n2 + node] = all(8);
+            Wd[(16 + v) * n2 + node] = all(12);
         }
-        AF[v] += dt * P.inv_hx * sx;
-        AG[v] += dt * P.inv_hy * sy;
-        Sbar_b[v] = dt * lc[v * n2 + node];
-    }
-    // final evaluation and time averages: q^(n)_k
-#pragma unroll 1
-    for (int k = 0; k < n; ++k) {
-        double q[4], qx[4], qy[4];
-        grads(iter(n, k), q, qx, qy);
-        const double wk = B.w[k];
-        double Fb[4], Gb[4], Sb[4], qb[4], qxb[4], qyb[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            Fb[v] = wk * AF[v];
-            Gb[v] = wk * AG[v];
-            Sb[v] = wk * Sbar_b[v];
-            qb[v] = wk * Aq[v];
-            qxb[v] = wk * Ax[v];
-            qyb[v] = wk * Ay[v];
-        }
-        ns_flux_adj(q, qx, qy, z, P, Fb, Gb, Sb, qb, qxb, qyb);
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            QB[k * SL + v * n2 + node] = qb[v];
-            QXB[k * SL + v * n2 + node] = qxb[v];
-            QYB[k * SL + v * n2 + node] = qyb[v];
-        }
-    }
     __syncthreads();
-    // fold the gradient adjoints back: q_bar(j,p) += (1/h) sum_i' D[i'][p] qx_bar(j,i')
-    auto fold = [&]() {
-#pragma unroll 1
-        for (int k = 0; k < n; ++k) {
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                double sx = 0.0, sy = 0.0;
-#pragma unroll
-                for (int p = 0; p < n; ++p) {
-                    sx += B.D[p][i] * QXB[k * SL + v * n2 + j * n + p];
-                    sy += B.D[p][j] * QYB[k * SL + v * n2 + p * n + i];
-                }
-                QB[k * SL + v * n2 + node] += sx * P.inv_hx + sy * P.inv_hy;
-            }
-        }
-    };
-    fold();
-    __syncthreads();
-
-    // ---------------- reverse sweeps r = n .. 2
-    double ub[4] = {0, 0, 0, 0};
-#pragma unroll 1
-    for (int r = n; r >= 2; --r) {
-        // q^(r)_l = u + dt sum_k Kw[l][k] R_k(q^(r-1))
-        double Rb[n][4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            double qbl[n];
-#pragma unroll
-            for (int l = 0; l < n; ++l) {
-                qbl[l] = QB[l * SL + v * n2 + node];
-                ub[v] += qbl[l];
-            }
-#pragma unroll
-            for (int k = 0; k < n; ++k) {
-                double acc = 0.0;
-#pragma unroll
-                for (int l = 0; l < n; ++l) acc += B.Kw[l][k] * qbl[l];
-                Rb[k][v] = dt * acc;
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < n; ++k)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) RB[k * SL + v * n2 + node] = Rb[k][v];
-        __syncthreads();
-        // R_k = -(1/hx) D_x F_k - (1/hy) D_y G_k + S_k: F_bar(j,p) = -(1/hx) sum_i' D[i'][p] Rb(j,i')
-#pragma unroll 1
-        for (int k = 0; k < n; ++k) {
-            double Fb[4], Gb[4], Sb[4];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                double sx = 0.0, sy = 0.0;
-#pragma unroll
-                for (int p = 0; p < n; ++p) {
-                    sx += B.D[p][i] * RB[k * SL + v * n2 + j * n + p];
-                    sy += B.D[p][j] * RB[k * SL + v * n2 + p * n + i];
-                }
-                Fb[v] = -sx * P.inv_hx;
-                Gb[v] = -sy * P.inv_hy;
-                Sb[v] = Rb[k][v];
-            }
-            double q[4], qx[4], qy[4];
-            grads(iter(r - 1, k), q, qx, qy);
-            double qb[4] = {0, 0, 0, 0}, qxb[4] = {0, 0, 0, 0}, qyb[4] = {0, 0, 0, 0};
-            ns_flux_adj(q, qx, qy, z, P, Fb, Gb, Sb, qb, qxb, qyb);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                QXB[k * SL + v * n2 + node] = qxb[v];
-                QYB[k * SL + v * n2 + node] = qyb[v];
-                Rb[k][v] = qb[v];  // reuse: point-wise part of q^(r-1)_k bar
-            }
-        }
-        __syncthreads();  // all reads of QB (this sweep) and RB done, QXB/QYB complete
-#pragma unroll
-        for (int k = 0; k < n; ++k)
-#pragma unroll
-            for (int v = 0; v < 4; ++v) QB[k * SL + v * n2 + node] = Rb[k][v];
-        fold();
-        __syncthreads();
-    }
-    // ---------------- sweep 1: q^(1)_l = u + dt Kw1[l] R(u)
+    // final evaluation and time averages: q^(n)_k (still in q)
+    double qb[4], gxb[4], gyb[4], ub[4] = {0.0, 0.0, 0.0, 0.0};
     {
-        double R0b[4];
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            double acc = 0.0;
-#pragma unroll
-            for (int l = 0; l < n; ++l) {
-                const double b = QB[l * SL + v * n2 + node];
-                ub[v] += b;
-                acc += B.Kw1[l] * b;
-            }
-            R0b[v] = dt * acc;
-            RB[v * n2 + node] = R0b[v];
-        }
-        __syncthreads();
+        const double wk = B.w[k];
         double Fb[4], Gb[4];
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            double sx = 0.0, sy = 0.0;
-#pragma unroll
-            for (int p = 0; p < n; ++p) {
-                sx += B.D[p][i] * RB[v * n2 + j * n + p];
-                sy += B.D[p][j] * RB[v * n2 + p * n + i];
-            }
-            Fb[v] = -sx * P.inv_hx;
-            Gb[v] = -sy * P.inv_hy;
+            qb[v] = wk * Wd[v * n2 + node];
+            Fb[v] = wk * Wd[(4 + v) * n2 + node];
+            Gb[v] = wk * Wd[(8 + v) * n2 + node];
+            gxb[v] = wk * Wd[(12 + v) * n2 + node];
+            gyb[v] = wk * Wd[(16 + v) * n2 + node];
         }
-        double q[4], qx[4], qy[4];
-        grads(U0, q, qx, qy);
-        double qb[4] = {0, 0, 0, 0}, qxb[4] = {0, 0, 0, 0}, qyb[4] = {0, 0, 0, 0};
-        ns_flux_adj(q, qx, qy, z, P, Fb, Gb, R0b, qb, qxb, qyb);
+        double gx[4], gy[4];
+        long long R0;
+        gradients(IT + (n - 1) * 4 * n3 + k * n2, n3, EX + 4 * n, gx, gy, R0);
+        ns_flux5_adj(q, gx, gy, g, gz, P.gm1, P.mu, mu23, kR, Fb, Gb, wk * dt * lc[2 * n2 + node], qb, gxb, gyb);
+    }
+    // fold the gradient adjoints back: q_bar(j,p) += (1/h) sum_i' D[i'][p] qx_bar(j,i'); slices: time nodes that hold data
+    auto fold = [&](bool mine) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) push(v, mine ? max(fx_mag(gxb[v]), fx_mag(gyb[v])) : 0u);
+        __syncthreads();
+        int E[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) E[v] = fx_exp(mx[v]);
+        if (on && mine) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                W[(v * n + k) * n2 + node] = fx_limbs(gxb[v], E[v]);
+                W[((4 + v) * n + k) * n2 + node] = fx_limbs(gyb[v], E[v]);
+            }
+        }
+        __syncthreads();
+        if (tid < 4) mx[tid] = 0;
+        if (!mine) return;
+        FxSum a[4];
+#pragma unroll
+        for (int p = 0; p < n; ++p) {
+            const Limbs dx = DT[p * n + i], dy = DT[n2 + p * n + j];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                a[v].add(dx, W[(v * n + k) * n2 + j * n + p]);
+                a[v].add(dy, W[((4 + v) * n + k) * n2 + p * n + i]);
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) qb[v] += fx_to(a[v].value(), E[v] + ed - 2102);
+    };
+    fold(true);
+
+    // ---------------- reverse sweeps r = n .. 1: q^(r)_l = u + dt sum_k Kw[l][k] R_k(q^(r-1));
+    // in sweep 1 the residual R(u) is one time slice's, weighted by the row sums of Kw
+#pragma unroll 1
+    for (int r = n; r >= 1; --r) {
+        const bool mine = r > 1 || k == 0;
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            QXB[v * n2 + node] = qxb[v];
-            QYB[v * n2 + node] = qyb[v];
             ub[v] += qb[v];
+            push(4 + v, fx_mag(qb[v]));
+        }
+        __syncthreads();  // also: every thread has folded, W is free
+        int E[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) E[v] = fx_exp(mx[4 + v]);
+        if (on) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) W[(v * n + k) * n2 + node] = fx_limbs(qb[v], E[v]);
+        }
+        __syncthreads();
+        if (tid < 4) mx[4 + tid] = 0;
+        double R2 = 0.0;
+        if (mine) {
+            const int eK = r > 1 ? B.KwE : B.KwE + 3;
+            FxSum a[4];
+#pragma unroll
+            for (int l = 0; l < n; ++l) {
+                const Limbs d = r > 1 ? K[l * n + k] : K[n2 + l];
+#pragma unroll
+                for (int v = 0; v < 4; ++v) a[v].add(d, W[(v * n + l) * n2 + node]);
+            }
+            R2 = fx_to(a[2].value(), E[2] + eK - 2102);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                E[v] += eK - 2102 + 3 + 1080;  // |sum| < 2^61: below 2^58 after the shift
+                if (on) W[((4 + v) * n + k) * n2 + node] = fx_split(a[v].value() >> 3);
+            }
         }
         __syncthreads();
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            double sx = 0.0, sy = 0.0;
+        for (int v = 0; v < 4; ++v) qb[v] = gxb[v] = gyb[v] = 0.0;
+        if (mine) {
+            // R_k = -(1/hx) D_x F_k - (1/hy) D_y G_k + S_k: F_bar(j,p) = -(dt/hx) sum_i' D[i'][p] R_bar(j,i')
+            double Fb[4], Gb[4];
+            {
+                FxSum a[4], b[4];
 #pragma unroll
-            for (int p = 0; p < n; ++p) {
-                sx += B.D[p][i] * QXB[v * n2 + j * n + p];
-                sy += B.D[p][j] * QYB[v * n2 + p * n + i];
+                for (int p = 0; p < n; ++p) {
+                    const Limbs dx = DM[p * n + i], dy = DM[n2 + p * n + j];
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        a[v].add(dx, W[((4 + v) * n + k) * n2 + j * n + p]);
+                        b[v].add(dy, W[((4 + v) * n + k) * n2 + p * n + i]);
+                    }
+                }
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    Fb[v] = fx_to(a[v].value(), E[v] + em - 2102);
+                    Gb[v] = fx_to(b[v].value(), E[v] + em - 2102);
+                }
             }
-            ub[v] += sx * P.inv_hx + sy * P.inv_hy;
-        }
-    }
-    if (active) {
-        double* lo = lam_out + (size_t)cell * SL;
+            const Limbs* Qk = r == 1 ? U0 : IT + (r - 2) * 4 * n3 + k * n2;
+            const int ps = r == 1 ? n2 : n3;
+            const int* eq = EX + 4 * (r - 1);
+            double gx[4], gy[4];
+            long long R0;
+            gradients(Qk, ps, eq, gx, gy, R0);
 #pragma unroll
-        for (int v = 0; v < 4; ++v) lo[v * n2 + node] = lc[v * n2 + node] + ub[v];
+            for (int v = 0; v < 4; ++v) {
+                const Limbs o = Qk[v * ps + node];
+                q[v] = r == 1 ? US[v * n2 + node] : fx_to((long long)o.h * (1ll << 29) + o.l, eq[gv(v)] - 1080);
+            }
+            ns_flux5_adj(q, gx, gy, g, gz, P.gm1, P.mu, mu23, kR, Fb, Gb, dt * R2, qb, gxb, gyb);
+        }
+        fold(mine);
     }
+    // sum over the time nodes of the adjoints that reached u
+    __syncthreads();
+    if (on) {
+#pragma unroll
+        for (int v = 0; v < 4; ++v) Wd[(v * n + k) * n2 + node] = ub[v] + qb[v];
+    }
+    __syncthreads();
+    if (on && active)
+        for (int v = k; v < 4; v += n) {
+            double s = lc[v * n2 + node];
+#pragma unroll
+            for (int l = 0; l < n; ++l) s += Wd[(v * n + l) * n2 + node];
+            lam_out[(size_t)cell * SL + v * n2 + node] = s;
+        }
 }
 
 template <int N>
 static int adj_n(const double* u, const double* lam, double* lam_out, const double* trace, double* trace_bar,
                  int cells, double dt, const Basis& B, const Phys& P, const Background& bg, cudaStream_t s) {
     using C = AdjCfg<N>;
-    const int blocks = (cells + C::cpb - 1) / C::cpb;
-    k_corrector_adj_fp64<N, C::cpb><<<blocks, C::threads, 0, s>>>(lam, trace, trace_bar, cells, dt, B, P, bg);
+    constexpr int cpb = N <= 2 ? 4 : N <= 4 ? 2 : 1;  // cells per block of the corrector's adjoint
+    k_corrector_adj_fp64<N, cpb><<<(cells + cpb - 1) / cpb, cpb*(N + 1) * (N + 1), 0, s>>>(lam, trace, trace_bar, cells,
+                                                                                      dt, B, P, bg);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return (int)e;
-    auto kern = k_predictor_adj_fp64<N, C::cpb>;
+    auto kern = k_predictor_adj_fp64<N>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
     if (e != cudaSuccess) return (int)e;
-    kern<<<blocks, C::threads, C::smem, s>>>(u, lam, trace, trace_bar, lam_out, cells, dt, B, P, bg);
+    kern<<<(cells + C::cpb - 1) / C::cpb, C::threads, C::smem, s>>>(u, lam, trace, trace_bar, lam_out, cells, dt, B, P,
+                                                               bg);
     return (int)cudaGetLastError();
 }
 
