@@ -13,13 +13,14 @@
 // a slip-wall ghost with the background of Eq. 6 and the heat flux of
 // Eq. 10, or the analytic ABC field) and the FP64 update u += dt (rvol - lift).
 //
-// Thread mapping: CPB cells per block, one thread per spatial node (l, j, i);
-// each thread walks the n time nodes of its node, so the Picard update's
-// time contraction stays in registers.  Shared memory per cell: the n time
-// slices of the iterate and the F, G, H of one time slice (the divergence of
-// slice k is taken before slice k+1's fluxes overwrite them); after the last
-// sweep the same space holds the seven time-averaged fields the volume term
-// and the traces contract.
+// Thread mapping: the FP64 predictor runs one thread per space-time node (see
+// k3_predictor); the mixed predictor and the corrector CPB cells per block, one
+// thread per spatial node (l, j, i).  A thread of the mixed predictor walks the
+// n time nodes of its node, so the Picard update's time contraction stays in
+// registers; its shared memory holds per cell the n time slices of the iterate
+// and the F, G, H of one time slice (the divergence of slice k is taken before
+// slice k+1's fluxes overwrite them), after the last sweep the seven
+// time-averaged fields the volume term and the traces contract.
 //
 // Layouts: u[c][v][l][j][i], c = (iz ny + iy) nx + ix, v in (rho, rho u,
 // rho v, rho w, rho E); traces [c][face E W N S T B][kTr3][n^2], face nodes
@@ -33,6 +34,7 @@
 #include <vector>
 
 #include "adg_convert.cuh"
+#include "adg_fixed.cuh"
 #include "adg_internal.h"
 #include "adg_mesh.h"
 
@@ -159,212 +161,360 @@ struct Cfg3 {
     static constexpr size_t smem = (size_t)cpb * slots * 5 * n3 * sizeof(double);
 };
 
+// FP64 predictor: the scheme of the 2D one (adg_fp64_body.cuh) -- one thread
+// per space-time node (k, l, j, i), every contraction on the integer pipe in
+// 58-bit block-scaled fixed point (adg_fixed.cuh), the point-wise fluxes alone
+// in FP64.
 template <int N>
-__global__ void __launch_bounds__(Cfg3<N>::threads)
+struct Fx3Cfg {
+    static constexpr int n = N + 1, n2 = n * n, n3 = n2 * n, n4 = n3 * n;
+    // degree 2 (81 threads a cell) lets cells share warps: 96 would idle 16% of
+    // the FP64 lanes; elsewhere whole warps (degree 1: half warps) per cell
+    static constexpr int tpc = N == 2 ? 81 : N == 4 ? 640 : n4;
+    static constexpr int cpb = N == 1 ? 8 : N == 2 ? 3 : 1;
+    static constexpr int threads = (cpb * tpc + 31) / 32 * 32;
+    // blocks per SM asked of the register allocator; us a step at 3 / 4 / 5 / 6: degree 1 (41^3 cells)
+    // 1098 / 1126 / 1144 / 1140, 2 (25^3) 1297 / 1281 / 1255 / 1301, 3 (17^3) 1299 / 1342 / 1279 / 1327;
+    // degree 4 (13^3) 2134 with 1, 2152 with 2
+    static constexpr int resident = N == 1 ? 3 : N == 4 ? 1 : 5;
+    // per cell, in 8-byte words: q (5) and the fluxes (9) of every space-time
+    // node, u, D/h, the face values of q-bar, the group magnitudes
+    static constexpr int words = 14 * n4 + 5 * n3 + 3 * n2 + 30 * n2 + 4;
+    static constexpr size_t smem = ((size_t)cpb * words + n2) * 8;
+};
+
+// Point-wise fluxes (Eqs. 1-5, 7) in 78 FP64 operations: the mass fluxes are
+// the momenta; t: xx, xy, xz, yy, yz, zz of the symmetric momentum flux; e:
+// energy flux; with w_ab = d_b(rho v_a) - v_a d_b(rho),
+//   c_v rho d_b T = d_b E - (E/rho) d_b rho - v.w_b - rho g (b = z).
+struct Fx3Flux {
+    double t[6], e[3];
+};
+__device__ __forceinline__ Fx3Flux ns_flux9(const double q[5], const double g[3][5], double gg, double gz, double pbar,
+                                            double gm1, double mu, double mu23, double kR) {
+    const double rinv = fx_rcp(q[0]);
+    const double v[3] = {q[1] * rinv, q[2] * rinv, q[3] * rinv};
+    const double ke2 = fma(q[3], v[2], fma(q[2], v[1], q[1] * v[0]));
+    const double p = gm1 * fma(-0.5, ke2, fma(-gz, q[0], q[4]));
+    const double pp = p - pbar, Ep = q[4] + p, eR = q[4] * rinv;
+    double w[3][3];  // w[a][b], rho times the velocity gradient
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) w[a][b] = fma(-v[a], g[b][0], g[b][1 + a]);
+    const double m23 = mu23 * rinv, mr = -mu * rinv, kr = kR * rinv;
+    const double div = w[0][0] + w[1][1] + w[2][2];
+    const double sd[3] = {m23 * fma(-3.0, w[0][0], div), m23 * fma(-3.0, w[1][1], div), m23 * fma(-3.0, w[2][2], div)};
+    const double sxy = mr * (w[0][1] + w[1][0]), sxz = mr * (w[0][2] + w[2][0]), syz = mr * (w[1][2] + w[2][1]);
+    Fx3Flux f;
+    f.t[0] = fma(q[1], v[0], pp + sd[0]);
+    f.t[1] = fma(q[1], v[1], sxy);
+    f.t[2] = fma(q[1], v[2], sxz);
+    f.t[3] = fma(q[2], v[1], pp + sd[1]);
+    f.t[4] = fma(q[2], v[2], syz);
+    f.t[5] = fma(q[3], v[2], pp + sd[2]);
+    const double so[3][2] = {{sxy, sxz}, {sxy, syz}, {sxz, syz}};
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        double h = fma(-v[2], w[2][b], fma(-v[1], w[1][b], fma(-v[0], w[0][b], fma(-eR, g[b][0], g[b][4]))));
+        if (b == 2) h = fma(-gg, q[0], h);
+        f.e[b] = fma(-kr, h, fma(v[b], Ep + sd[b], fma(v[b == 0 ? 1 : 0], so[b][0], v[b == 2 ? 1 : 2] * so[b][1])));
+    }
+    return f;
+}
+
+// slot of the momentum flux (a, b) among the six; slot of component c of a face
+// record in direction dir (q, then the normal flux) among q (5), t (6), e (3)
+__device__ __forceinline__ int fx3_t(int a, int b) { return a + b + (a > 0 && b > 0 ? 1 : 0); }
+__device__ __forceinline__ int fx3_slot(int c, int dir) {
+    return c < 5 ? c : c == 5 ? 1 + dir : c < 9 ? 5 + fx3_t(c - 6, dir) : 11 + dir;
+}
+
+template <int N>
+__global__ void __launch_bounds__(Fx3Cfg<N>::threads, Fx3Cfg<N>::resident)
 k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __restrict__ trace, int cells,
              double dt, const Basis B, const Phys3 P, const Bg3 bg) {
-    using C = Cfg3<N>;
-    constexpr int n = C::n, n2 = C::n2, n3 = C::n3, SL = 5 * n3;
+    using C = Fx3Cfg<N>;
+    constexpr int n = C::n, n2 = C::n2, n3 = C::n3, n4 = C::n4, SL = 5 * n3;
     extern __shared__ double sm[];
-    const int cl = threadIdx.x / n3;
-    const int node = threadIdx.x - cl * n3;
-    const int l = node / n2, j = (node / n) % n, i = node % n;
-    const int cell_raw = blockIdx.x * C::cpb + cl;
-    const bool active = cell_raw < cells;
-    const int cell = active ? cell_raw : cells - 1;
-    const int iz = cell / (P.nc[0] * P.nc[1]);
-    double* Q = sm + (size_t)cl * C::slots * SL;  // [n][5][n3]
-    double* Fs = Q + n * SL;                      // [3][5][n3]: F, G, H of one time slice
-    const double z = P.org[2] + (iz + B.xi[l]) * P.h[2];
-    const double pbar = bg.pn[iz * n + l], rhobar = bg.rn[iz * n + l];
+    const int cl = min((int)threadIdx.x / C::tpc, C::cpb - 1);
+    const int tid = threadIdx.x - cl * C::tpc;
+    const bool on = tid < n4;  // the rest repeats the last node without stores
+    const int id = on ? tid : n4 - 1;
+    const int k = id / n3, node = id - k * n3, l = node / n2, j = (node / n) % n, i = node % n;
+    double* base = sm + (size_t)cl * C::words;
+    Limbs* Q = reinterpret_cast<Limbs*>(base);  // [5][n][n3]; the residual between the sweeps' halves
+    Limbs* F = Q + 5 * n4;                      // [9][n][n3]
+    double* US = base + 14 * n4;                // [5][n3]
+    Limbs* DT = reinterpret_cast<Limbs*>(US + 5 * n3);  // [3][n][n]
+    double* TQ = US + 5 * n3 + 3 * n2;          // [6][5][n2]
+    uint32_t* mx = reinterpret_cast<uint32_t*>(TQ + 30 * n2);
+    Limbs* K = reinterpret_cast<Limbs*>(sm + (size_t)C::cpb * C::words);
+    for (int a = threadIdx.x; a < n2; a += blockDim.x) K[a] = Limbs{B.KwH[a / n][a % n], B.KwL[a / n][a % n]};
+    const int ed = fx_exp(fx_mag(B.Dmax * fmax(P.inv_h[0], fmax(P.inv_h[1], P.inv_h[2]))));
+    const int sh = (int)(fx_mag(B.Drow * (P.inv_h[0] + P.inv_h[1] + P.inv_h[2])) >> 20) - ed + 1;
+    for (int a = tid; a < 3 * n2; a += C::tpc)
+        if (on) DT[a] = fx_split_centred(fx_from(B.D[a % n2 / n][a % n] * P.inv_h[a / n2], ed));
+    const double gg = P.gravity ? P.g : 0.0, mu23 = (2.0 / 3.0) * P.mu, kR = P.gm1 * P.kappa * P.invR;
 
-    double uu[5];
-    const double* uc = u + (size_t)cell * SL;
+    // largest magnitude of a group over the cell's threads: a warp reduction and
+    // one shared-memory atomic per warp and cell in it
+    auto push = [&](int slot, uint32_t m) {
+        if constexpr (C::tpc % 32 == 0) {
+            m = __reduce_max_sync(0xffffffffu, m);
+            if ((threadIdx.x & 31) == 0) atomicMax(mx + slot, m);
+        } else if constexpr (C::tpc < 32) {
 #pragma unroll
-    for (int v = 0; v < 5; ++v) {
-        uu[v] = uc[v * n3 + node];
-        Q[v * n3 + node] = uu[v];
-    }
-    __syncthreads();
-
-    // state, gradients and fluxes of time slice Qk at this node
-    auto eval = [&](const double* Qk, double q[5], double g[3][5], double f[3][5], double& src) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) {
-            const double* Qv = Qk + v * n3;
-            q[v] = Qv[node];
-            double sx = 0.0, sy = 0.0, sz = 0.0;
-#pragma unroll
-            for (int p = 0; p < n; ++p) {
-                sx += B.D[i][p] * Qv[(l * n + j) * n + p];
-                sy += B.D[j][p] * Qv[(l * n + p) * n + i];
-                sz += B.D[l][p] * Qv[(p * n + j) * n + i];
-            }
-            g[0][v] = sx * P.inv_h[0];
-            g[1][v] = sy * P.inv_h[1];
-            g[2][v] = sz * P.inv_h[2];
+            for (int o = 1; o < C::tpc; o *= 2) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if (tid == 0) mx[slot] = max(mx[slot], m);
+        } else {  // at most two cells in a warp
+            const int first = __shfl_sync(0xffffffffu, cl, 0);
+            const uint32_t a = __reduce_max_sync(0xffffffffu, cl == first ? m : 0u);
+            const uint32_t b = __reduce_max_sync(0xffffffffu, cl == first ? 0u : m);
+            if ((threadIdx.x & 31) == 0) atomicMax(mx + slot, a);
+            if ((threadIdx.x & 31) == 31 && cl != first) atomicMax(mx + slot, b);
         }
-        ns_flux3(q, g, z, pbar, rhobar, P, false, f, src);
     };
-    auto store = [&](const double f[3][5]) {
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-#pragma unroll
-            for (int v = 0; v < 5; ++v) Fs[(b * 5 + v) * n3 + node] = f[b][v];
-    };
-    // -dF/dx - dG/dy - dH/dz at this node from the slice in Fs
-    auto divergence = [&](int v) {
-        const double* Fv = Fs + v * n3;
-        const double* Gv = Fs + (5 + v) * n3;
-        const double* Hv = Fs + (10 + v) * n3;
-        double sx = 0.0, sy = 0.0, sz = 0.0;
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-            sx += B.D[i][p] * Fv[(l * n + j) * n + p];
-            sy += B.D[j][p] * Gv[(l * n + p) * n + i];
-            sz += B.D[l][p] * Hv[(p * n + j) * n + i];
-        }
-        return -(sx * P.inv_h[0] + sy * P.inv_h[1] + sz * P.inv_h[2]);
-    };
+    const Limbs *Dx = DT + i * n, *Dy = DT + n2 + j * n, *Dz = DT + 2 * n2 + l * n;
+    const int ox = (l * n + j) * n, oy = l * n2 + i, oz = j * n + i;  // lines through the node: strides 1, n, n2
 
-    // sweep 1: the iterate is u at every time node: one flux evaluation
-    {
-        double q[5], g[3][5], f[3][5], src;
-        eval(Q, q, g, f, src);
-        store(f);
-        __syncthreads();
-        double R0[5];
-#pragma unroll
-        for (int v = 0; v < 5; ++v) R0[v] = (v == 3 ? src : 0.0) + divergence(v);
-#pragma unroll
-        for (int k = 0; k < n; ++k)
-#pragma unroll
-            for (int v = 0; v < 5; ++v) Q[k * SL + v * n3 + node] = uu[v] + dt * (B.Kw1[k] * R0[v]);
-        __syncthreads();
-    }
-    // sweeps 2..n
 #pragma unroll 1
-    for (int r = 1; r < n; ++r) {
-        double R[n][5];
+    for (int c0 = blockIdx.x * C::cpb; c0 < cells; c0 += gridDim.x * C::cpb) {
+        const bool active = c0 + cl < cells;
+        const int cell = active ? c0 + cl : cells - 1;
+        const int ic0 = cell % P.nc[0], ic1 = (cell / P.nc[0]) % P.nc[1], iz = cell / (P.nc[0] * P.nc[1]);
+        const double gz = gg * (P.org[2] + (iz + B.xi[l]) * P.h[2]);
+        const double pbar = bg.pn[iz * n + l], rhobar = bg.rn[iz * n + l];
+        double q[5];
 #pragma unroll
-        for (int k = 0; k < n; ++k) {
-            double q[5], g[3][5], f[3][5], src;
-            eval(Q + k * SL, q, g, f, src);
-            __syncthreads();  // the previous slice's divergence has read Fs
-            store(f);
-            __syncthreads();
+        for (int v = 0; v < 5; ++v) q[v] = u[(size_t)cell * SL + v * n3 + node];
+        int EQ[3], EF[2];
+        auto push_q = [&]() {
+            push(0, fx_mag(q[0]));
+            push(1, max(max(fx_mag(q[1]), fx_mag(q[2])), fx_mag(q[3])));
+            push(2, fx_mag(q[4]));
+        };
+        auto eq = [&](int v) { return EQ[v == 0 ? 0 : v == 4 ? 2 : 1]; };
+        auto store_q = [&](int slice) {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) R[k][v] = (v == 3 ? src : 0.0) + divergence(v);
-        }
-#pragma unroll
-        for (int k = 0; k < n; ++k)
-#pragma unroll
-            for (int v = 0; v < 5; ++v) {
-                double acc = 0.0;
-#pragma unroll
-                for (int m = 0; m < n; ++m) acc += B.Kw[k][m] * R[m][v];
-                Q[k * SL + v * n3 + node] = uu[v] + dt * acc;
-            }
+            for (int v = 0; v < 5; ++v) Q[(v * n + slice) * n3 + node] = fx_limbs(q[v], eq(v));
+        };
+        if (tid < 5) mx[tid] = 0;
         __syncthreads();
-    }
+        push_q();
+        __syncthreads();
+#pragma unroll
+        for (int a = 0; a < 3; ++a) EQ[a] = fx_exp(mx[a]);
+        if (id < n3 && on) {
+            store_q(0);
+#pragma unroll
+            for (int v = 0; v < 5; ++v) US[v * n3 + node] = q[v];
+        }
+        __syncthreads();
+        if (tid < 3) mx[tid] = 0;
 
-    // final evaluation on the converged iterate: time averages
-    double qb[5], fb[3][5], gb[3][5], sb = 0.0;
+        Fx3Flux f;
+        // sweeps 0..n-1 and the final evaluation r = n; in sweep 0 the iterate is
+        // u at every time node: the threads of time node 0 evaluate the fluxes
+#pragma unroll 1
+        for (int r = 0;; ++r) {
+            const int ks = r == 0 ? 0 : k;
+            const Limbs* Qk = Q + ks * n3;
+            long long R0;  // divergence of the momentum
 #pragma unroll
-    for (int v = 0; v < 5; ++v) {
-        qb[v] = 0.0;
-#pragma unroll
-        for (int b = 0; b < 3; ++b) fb[b][v] = gb[b][v] = 0.0;
-    }
-#pragma unroll
-    for (int k = 0; k < n; ++k) {
-        double q[5], g[3][5], f[3][5], src;
-        eval(Q + k * SL, q, g, f, src);
-        const double wk = B.w[k];
-        sb += wk * src;
-#pragma unroll
-        for (int v = 0; v < 5; ++v) {
-            qb[v] += wk * q[v];
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                fb[b][v] += wk * f[b][v];
-                gb[b][v] += wk * g[b][v];
-            }
-        }
-    }
-    __syncthreads();
-    // slots: 0 q-bar, 1..3 F-, G-, H-bar, 4..6 qx-, qy-, qz-bar
-    double* A = Q;
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-        A[v * n3 + node] = qb[v];
-#pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            A[(1 + b) * SL + v * n3 + node] = fb[b][v];
-            A[(4 + b) * SL + v * n3 + node] = gb[b][v];
-        }
-    }
-    __syncthreads();
-    if (active) {
-        double* rc = rvol + (size_t)cell * SL;
-#pragma unroll
-        for (int v = 0; v < 5; ++v) {
-            const double* Fv = A + 1 * SL + v * n3;
-            const double* Gv = A + 2 * SL + v * n3;
-            const double* Hv = A + 3 * SL + v * n3;
-            double sx = 0.0, sy = 0.0, sz = 0.0;
-#pragma unroll
-            for (int p = 0; p < n; ++p) {
-                sx += B.Vx[p][i] * Fv[(l * n + j) * n + p];
-                sy += B.Vx[p][j] * Gv[(l * n + p) * n + i];
-                sz += B.Vx[p][l] * Hv[(p * n + j) * n + i];
-            }
-            rc[v * n3 + node] = sx * P.inv_h[0] + sy * P.inv_h[1] + sz * P.inv_h[2] + (v == 3 ? sb : 0.0);
-        }
-    }
-    // boundary-extrapolated traces of faces E, W (x), N, S (y), T, B (z)
-    const int ic0 = cell % P.nc[0], ic1 = (cell / P.nc[0]) % P.nc[1];
-    for (int idx = node; idx < 6 * n2; idx += n3) {
-        const int f = idx / n2, m = idx - f * n2;
-        const int a = m / n, b = m - a * n;
-        const int dir = f >> 1;
-        const double* phi = (f & 1) ? B.phi0 : B.phi1;
-        // the gradient components are read only by slip-wall ghosts: written
-        // for wall faces alone
-        const int icd = dir == 0 ? ic0 : dir == 1 ? ic1 : iz;
-        const int ncd = dir == 0 ? P.nc[0] : dir == 1 ? P.nc[1] : P.nc[2];
-        const int bcd = dir == 0 ? P.bc[0] : dir == 1 ? P.bc[1] : P.bc[2];
-        const bool wallface = bcd == ADG_BC_WALL && ((f & 1) ? icd == 0 : icd == ncd - 1);
-        double rec[kTr3];
-#pragma unroll
-        for (int c = 0; c < 5; ++c) {
-            if (c >= 2 && !wallface) {
-#pragma unroll
-                for (int v = 0; v < 5; ++v) rec[c * 5 + v] = 0.0;
-                continue;
-            }
-            const int slot = c == 0 ? 0 : c == 1 ? 1 + dir : 2 + c;  // q, normal flux, qx, qy, qz
-#pragma unroll
-            for (int v = 0; v < 5; ++v) {
-                const double* S = A + slot * SL + v * n3;
-                double s = 0.0;
+            for (int a = 0; a < 6; ++a) f.t[a] = 0.0;
+            f.e[0] = f.e[1] = f.e[2] = 0.0;
+            if (r == 0 && k > 0) {
+                FxSum a;
 #pragma unroll
                 for (int p = 0; p < n; ++p) {
-                    const int at = dir == 0 ? (a * n + b) * n + p : dir == 1 ? (a * n + p) * n + b : (p * n + a) * n + b;
-                    s += phi[p] * S[at];
+                    a.add(Dx[p], Qk[n4 + ox + p]);
+                    a.add(Dy[p], Qk[2 * n4 + oy + p * n]);
+                    a.add(Dz[p], Qk[3 * n4 + oz + p * n2]);
                 }
-                rec[c * 5 + v] = s;
+                R0 = a.value();
+            } else {
+                double g[3][5];
+                R0 = 0;
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    const Limbs* D = b == 0 ? Dx : b == 1 ? Dy : Dz;
+                    const Limbs* L = Qk + (b == 0 ? ox : b == 1 ? oy : oz);
+                    FxSum a[5];
+#pragma unroll
+                    for (int p = 0; p < n; ++p) {
+                        const Limbs d = D[p];
+#pragma unroll
+                        for (int v = 0; v < 5; ++v) a[v].add(d, L[v * n4 + p * (b == 0 ? 1 : b == 1 ? n : n2)]);
+                    }
+                    R0 += a[1 + b].value();
+#pragma unroll
+                    for (int v = 0; v < 5; ++v) g[b][v] = fx_to(a[v].value(), eq(v) + ed - 2102);
+                }
+                f = ns_flux9(q, g, gg, gz, pbar, P.gm1, P.mu, mu23, kR);
+            }
+            if (r == n) break;
+            const double S = P.gravity ? -gg * (q[0] - rhobar) : 0.0;
+            uint32_t m3 = 0, m4 = 0;
+            if (P.gravity) {  // magnitude the momentum group must have for S to fit the residual's scale
+                const uint32_t hs = fx_mag(S);
+                const int e = (int)(hs >> 20) - ed + 1023 - sh;
+                m3 = hs >= 0x7ff00000u ? hs : (hs < 0x100000u || e <= 0) ? 0u : (uint32_t)e << 20;
+            }
+#pragma unroll
+            for (int a = 0; a < 6; ++a) m3 = max(m3, fx_mag(f.t[a]));
+#pragma unroll
+            for (int a = 0; a < 3; ++a) m4 = max(m4, fx_mag(f.e[a]));
+            push(3, m3);
+            push(4, m4);
+            __syncthreads();
+            EF[0] = fx_exp(mx[3]);
+            EF[1] = fx_exp(mx[4]);
+            if (on && (r > 0 || k == 0)) {
+                Limbs* Fk = F + k * n3 + node;
+#pragma unroll
+                for (int a = 0; a < 6; ++a) Fk[a * n4] = fx_limbs(f.t[a], EF[0]);
+#pragma unroll
+                for (int a = 0; a < 3; ++a) Fk[(6 + a) * n4] = fx_limbs(f.e[a], EF[1]);
+            }
+            __syncthreads();
+            if (tid < 2) mx[3 + tid] = 0;
+            // residual -div F + S, in Q's place
+            const int ER[3] = {EQ[1] + ed - 1022 + sh, EF[0] + ed - 1022 + sh, EF[1] + ed - 1022 + sh};
+            {
+                FxSum a[4];
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    const Limbs* D = b == 0 ? Dx : b == 1 ? Dy : Dz;
+                    const Limbs* L = F + ks * n3 + (b == 0 ? ox : b == 1 ? oy : oz);
+#pragma unroll
+                    for (int p = 0; p < n; ++p) {
+                        const Limbs d = D[p];
+                        const int o = p * (b == 0 ? 1 : b == 1 ? n : n2);
+#pragma unroll
+                        for (int v = 0; v < 3; ++v) a[v].add(d, L[fx3_t(v, b) * n4 + o]);
+                        a[3].add(d, L[(6 + b) * n4 + o]);
+                    }
+                }
+                long long R[5];
+                R[0] = -(R0 >> sh);
+#pragma unroll
+                for (int v = 0; v < 4; ++v) R[v + 1] = -(a[v].value() >> sh);
+                if (P.gravity) R[3] += fx_from(S, ER[1]);
+                if (on) {
+#pragma unroll
+                    for (int v = 0; v < 5; ++v) Q[(v * n + k) * n3 + node] = fx_split(R[v]);
+                }
+            }
+            __syncthreads();
+            {  // time contraction: this thread's time node of the next iterate
+                FxSum a[5];
+#pragma unroll
+                for (int kk = 0; kk < n; ++kk) {
+                    const Limbs d = K[k * n + kk];
+#pragma unroll
+                    for (int v = 0; v < 5; ++v) a[v].add(d, Q[(v * n + kk) * n3 + node]);
+                }
+#pragma unroll
+                for (int v = 0; v < 5; ++v)
+                    q[v] = fma(dt, fx_to(a[v].value(), ER[v == 0 ? 0 : v == 4 ? 2 : 1] + B.KwE - 2102), US[v * n3 + node]);
+            }
+            push_q();
+            __syncthreads();
+#pragma unroll
+            for (int a = 0; a < 3; ++a) EQ[a] = fx_exp(mx[a]);
+            if (on) store_q(k);
+            __syncthreads();
+            if (tid < 3) mx[tid] = 0;
+        }
+
+        // time averages: slots q (5), t (6), e (3)
+        double* A = base;
+        __syncthreads();
+        if (on) {
+            double* Ak = A + k * n3 + node;
+#pragma unroll
+            for (int v = 0; v < 5; ++v) Ak[v * n4] = q[v];
+#pragma unroll
+            for (int a = 0; a < 6; ++a) Ak[(5 + a) * n4] = f.t[a];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) Ak[(11 + a) * n4] = f.e[a];
+        }
+        __syncthreads();
+        if (on)
+            for (int s = k; s < 14; s += n) {
+                double a = 0.0;
+#pragma unroll
+                for (int kk = 0; kk < n; ++kk) a = fma(B.w[kk], A[s * n4 + kk * n3 + node], a);
+                A[s * n4 + node] = a;  // time node 0's place, read by this thread alone
+            }
+        __syncthreads();
+        if (on && active) {
+            for (int v = k; v < 5; v += n) {
+                const double* Fv = A + fx3_slot(5 + v, 0) * n4 + ox;
+                const double* Gv = A + fx3_slot(5 + v, 1) * n4 + oy;
+                const double* Hv = A + fx3_slot(5 + v, 2) * n4 + oz;
+                double sx = 0.0, sy = 0.0, sz = 0.0;
+#pragma unroll
+                for (int p = 0; p < n; ++p) {
+                    sx = fma(B.Vx[p][i], Fv[p], sx);
+                    sy = fma(B.Vx[p][j], Gv[p * n], sy);
+                    sz = fma(B.Vx[p][l], Hv[p * n2], sz);
+                }
+                const double S = P.gravity && v == 3 ? -gg * (A[node] - rhobar) : 0.0;
+                rvol[(size_t)cell * SL + v * n3 + node] = fma(sx, P.inv_h[0], fma(sy, P.inv_h[1], fma(sz, P.inv_h[2], S)));
             }
         }
-        const double zf = dir < 2 ? P.org[2] + (iz + B.xi[a]) * P.h[2] : P.org[2] + (iz + ((f & 1) ? 0 : 1)) * P.h[2];
-        rec[25] = wave_speed3(rec, zf, dir, P);
-        if (active) {
-            double* tr = trace + ((size_t)cell * 6 + f) * kTr3 * n2;
+        // boundary-extrapolated traces of faces E, W (x), N, S (y), T, B (z)
+        auto face_at = [](int dir, int a, int b, int p) {
+            return dir == 0 ? (a * n + b) * n + p : dir == 1 ? (a * n + p) * n + b : (p * n + a) * n + b;
+        };
+        double* tr = trace + (size_t)cell * 6 * kTr3 * n2;
+        if (on)
+            for (int o = tid; o < 60 * n2; o += n4) {
+                const int m = o % n2, c = o / n2 % 10, fc = o / (10 * n2), dir = fc >> 1;
+                const double* phi = (fc & 1) ? B.phi0 : B.phi1;
+                const double* S = A + fx3_slot(c, dir) * n4;
+                double s = 0.0;
 #pragma unroll
-            for (int c = 0; c < kTr3; ++c)
-                if (c < 10 || c == 25 || wallface) tr[c * n2 + m] = rec[c];
-        }
-    }    pdl_trigger();
+                for (int p = 0; p < n; ++p) s = fma(phi[p], S[face_at(dir, m / n, m % n, p)], s);
+                if (c < 5) TQ[(fc * 5 + c) * n2 + m] = s;
+                if (active) tr[(fc * kTr3 + c) * n2 + m] = s;
+            }
+        __syncthreads();
+        // Rusanov speed; grad q-bar on slip walls, which alone read it: along the
+        // normal from the cell's nodes, along the face from the face's own values
+        if (on)
+            for (int o = tid; o < 6 * n2; o += n4) {
+                const int fc = o / n2, m = o - fc * n2, dir = fc >> 1, a = m / n, b = m - a * n;
+                double rec[5];
+#pragma unroll
+                for (int v = 0; v < 5; ++v) rec[v] = TQ[(fc * 5 + v) * n2 + m];
+                const double zf = dir < 2 ? P.org[2] + (iz + B.xi[a]) * P.h[2] : P.org[2] + (iz + ((fc & 1) ? 0 : 1)) * P.h[2];
+                if (active) tr[(fc * kTr3 + 25) * n2 + m] = wave_speed3(rec, zf, dir, P);
+                const int icd = dir == 0 ? ic0 : dir == 1 ? ic1 : iz;
+                const int ncd = dir == 0 ? P.nc[0] : dir == 1 ? P.nc[1] : P.nc[2];
+                const int bcd = dir == 0 ? P.bc[0] : dir == 1 ? P.bc[1] : P.bc[2];
+                if (!(active && bcd == ADG_BC_WALL && ((fc & 1) ? icd == 0 : icd == ncd - 1))) continue;
+                const double* dphi = (fc & 1) ? B.dphi0 : B.dphi1;
+                for (int v = 0; v < 5; ++v) {
+                    const double* T = TQ + (fc * 5 + v) * n2;
+                    double sn = 0.0, sa = 0.0, sb = 0.0;  // normal, along the face's first and second index
+#pragma unroll
+                    for (int p = 0; p < n; ++p) {
+                        sn = fma(dphi[p], A[v * n4 + face_at(dir, a, b, p)], sn);
+                        sa = fma(B.D[a][p], T[p * n + b], sa);
+                        sb = fma(B.D[b][p], T[a * n + p], sb);
+                    }
+                    const double gx = dir == 0 ? sn : sb, gy = dir == 1 ? sn : dir == 0 ? sb : sa, gz3 = dir == 2 ? sn : sa;
+                    double* tw = tr + (fc * kTr3 + 10 + v) * n2 + m;
+                    tw[0] = gx * P.inv_h[0];
+                    tw[5 * n2] = gy * P.inv_h[1];
+                    tw[10 * n2] = gz3 * P.inv_h[2];
+                }
+            }
+    }
+    pdl_trigger();
 }
 
 struct Phys3f {
@@ -990,9 +1140,11 @@ int launch3(bool pred, double* u, double* rvol, double* trace, int cells, double
     using C = Cfg3<N>;
     const int blocks = (cells + C::cpb - 1) / C::cpb;
     if (pred) {
-        cudaError_t e = cudaFuncSetAttribute(k3_predictor<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem);
+        using X = Fx3Cfg<N>;
+        cudaError_t e = cudaFuncSetAttribute(k3_predictor<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)X::smem);
         if (e != cudaSuccess) return (int)e;
-        k3_predictor<N><<<blocks, C::threads, C::smem, s>>>(u, rvol, trace, cells, dt, B, P, bg);
+        k3_predictor<N><<<fx_grid((cells + X::cpb - 1) / X::cpb, X::resident), X::threads, X::smem, s>>>(
+            u, rvol, trace, cells, dt, B, P, bg);
     } else {
         // programmatic launch: scheduled while the predictor drains
         cudaLaunchConfig_t cfg = {};

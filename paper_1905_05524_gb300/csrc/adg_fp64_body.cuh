@@ -36,16 +36,6 @@ struct FxCfg {
     static constexpr size_t smem(bool tsrc) { return ((size_t)cpb * words(tsrc) + n2) * 8; }
 };
 
-// Blocks of a launch that strides over `tiles` tiles: as many rounds as the
-// resident blocks need, the tiles spread evenly over them.
-inline int fx_grid(int tiles, int resident) {
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int rounds = (tiles + sms * resident - 1) / (sms * resident);
-    return (tiles + rounds - 1) / rounds;
-}
-
 // D / hx and D / hy of a cell in fixed point, in shared memory: in registers
 // the two rows of a node (24 at degree 5) leave two resident blocks, and the
 // kernel waits on its own dependent chains (1.55 ms on the 81x81 degree-5 mesh).
