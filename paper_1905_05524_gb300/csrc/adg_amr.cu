@@ -40,6 +40,7 @@
 
 namespace adg {
 
+constexpr int kGeo = 8;      // per leaf: x0, y0, hx, hy, 1/hx, 1/hy, the penalties eta_x, eta_y
 constexpr int kNbrInts = 5;  // type, id0, id1, id2, sub-face
 enum { NB_CONF = 0, NB_COARSE = 1, NB_FINE = 2, NB_WALL = 3 };
 
@@ -145,7 +146,7 @@ static int upload_tables(adg_mesh* m) {
     const int L = (int)T->leaves.size(), n = m->n;
     const adg_mesh_desc* d = &m->d;
     const bool mixed = d->precision == ADG_PREC_MIXED;
-    std::vector<double> geo((size_t)L * 4), bgl((size_t)L * n * 2 + (size_t)L * 4, 0.0);
+    std::vector<double> geo((size_t)L * kGeo), bgl((size_t)L * n * 2 + (size_t)L * 4, 0.0);
     std::vector<int> nbr((size_t)L * 4 * kNbrInts);
     std::vector<double> h64(mixed ? (size_t)L * n * 2 + (size_t)L * 4 : 0, 0.0);
     std::vector<float> h32(mixed ? (size_t)L * n * 3 + (size_t)L * 4 : 0, 0.0f);
@@ -207,10 +208,15 @@ static int upload_tables(adg_mesh* m) {
         const int l = T->leaves[k][0], ix = T->leaves[k][1], iy = T->leaves[k][2];
         const double hx = d->Lx / (d->nx * AmrTree::ipow3(l)), hy = d->Ly / (d->ny * AmrTree::ipow3(l));
         hmin = std::fmin(hmin, std::fmin(hx, hy));
-        geo[k * 4 + 0] = d->x0 + ix * hx;
-        geo[k * 4 + 1] = d->y0 + iy * hy;
-        geo[k * 4 + 2] = hx;
-        geo[k * 4 + 3] = hy;
+        double* g = &geo[(size_t)k * kGeo];
+        g[0] = d->x0 + ix * hx;
+        g[1] = d->y0 + iy * hy;
+        g[2] = hx;
+        g[3] = hy;
+        g[4] = 1.0 / hx;  // divided once here: four divisions a thread cost the corrector more than its faces
+        g[5] = 1.0 / hy;
+        g[6] = (2.0 * m->N + 1.0) / (hx * 1.2533141373155002);  // sqrt(pi/2)
+        g[7] = (2.0 * m->N + 1.0) / (hy * 1.2533141373155002);
         const std::vector<double>& r = row_of(l, iy, hy);
         for (int j = 0; j < n; ++j) {
             bgl[((size_t)k * n + j) * 2] = r[(size_t)j * 2];
@@ -239,7 +245,7 @@ static int upload_tables(adg_mesh* m) {
     // ensure_capacity); the layouts are those of the current L leaves
     const size_t C = (size_t)m->leaf_cap;
     if (!m->geo) {
-        if (cudaMalloc(&m->geo, C * 4 * 8) != cudaSuccess || cudaMalloc(&m->nbr, C * 4 * kNbrInts * 4) != cudaSuccess ||
+        if (cudaMalloc(&m->geo, C * kGeo * 8) != cudaSuccess || cudaMalloc(&m->nbr, C * 4 * kNbrInts * 4) != cudaSuccess ||
             cudaMalloc(&m->bgl, (C * n * 2 + C * 4) * 8) != cudaSuccess) {
             cudaGetLastError();
             return fail(ADG_ENOMEM, "adaptive mesh: tables");
@@ -360,14 +366,16 @@ void amr_free(adg_mesh* m) {
 }
 
 // per-leaf constants: P with the leaf's cell sizes
-__device__ __forceinline__ Phys leaf_phys(const Phys& P0, const double* geo, int cell, int N) {
+__device__ __forceinline__ Phys leaf_phys(const Phys& P0, const double* geo, int cell) {
     Phys P = P0;
-    P.hx = geo[cell * 4 + 2];
-    P.hy = geo[cell * 4 + 3];
-    P.inv_hx = 1.0 / P.hx;
-    P.inv_hy = 1.0 / P.hy;
-    P.eta_x = (2.0 * N + 1.0) / (P.hx * 1.2533141373155002);  // sqrt(pi/2)
-    P.eta_y = (2.0 * N + 1.0) / (P.hy * 1.2533141373155002);
+    const double2* g = reinterpret_cast<const double2*>(geo + (size_t)cell * kGeo + 2);
+    const double2 h = g[0], ih = g[1], eta = g[2];
+    P.hx = h.x;
+    P.hy = h.y;
+    P.inv_hx = ih.x;
+    P.inv_hy = ih.y;
+    P.eta_x = eta.x;
+    P.eta_y = eta.y;
     return P;
 }
 
@@ -392,9 +400,9 @@ k_predictor_amr(const double* __restrict__ u, double* __restrict__ rvol, double*
     for (int c0 = first + blockIdx.x * C::cpb; c0 < end; c0 += gridDim.x * C::cpb) {
         const bool active = c0 + cl < end;
         const int cell = active ? c0 + cl : end - 1;
-        const double4 ge = *reinterpret_cast<const double4*>(geo + (size_t)cell * 4);
+        const double4 ge = *reinterpret_cast<const double4*>(geo + (size_t)cell * kGeo);
         if (ge.z != P.hx || ge.w != P.hy) {
-            P = leaf_phys(P0, geo, cell, N);
+            P = leaf_phys(P0, geo, cell);
             O.make(B, fx_tab<N, false>(sm, cl), tid, P.inv_hx, P.inv_hy);
         }
         unsigned gmask = 0;
@@ -464,7 +472,7 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
     unsigned wf = 0;  // wall faces: grad q-bar is read there only
 #pragma unroll
     for (int f = 0; f < 4; ++f) wf |= nbr[((size_t)cell * 4 + f) * kNbrInts] == NB_WALL ? 1u << f : 0u;
-    const double hx = geo[cell * 4 + 2], hy = geo[cell * 4 + 3], yorg = geo[cell * 4 + 1];
+    const double hx = geo[(size_t)cell * kGeo + 2], hy = geo[(size_t)cell * kGeo + 3], yorg = geo[(size_t)cell * kGeo + 1];
     const float inv_hx = (float)(1.0 / hx), inv_hy = (float)(1.0 / hy);
     const float z = (float)(yorg + (double)B.xi[j] * hy);
     const size_t rowj = (size_t)cell * n + j;
@@ -762,99 +770,79 @@ __device__ __forceinline__ void corrector_amr_body(double* __restrict__ u, const
     const int cell_raw = c0 + cl;
     const bool active = cell_raw < cells;
     const int cell = active ? cell_raw : cells - 1;
-    const Phys P = leaf_phys(P0, geo, cell, N);
-    const double yorg = geo[cell * 4 + 1];
+    const Phys P = leaf_phys(P0, geo, cell);
+    const double yorg = geo[(size_t)cell * kGeo + 1];
 
-    for (int idx = node; idx < 4 * 3 * n; idx += n2) {
-        const int f = idx / (3 * n), rem = idx - f * 3 * n, s = rem / n, m = rem - s * n;
+    // faces without finer neighbours, one thread per face node (a loop over
+    // thirds of all faces, with those of other faces skipped, kept a third of
+    // the lanes of twice the warps busy)
+    bool fine = false;
+    for (int idx = node; idx < 4 * n; idx += n2) {
+        const int f = idx / n, m = idx - f * n;
         const int* nb = nbr + ((size_t)cell * 4 + f) * kNbrInts;
         const int type = nb[0];
-        if (type != NB_FINE && s > 0) continue;
+        if (type == NB_FINE) {
+            fine = true;
+            continue;
+        }
         const bool xface = f < 2;
         const int of = f ^ 1;  // opposite face: E<->W, N<->S
         const bool own_minus = (f == 0 || f == 2);
         const double* own = trace + ((size_t)cell * 4 + f) * TR;
-        double qo[4], fo[4], so;
-        double qn[4], fn[4], sn;
-        if (LTS && type == NB_FINE) {
-            // coarse side under local time stepping: the fine leaves' fluxes, averaged over their sub-steps
-            const double* a = lts->acc + ((((size_t)cell * 4 + f) * 3 + s) * 4) * n;
+        double rec[kTraceComps];
 #pragma unroll
-            for (int v = 0; v < 4; ++v) Fsub[cl][f][s][v][m] = a[v * n + m];
-            continue;
+        for (int c = 0; c < kTraceComps; ++c)
+            if (c < 8 || c == 16 || type == NB_WALL) rec[c] = own[c * n + m];
+        double qo[4], fo[4], qn[4], fn[4], sn;
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            qo[v] = rec[v];
+            fo[v] = rec[4 + v];
         }
-        if (type == NB_FINE) {
-            // coarse side of a hanging face: own trace on third s vs fine neighbour s
-            const int o = nb[1 + s];
-            const Phys Pf = leaf_phys(P0, geo, o, N);
-            // heights of the fine neighbour's face nodes (the same expression it uses itself)
-            const double z = geo[o * 4 + 1] + (xface ? B.xi[m] * Pf.hy : (f == 2 ? 0.0 : Pf.hy));
-            prolong_rec(own, n, O, s, m, qo, fo);
-            so = wave_speed(qo, z, xface, Pf);
-            const double* ot = trace + ((size_t)o * 4 + of) * TR;
+        const double so = rec[16];
+        const double z = xface ? yorg + B.xi[m] * P.hy : yorg + (f == 2 ? P.hy : 0.0);
+        if (type == NB_WALL) {
+            double pb, rb;
+            if (xface) {
+                pb = bgl[((size_t)cell * n + m) * 2];
+                rb = bgl[((size_t)cell * n + m) * 2 + 1];
+            } else {
+                const double* fb = bgl + (size_t)(LTS ? lts->total : cells) * n * 2 + (size_t)cell * 4 + (f == 2 ? 0 : 2);
+                pb = fb[0];
+                rb = fb[1];
+            }
+            const double nx = f == 0 ? 1.0 : f == 1 ? -1.0 : 0.0;
+            const double ny = f == 2 ? 1.0 : f == 3 ? -1.0 : 0.0;
+            const double mn = rec[1] * nx + rec[2] * ny;
+            qn[1] = rec[1] - 2.0 * mn * nx;
+            qn[2] = rec[2] - 2.0 * mn * ny;
+            qn[0] = P.gravity ? rb : rec[0];
+            qn[3] = P.gravity ? pb / P.gm1 + rb * P.g * z : rec[3];
+            Flux4 fl;
+            ns_flux(qn, rec + 8, rec + 12, z, pb, rb, P, fl, true, 0.0, P.gravity ? -P.g / P.cp : 0.0);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) fn[v] = xface ? fl.F[v] : fl.G[v];
+            sn = wave_speed(qn, z, xface, P);
+        } else if (type == NB_CONF) {
+            const double* ot = trace + ((size_t)nb[1] * 4 + of) * TR;
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 qn[v] = ot[v * n + m];
                 fn[v] = ot[(4 + v) * n + m];
             }
             sn = ot[16 * n + m];
-        } else {
-            double rec[kTraceComps];
-#pragma unroll
-            for (int c = 0; c < kTraceComps; ++c)
-                if (c < 8 || c == 16 || type == NB_WALL) rec[c] = own[c * n + m];
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                qo[v] = rec[v];
-                fo[v] = rec[4 + v];
+        } else if (LTS) {  // NB_COARSE under local time stepping: the coarse trace averaged over this step
+            double av[8 * n];
+            for (int c = 0; c < 8 * n; ++c) av[c] = 0.0;
+            for (int k = 0; k < n; ++k) {
+                const double* tk = lts->ttrace + ((((size_t)nb[1] * n + k) * 4 + of) * 16) * n;
+                for (int c = 0; c < 8 * n; ++c) av[c] += lts->W[k] * tk[c];
             }
-            so = rec[16];
-            const double z = xface ? yorg + B.xi[m] * P.hy : yorg + (f == 2 ? P.hy : 0.0);
-            if (type == NB_WALL) {
-                double pb, rb;
-                if (xface) {
-                    pb = bgl[((size_t)cell * n + m) * 2];
-                    rb = bgl[((size_t)cell * n + m) * 2 + 1];
-                } else {
-                    const double* fb = bgl + (size_t)(LTS ? lts->total : cells) * n * 2 + (size_t)cell * 4 +
-                                       (f == 2 ? 0 : 2);
-                    pb = fb[0];
-                    rb = fb[1];
-                }
-                const double nx = f == 0 ? 1.0 : f == 1 ? -1.0 : 0.0;
-                const double ny = f == 2 ? 1.0 : f == 3 ? -1.0 : 0.0;
-                const double mn = rec[1] * nx + rec[2] * ny;
-                qn[1] = rec[1] - 2.0 * mn * nx;
-                qn[2] = rec[2] - 2.0 * mn * ny;
-                qn[0] = P.gravity ? rb : rec[0];
-                qn[3] = P.gravity ? pb / P.gm1 + rb * P.g * z : rec[3];
-                Flux4 fl;
-                ns_flux(qn, rec + 8, rec + 12, z, pb, rb, P, fl, true, 0.0, P.gravity ? -P.g / P.cp : 0.0);
-#pragma unroll
-                for (int v = 0; v < 4; ++v) fn[v] = xface ? fl.F[v] : fl.G[v];
-                sn = wave_speed(qn, z, xface, P);
-            } else if (type == NB_CONF) {
-                const double* ot = trace + ((size_t)nb[1] * 4 + of) * TR;
-#pragma unroll
-                for (int v = 0; v < 4; ++v) {
-                    qn[v] = ot[v * n + m];
-                    fn[v] = ot[(4 + v) * n + m];
-                }
-                sn = ot[16 * n + m];
-            } else if (LTS) {  // NB_COARSE under local time stepping: the coarse trace averaged over this step
-                double rec[8 * n];
-                for (int c = 0; c < 8 * n; ++c) rec[c] = 0.0;
-                for (int k = 0; k < n; ++k) {
-                    const double* tk = lts->ttrace + ((((size_t)nb[1] * n + k) * 4 + of) * 16) * n;
-                    for (int c = 0; c < 8 * n; ++c) rec[c] += lts->W[k] * tk[c];
-                }
-                prolong_rec(rec, n, O, nb[4], m, qn, fn);
-                sn = wave_speed(qn, z, xface, P);
-            } else {  // NB_COARSE: the coarse trace on this cell's third of the face
-                const double* ot = trace + ((size_t)nb[1] * 4 + of) * TR;
-                prolong_rec(ot, n, O, nb[4], m, qn, fn);
-                sn = wave_speed(qn, z, xface, P);
-            }
+            prolong_rec(av, n, O, nb[4], m, qn, fn);
+            sn = wave_speed(qn, z, xface, P);
+        } else {  // NB_COARSE: the coarse trace on this cell's third of the face
+            prolong_rec(trace + ((size_t)nb[1] * 4 + of) * TR, n, O, nb[4], m, qn, fn);
+            sn = wave_speed(qn, z, xface, P);
         }
         double out[4];
         if (own_minus) rusanov(qo, fo, so, qn, fn, sn, out);
@@ -865,26 +853,57 @@ __device__ __forceinline__ void corrector_amr_body(double* __restrict__ u, const
             for (int v = 0; v < 4; ++v) a[v * n + m] += out[v] * (1.0 / 3.0);
         }
 #pragma unroll
-        for (int v = 0; v < 4; ++v) Fsub[cl][f][s][v][m] = out[v];
+        for (int v = 0; v < 4; ++v) Fst[cl][f][v][m] = out[v];
     }
-    __syncthreads();
-    for (int idx = node; idx < 4 * n; idx += n2) {
-        const int f = idx / n, q = idx - f * n;
-        const bool fine = nbr[((size_t)cell * 4 + f) * kNbrInts] == NB_FINE;
+    // coarse side of hanging faces: the own trace on third s against fine
+    // neighbour s, then the restriction of the three fluxes
+    if (__syncthreads_or(fine)) {
+        for (int idx = node; idx < 4 * 3 * n; idx += n2) {
+            const int f = idx / (3 * n), rem = idx - f * 3 * n, s = rem / n, m = rem - s * n;
+            const int* nb = nbr + ((size_t)cell * 4 + f) * kNbrInts;
+            if (nb[0] != NB_FINE) continue;
+            double out[4];
+            if (LTS) {
+                // under local time stepping: the fine leaves' fluxes, averaged over their sub-steps
+                const double* a = lts->acc + ((((size_t)cell * 4 + f) * 3 + s) * 4) * n;
 #pragma unroll
-        for (int v = 0; v < 4; ++v) {
-            double a;
-            if (fine) {
-                a = 0.0;
+                for (int v = 0; v < 4; ++v) out[v] = a[v * n + m];
+            } else {
+                const bool xface = f < 2;
+                const int o = nb[1 + s];
+                const Phys Pf = leaf_phys(P0, geo, o);
+                // heights of the fine neighbour's face nodes (the same expression it uses itself)
+                const double z = geo[(size_t)o * kGeo + 1] + (xface ? B.xi[m] * Pf.hy : (f == 2 ? 0.0 : Pf.hy));
+                double qo[4], fo[4], qn[4], fn[4];
+                prolong_rec(trace + ((size_t)cell * 4 + f) * TR, n, O, s, m, qo, fo);
+                const double so = wave_speed(qo, z, xface, Pf);
+                const double* ot = trace + ((size_t)o * 4 + (f ^ 1)) * TR;
+#pragma unroll
+                for (int v = 0; v < 4; ++v) {
+                    qn[v] = ot[v * n + m];
+                    fn[v] = ot[(4 + v) * n + m];
+                }
+                const double sn = ot[16 * n + m];
+                if (f == 0 || f == 2) rusanov(qo, fo, so, qn, fn, sn, out);
+                else rusanov(qn, fn, sn, qo, fo, so, out);
+            }
+#pragma unroll
+            for (int v = 0; v < 4; ++v) Fsub[cl][f][s][v][m] = out[v];
+        }
+        __syncthreads();
+        for (int idx = node; idx < 4 * n; idx += n2) {
+            const int f = idx / n, q = idx - f * n;
+            if (nbr[((size_t)cell * 4 + f) * kNbrInts] != NB_FINE) continue;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                double a = 0.0;
                 for (int s = 0; s < 3; ++s)
                     for (int mm = 0; mm < n; ++mm) a += O.Rw[s][mm][q] * Fsub[cl][f][s][v][mm];
-            } else {
-                a = Fsub[cl][f][0][v][q];
+                Fst[cl][f][v][q] = a;
             }
-            Fst[cl][f][v][q] = a;
         }
+        __syncthreads();
     }
-    __syncthreads();
     if (!active) return;
     double* uc = u + (size_t)cell * SL;
     const double* rc = rvol + (size_t)cell * SL;
@@ -927,12 +946,12 @@ k_tv_cells_amr(const double* __restrict__ u, double* __restrict__ tv, double* __
     const int cell_raw = blockIdx.x * CPB + cl;
     const bool active = cell_raw < cells;
     const int cell = active ? cell_raw : cells - 1;
-    const Phys P = leaf_phys(P0, geo, cell, N);
+    const Phys P = leaf_phys(P0, geo, cell);
     const double* uc = u + (size_t)cell * SL;
     double q[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) q[v] = uc[v * n2 + node];
-    const double z = geo[cell * 4 + 1] + B.xi[j] * P.hy;
+    const double z = geo[(size_t)cell * kGeo + 1] + B.xi[j] * P.hy;
     const double f = var == ADG_TV_THETA ? theta_of(q, z, P) : q[0];
     const double r = tv_cell<N, double>(f, 0.0, node, i, j, B, P.inv_hx, P.inv_hy, fs[cl], red[cl], active,
                                         tv + cell);
@@ -947,8 +966,8 @@ __global__ void k_init_amr(double* __restrict__ u, int cells, int kind, double A
     if (gid >= cells * n2) return;
     const int cell = gid / n2, node = gid - cell * n2;
     const int j = node / n, i = node - j * n;
-    const double x = geo[cell * 4] + B.xi[i] * geo[cell * 4 + 2];
-    const double z = geo[cell * 4 + 1] + B.xi[j] * geo[cell * 4 + 3];
+    const double x = geo[(size_t)cell * kGeo] + B.xi[i] * geo[(size_t)cell * kGeo + 2];
+    const double z = geo[(size_t)cell * kGeo + 1] + B.xi[j] * geo[(size_t)cell * kGeo + 3];
     double q[4];
     if (kind == ADG_SCEN_STEADY) {
         const double k = 2.0 * 3.14159265358979323846 / P.sL;
@@ -992,7 +1011,7 @@ __global__ void k_max_speed_amr(const double* __restrict__ u, double* __restrict
     if (gid < cells * n2) {
         const int cell = gid / n2, node = gid - cell * n2;
         const int j = node / n;
-        const double z = geo[cell * 4 + 1] + B.xi[j] * geo[cell * 4 + 3];
+        const double z = geo[(size_t)cell * kGeo + 1] + B.xi[j] * geo[(size_t)cell * kGeo + 3];
         const double* uc = u + (size_t)cell * SL;
         const double rho = uc[node], mx = uc[n2 + node], my = uc[2 * n2 + node], E = uc[3 * n2 + node];
         const double p = P.gm1 * (E - 0.5 * (mx * mx + my * my) / rho - rho * (P.gravity ? P.g * z : 0.0));

@@ -36,7 +36,7 @@ struct adg_mesh {
     // adaptive 3:1 tree (desc.max_levels > 0); cells = number of leaves
     int amr = 0;
     void* tree = nullptr;         // host tree (adg_amr.cu)
-    double* geo = nullptr;        // [leaves][4]: x0, y0, hx, hy of each leaf
+    double* geo = nullptr;        // [leaves][8]: x0, y0, hx, hy, 1/hx, 1/hy, eta_x, eta_y of each leaf
     int* nbr = nullptr;           // [leaves][4 faces][5]: type, id0, id1, id2, sub-face
     double* bgl = nullptr;        // [leaves][n][2] node background, then [leaves][2][2] N/S faces
     double* mbl64 = nullptr;      // mixed precision: per-leaf FP64 background (adg_amr.cu upload_tables)
