@@ -48,6 +48,15 @@ __device__ __forceinline__ double f32_to_f64(float f) {
 // this block no longer needs to delay the dependent kernel.  Both are no-ops
 // for kernels launched without the attribute.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The pointer to what the previous kernel wrote, to be read after pdl_wait():
+// loads through a const __restrict__ parameter may be moved ahead of the wait
+// (they count as reads of memory that nobody writes), loads through the
+// returned pointer cannot, since it exists from here on only.
+template <typename T>
+__device__ __forceinline__ T* pdl_fresh(T* p) {
+    asm volatile("" : "+l"(p) : : "memory");
+    return p;
+}
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 }  // namespace adg

@@ -50,11 +50,10 @@ k_predictor_mixed_x2(const double* __restrict__ u, float* __restrict__ rvol, flo
 
 template <int N, int CPB, bool TV>
 __global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
-k_corrector_mixed(double* __restrict__ u, const float* __restrict__ rvol,
-                  const float* __restrict__ trace, int cells, double dt, const BasisF B,
+k_corrector_mixed(double* __restrict__ u, const float* rvol, const float* trace, int cells, double dt, const BasisF B,
                   const PhysF P, const MixedBg bg, const TvEpilogue epi) {
     pdl_wait();  // the predictor's residual and traces are complete and visible
-    corrector_mixed_body<N, CPB, TV>(u, rvol, trace, cells, blockIdx.x * CPB, dt, B, P, bg, epi);
+    corrector_mixed_body<N, CPB, TV>(u, pdl_fresh(rvol), pdl_fresh(trace), cells, blockIdx.x * CPB, dt, B, P, bg, epi);
     pdl_trigger();
 }
 

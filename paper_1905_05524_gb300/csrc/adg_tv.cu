@@ -138,7 +138,7 @@ __device__ __forceinline__ void chan_combine(double& m, double& m2, double mb, d
 constexpr int kFoldMax = 8;  // folds up to this length load all their triples in one batch
 
 __global__ void __launch_bounds__(kTvThreads)
-k_tv_stats_flags(const double* __restrict__ tv, const TvStatsArgs st, double T_r, double T_c,
+k_tv_stats_flags(const double* tv_in, TvStatsArgs st, double T_r, double T_c,
                  double* __restrict__ stats, int8_t* __restrict__ flags) {
     __shared__ double wm[kTvThreads / 32], w2[kTvThreads / 32];
     __shared__ TvThresholds thr;
@@ -163,6 +163,8 @@ k_tv_stats_flags(const double* __restrict__ tv, const TvStatsArgs st, double T_r
     // the block triples and the TV values come from the kernel before this
     // one (programmatic launch)
     pdl_wait();
+    const double* tv = pdl_fresh(tv_in);
+    st.part = pdl_fresh(st.part);
     const int c_first = blockIdx.x * kTvThreads + t;
     const double tv_first = (flags && c_first < st.cells) ? tv[c_first] : 0.0;
     // left fold of this thread's block triples
