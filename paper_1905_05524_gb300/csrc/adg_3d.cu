@@ -14,13 +14,15 @@
 // Eq. 10, or the analytic ABC field) and the FP64 update u += dt (rvol - lift).
 //
 // Thread mapping: the FP64 predictor runs one thread per space-time node (see
-// k3_predictor); the mixed predictor and the corrector CPB cells per block, one
-// thread per spatial node (l, j, i).  A thread of the mixed predictor walks the
-// n time nodes of its node, so the Picard update's time contraction stays in
+// there); the mixed predictor and the corrector CPB cells per block, one thread
+// per spatial node (l, j, i).  A thread of the mixed predictor walks the n time
+// nodes of its node, so the Picard update's time contraction stays in
 // registers; its shared memory holds per cell the n time slices of the iterate
-// and the F, G, H of one time slice (the divergence of slice k is taken before
-// slice k+1's fluxes overwrite them), after the last sweep the seven
-// time-averaged fields the volume term and the traces contract.
+// and the fluxes of one time slice (the divergence of slice k is taken before
+// slice k+1's fluxes overwrite them), after the last sweep the averaged fields
+// the volume term and the traces contract.  (One thread per space-time node,
+// scalar or with two slices packed, was measured for it too: 201 and 240 us
+// a step of the 25^3 degree-2 bubble against 200 before the nine-flux form.)
 //
 // Layouts: u[c][v][l][j][i], c = (iz ny + iy) nx + ix, v in (rho, rho u,
 // rho v, rho w, rho E); traces [c][face E W N S T B][kTr3][n^2], face nodes
@@ -37,6 +39,7 @@
 #include "adg_fixed.cuh"
 #include "adg_internal.h"
 #include "adg_mesh.h"
+#include "adg_mixed_point.cuh"
 
 namespace adg {
 namespace {
@@ -109,7 +112,7 @@ __device__ __forceinline__ void ns_flux3(const double q[5], const double g[3][5]
 
 // Rusanov speed |v_dir| + c + 2 eta_dir lambda_v / rho at height z
 __device__ __forceinline__ double wave_speed3(const double q[5], double z, int dir, const Phys3& P) {
-    const double rinv = 1.0 / q[0];
+    const double rinv = fx_rcp(q[0]);
     const double gg = P.gravity ? P.g : 0.0;
     const double p = P.gm1 * (q[4] - 0.5 * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) * rinv - q[0] * gg * z);
     const double mn = dir == 0 ? q[1] : dir == 1 ? q[2] : q[3];  // selects keep q in registers
@@ -157,8 +160,6 @@ struct Cfg3 {
     static constexpr int n = N + 1, n2 = n * n, n3 = n * n * n;
     static constexpr int cpb = N == 1 ? 16 : N == 2 ? 8 : N == 3 ? 4 : 2;
     static constexpr int threads = cpb * n3;
-    static constexpr int slots = (n + 3) > 7 ? n + 3 : 7;  // iterate + one slice of fluxes, or 7 averages
-    static constexpr size_t smem = (size_t)cpb * slots * 5 * n3 * sizeof(double);
 };
 
 // FP64 predictor: the scheme of the 2D one (adg_fp64_body.cuh) -- one thread
@@ -288,7 +289,7 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
         double q[5];
 #pragma unroll
         for (int v = 0; v < 5; ++v) q[v] = u[(size_t)cell * SL + v * n3 + node];
-        int EQ[3], EF[2];
+        int EQ[3] = {0, 0, 0}, EF[2];
         auto push_q = [&]() {
             push(0, fx_mag(q[0]));
             push(1, max(max(fx_mag(q[1]), fx_mag(q[2])), fx_mag(q[3])));
@@ -580,9 +581,10 @@ __device__ __forceinline__ void ns_flux3f(const float q[5], const float g[3][5],
 // face states converted to FP32, flux average and lifting in FP32, the
 // update in FP64 (ghost states stay FP64).
 template <int N, bool MX>
-__global__ void __launch_bounds__(Cfg3<N>::threads)
-k3_corrector(double* __restrict__ u, const double* __restrict__ rvol, const double* __restrict__ trace, int cells,
-             double dt, double t, const Basis B, const Phys3 P, const Bg3 bg, const Phys3f Pf) {
+// blocks per SM: 25^3 degree 2 mixed 157.9 / 154.9 / 153.9 / 156.8 us a step with 2 / 3 / 4 / 5
+__global__ void __launch_bounds__(Cfg3<N>::threads, (MX && N <= 2 ? 4 : 2))
+k3_corrector(double* __restrict__ u, const double* rvol_in, const double* trace_in, int cells, double dt, double t,
+              const Basis B, const Phys3 P, const Bg3 bg, const Phys3f Pf) {
     using C = Cfg3<N>;
     using FT = typename std::conditional<MX, float, double>::type;
     constexpr int n = C::n, n2 = C::n2, n3 = C::n3, SL = 5 * n3, TR = kTr3 * n2;
@@ -595,6 +597,7 @@ k3_corrector(double* __restrict__ u, const double* __restrict__ rvol, const doub
     const int cell = active ? cell_raw : cells - 1;
     const int ic0 = cell % P.nc[0], ic1 = (cell / P.nc[0]) % P.nc[1], ic2 = cell / (P.nc[0] * P.nc[1]);
     pdl_wait();  // programmatic launch: the predictor's residual and traces are complete and visible
+    const double *rvol = pdl_fresh(rvol_in), *trace = pdl_fresh(trace_in);
 
     for (int idx = node; idx < 6 * n2; idx += n3) {
         const int f = idx / n2, m = idx - f * n2;
@@ -785,13 +788,53 @@ k3_corrector(double* __restrict__ u, const double* __restrict__ rvol, const doub
 // the FP64 corrector runs unchanged.
 template <int N>
 struct Cfg3m {
-    static constexpr size_t smem = (size_t)Cfg3<N>::cpb * Cfg3<N>::slots * 5 * Cfg3<N>::n3 * sizeof(float);
-    // resident blocks asked of the register allocator: measured on the 25^3
-    // bubble, degree 2 runs 12% faster at 4 blocks (72 registers, some
-    // spills) than at the unconstrained 111 registers; degree 3 gains 1% at
-    // 3 and loses at 4; degree 1 is indifferent
-    static constexpr int minb = N == 2 ? 4 : N == 3 ? 3 : 1;
+    // per cell, in fields of n^3 floats: the n time slices of q' (5 each) and the
+    // nine fluxes of one slice, or the 29 averages (q', fluxes, grad q)
+    static constexpr int fields = 5 * (N + 1) + 9 > 29 ? 5 * (N + 1) + 9 : 29;
+    static constexpr size_t smem = (size_t)Cfg3<N>::cpb * fields * Cfg3<N>::n3 * sizeof(float);
+    // resident blocks asked of the register allocator (us a step): degree 2 on
+    // 25^3 cells 159 with 1, 3 or 4 and 177 with 5, degree 3 on 17^3 144 / 122 /
+    // 123 / 155 with 1 / 2 / 3 / 5, degree 4 on 13^3 209 / 187 / 187 / 286
+    static constexpr int minb = N == 2 ? 4 : N == 3 ? 3 : N == 4 ? 2 : 1;
 };
+
+// Fluxes on perturbations: the FP32 form of ns_flux9.
+struct Fx3FluxF {
+    float t[6], e[3];
+};
+__device__ __forceinline__ Fx3FluxF ns_flux9_pert(const float q[5], const float g[3][5], float gz, float rb, float Eb,
+                                                  float Hb, const Phys3f& P) {
+    const float rho = rb + q[0];
+    const float rinv = rcp_fast(rho);
+    const float v[3] = {q[1] * rinv, q[2] * rinv, q[3] * rinv};
+    const float ke2 = fmaf(q[3], v[2], fmaf(q[2], v[1], q[1] * v[0]));
+    const float pp = P.gm1 * fmaf(-0.5f, ke2, fmaf(-gz, q[0], q[4]));
+    const float H = Hb + (q[4] + pp), eR = (Eb + q[4]) * rinv;
+    float w[3][3];  // w[a][b], rho times the velocity gradient
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int b = 0; b < 3; ++b) w[a][b] = fmaf(-v[a], g[b][0], g[b][1 + a]);
+    const float m23 = (2.0f / 3.0f) * P.mu * rinv, mr = -P.mu * rinv, kr = P.gm1 * P.kappa * P.invR * rinv;
+    const float div = w[0][0] + w[1][1] + w[2][2];
+    const float sd[3] = {m23 * fmaf(-3.0f, w[0][0], div), m23 * fmaf(-3.0f, w[1][1], div), m23 * fmaf(-3.0f, w[2][2], div)};
+    const float sxy = mr * (w[0][1] + w[1][0]), sxz = mr * (w[0][2] + w[2][0]), syz = mr * (w[1][2] + w[2][1]);
+    Fx3FluxF f;
+    f.t[0] = fmaf(q[1], v[0], pp + sd[0]);
+    f.t[1] = fmaf(q[1], v[1], sxy);
+    f.t[2] = fmaf(q[1], v[2], sxz);
+    f.t[3] = fmaf(q[2], v[1], pp + sd[1]);
+    f.t[4] = fmaf(q[2], v[2], syz);
+    f.t[5] = fmaf(q[3], v[2], pp + sd[2]);
+    const float so[3][2] = {{sxy, sxz}, {sxy, syz}, {sxz, syz}};
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        float h = fmaf(-v[2], w[2][b], fmaf(-v[1], w[1][b], fmaf(-v[0], w[0][b], fmaf(-eR, g[b][0], g[b][4]))));
+        if (b == 2) h = fmaf(-P.g, rho, h);
+        f.e[b] = fmaf(-kr, h, fmaf(v[b], H + sd[b], fmaf(v[b == 0 ? 1 : 0], so[b][0], v[b == 2 ? 1 : 2] * so[b][1])));
+    }
+    return f;
+}
 
 template <int N>
 __global__ void __launch_bounds__(Cfg3<N>::threads, Cfg3m<N>::minb)
@@ -807,10 +850,11 @@ k3_predictor_mixed(const double* __restrict__ u, double* __restrict__ rvol, doub
     const bool active = cell_raw < cells;
     const int cell = active ? cell_raw : cells - 1;
     const int iz = cell / (P64.nc[0] * P64.nc[1]);
-    float* Q = smf + (size_t)cl * C::slots * SL;
-    float* Fs = Q + n * SL;
+    float* Q = smf + (size_t)cl * Cfg3m<N>::fields * n3;
+    float* Fs = Q + n * SL;  // six momentum, three energy fluxes
     const int nb = iz * n + l;
-    const float rb = bg.rbf[nb], pb = bg.pbf[nb], Hb = bg.Hbf[nb], dzr = bg.dzr[nb], dzE = bg.dzE[nb];
+    const float rb = bg.rbf[nb], Hb = bg.Hbf[nb], dzr = bg.dzr[nb], dzE = bg.dzE[nb];
+    const float Eb = f64_to_f32(bg.Eb[nb]);
     const float gz = (float)(P64.g * bg.zn[nb]);
 
     float uu[5];
@@ -826,68 +870,71 @@ k3_predictor_mixed(const double* __restrict__ u, double* __restrict__ rvol, doub
     for (int v = 0; v < 5; ++v) Q[v * n3 + node] = uu[v];
     __syncthreads();
 
-    auto eval = [&](const float* Qk, float q[5], float g[3][5], float f[3][5], float& src) {
+    // this node's rows of D, scaled by 1/h
+    float dI[3][n];
+#pragma unroll
+    for (int p = 0; p < n; ++p) {
+        dI[0][p] = B.D[i][p] * P.inv_h[0];
+        dI[1][p] = B.D[j][p] * P.inv_h[1];
+        dI[2][p] = B.D[l][p] * P.inv_h[2];
+    }
+    auto line = [&](const float* S, int b) {
+        const int o = b == 0 ? (l * n + j) * n : b == 1 ? l * n2 + i : j * n + i, st = b == 0 ? 1 : b == 1 ? n : n2;
+        float s = dI[b][0] * S[o];
+#pragma unroll
+        for (int p = 1; p < n; ++p) s = fmaf(dI[b][p], S[o + p * st], s);
+        return s;
+    };
+    // state, gradients and fluxes of time slice Qk; md: divergence of the mass flux, minus the source of the
+    // z-momentum
+    auto eval = [&](const float* Qk, float q[5], float g[3][5], Fx3FluxF& f, float& md) {
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
-            const float* Qv = Qk + v * n3;
-            q[v] = Qv[node];
-            float sx = 0.0f, sy = 0.0f, sz = 0.0f;
+            q[v] = Qk[v * n3 + node];
 #pragma unroll
-            for (int p = 0; p < n; ++p) {
-                sx = fmaf(B.D[i][p], Qv[(l * n + j) * n + p], sx);
-                sy = fmaf(B.D[j][p], Qv[(l * n + p) * n + i], sy);
-                sz = fmaf(B.D[l][p], Qv[(p * n + j) * n + i], sz);
-            }
-            g[0][v] = sx * P.inv_h[0];
-            g[1][v] = sy * P.inv_h[1];
-            g[2][v] = sz * P.inv_h[2];
+            for (int b = 0; b < 3; ++b) g[b][v] = line(Qk + v * n3, b);
         }
+        md = g[0][1] + g[1][2] + g[2][3];
         g[2][0] += dzr;
         g[2][4] += dzE;
-        ns_flux3f(q, g, gz, rb, pb, Hb, P, f, src);
+        f = ns_flux9_pert(q, g, gz, rb, Eb, Hb, P);
     };
-    auto store = [&](const float f[3][5]) {
+    auto store = [&](const Fx3FluxF& f) {
 #pragma unroll
-        for (int b = 0; b < 3; ++b)
+        for (int a = 0; a < 6; ++a) Fs[a * n3 + node] = f.t[a];
 #pragma unroll
-            for (int v = 0; v < 5; ++v) Fs[(b * 5 + v) * n3 + node] = f[b][v];
+        for (int a = 0; a < 3; ++a) Fs[(6 + a) * n3 + node] = f.e[a];
     };
-    auto divergence = [&](int v) {
-        const float* Fv = Fs + v * n3;
-        const float* Gv = Fs + (5 + v) * n3;
-        const float* Hv = Fs + (10 + v) * n3;
-        float sx = 0.0f, sy = 0.0f, sz = 0.0f;
-#pragma unroll
-        for (int p = 0; p < n; ++p) {
-            sx = fmaf(B.D[i][p], Fv[(l * n + j) * n + p], sx);
-            sy = fmaf(B.D[j][p], Gv[(l * n + p) * n + i], sy);
-            sz = fmaf(B.D[l][p], Hv[(p * n + j) * n + i], sz);
-        }
-        return -(sx * P.inv_h[0] + sy * P.inv_h[1] + sz * P.inv_h[2]);
+    // residual of variable v at this node from the slice in Fs (v = 0: from md)
+    auto residual = [&](int v, float md, const float q[5]) {
+        if (v == 0) return -md;
+        float s;
+        if (v < 4) s = line(Fs + fx3_t(v - 1, 0) * n3, 0) + line(Fs + fx3_t(v - 1, 1) * n3, 1) + line(Fs + fx3_t(v - 1, 2) * n3, 2);
+        else s = line(Fs + 6 * n3, 0) + line(Fs + 7 * n3, 1) + line(Fs + 8 * n3, 2);
+        return v == 3 && P.gravity ? fmaf(-P.g, q[0], -s) : -s;
     };
 
     {
-        float q[5], g[3][5], f[3][5], src;
-        eval(Q, q, g, f, src);
+        float q[5], g[3][5], md;
+        Fx3FluxF f;
+        eval(Q, q, g, f, md);
         store(f);
         __syncthreads();
         float R0[5];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) R0[v] = (v == 3 ? src : 0.0f) + divergence(v);
+        for (int v = 0; v < 5; ++v) R0[v] = residual(v, md, q);
 #pragma unroll
         for (int k = 0; k < n; ++k)
 #pragma unroll
             for (int v = 0; v < 5; ++v) Q[k * SL + v * n3 + node] = uu[v] + dt * (B.Kw1[k] * R0[v]);
         __syncthreads();
     }
-    // Sweeps 2..n.  Degrees <= 2 walk the time slices with a rolled loop
-    // and accumulate the time contraction slice by slice (the same order as
-    // a row-by-row sum; no register array indexed at run time): one inlined
-    // flux evaluation instead of n.  Measured on the 25^3 bubble: degree 2
-    // runs 4% faster this way (the unrolled kernel stalled on instruction
-    // fetch), degrees 3 and 4 3% and 16% slower, so they keep the unrolled
-    // form with the residuals of all slices in registers.
-    constexpr int kSliceUnroll = N <= 2 ? 1 : n;
+    // Sweeps 2..n.  Degrees <= 2 accumulate the time contraction slice by
+    // slice (the same order as a row-by-row sum), degree 1 with a rolled loop
+    // (142.0 against 145.5 us a step on 41^3 cells unrolled; degree 2 159.3
+    // rolled, 157.0 unrolled on 25^3); degrees 3 and 4 keep the residuals of all
+    // slices in registers.
+    constexpr int kSliceUnroll = N == 1 ? 1 : n;
 #pragma unroll 1
     for (int r = 1; r < n; ++r) {
         if constexpr (N <= 2) {
@@ -896,16 +943,17 @@ k3_predictor_mixed(const double* __restrict__ u, double* __restrict__ rvol, doub
             for (int k = 0; k < n; ++k)
 #pragma unroll
                 for (int v = 0; v < 5; ++v) acc[k][v] = 0.0f;
-#pragma unroll 1
+#pragma unroll kSliceUnroll
             for (int m = 0; m < n; ++m) {
-                float q[5], g[3][5], f[3][5], src;
-                eval(Q + m * SL, q, g, f, src);
+                float q[5], g[3][5], md;
+                Fx3FluxF f;
+                eval(Q + m * SL, q, g, f, md);
                 __syncthreads();
                 store(f);
                 __syncthreads();
 #pragma unroll
                 for (int v = 0; v < 5; ++v) {
-                    const float Rm = (v == 3 ? src : 0.0f) + divergence(v);
+                    const float Rm = residual(v, md, q);
 #pragma unroll
                     for (int k = 0; k < n; ++k) acc[k][v] = fmaf(B.Kw[k][m], Rm, acc[k][v]);
                 }
@@ -918,13 +966,14 @@ k3_predictor_mixed(const double* __restrict__ u, double* __restrict__ rvol, doub
             float R[n][5];
 #pragma unroll
             for (int k = 0; k < n; ++k) {
-                float q[5], g[3][5], f[3][5], src;
-                eval(Q + k * SL, q, g, f, src);
+                float q[5], g[3][5], md;
+                Fx3FluxF f;
+                eval(Q + k * SL, q, g, f, md);
                 __syncthreads();
                 store(f);
                 __syncthreads();
 #pragma unroll
-                for (int v = 0; v < 5; ++v) R[k][v] = (v == 3 ? src : 0.0f) + divergence(v);
+                for (int v = 0; v < 5; ++v) R[k][v] = residual(v, md, q);
             }
 #pragma unroll
             for (int k = 0; k < n; ++k)
@@ -939,48 +988,65 @@ k3_predictor_mixed(const double* __restrict__ u, double* __restrict__ rvol, doub
         __syncthreads();
     }
 
-    float qb[5], fb[3][5], gb[3][5], sb = 0.0f;
+    const int ic0 = cell % P64.nc[0], ic1 = (cell / P64.nc[0]) % P64.nc[1];
+    unsigned wf = 0;  // slip-wall faces, which alone read grad q-bar
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int ic = d == 0 ? ic0 : d == 1 ? ic1 : iz;
+        if (P64.bc[d] == ADG_BC_WALL) wf |= (ic == P64.nc[d] - 1 ? 1u << (2 * d) : 0u) | (ic == 0 ? 2u << (2 * d) : 0u);
+    }
+    float qb[5], tb[6], eb[3], gb[3][5];
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
         qb[v] = 0.0f;
 #pragma unroll
-        for (int b = 0; b < 3; ++b) fb[b][v] = gb[b][v] = 0.0f;
+        for (int b = 0; b < 3; ++b) gb[b][v] = 0.0f;
     }
+#pragma unroll
+    for (int a = 0; a < 6; ++a) tb[a] = 0.0f;
+    eb[0] = eb[1] = eb[2] = 0.0f;
 #pragma unroll kSliceUnroll
     for (int k = 0; k < n; ++k) {
-        float q[5], g[3][5], f[3][5], src;
-        eval(Q + k * SL, q, g, f, src);
+        float q[5], g[3][5], md;
+        Fx3FluxF f;
+        eval(Q + k * SL, q, g, f, md);
         const float wk = B.w[k];
-        sb = fmaf(wk, src, sb);
 #pragma unroll
-        for (int v = 0; v < 5; ++v) {
-            qb[v] = fmaf(wk, q[v], qb[v]);
+        for (int v = 0; v < 5; ++v) qb[v] = fmaf(wk, q[v], qb[v]);
 #pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                fb[b][v] = fmaf(wk, f[b][v], fb[b][v]);
-                gb[b][v] = fmaf(wk, g[b][v], gb[b][v]);
-            }
+        for (int a = 0; a < 6; ++a) tb[a] = fmaf(wk, f.t[a], tb[a]);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) eb[a] = fmaf(wk, f.e[a], eb[a]);
+        if (wf) {
+#pragma unroll
+            for (int v = 0; v < 5; ++v)
+#pragma unroll
+                for (int b = 0; b < 3; ++b) gb[b][v] = fmaf(wk, g[b][v], gb[b][v]);
         }
     }
     __syncthreads();
+    // fields: q' (5), momentum fluxes (6), energy fluxes (3), grad q (15)
     float* A = Q;
 #pragma unroll
-    for (int v = 0; v < 5; ++v) {
-        A[v * n3 + node] = qb[v];
+    for (int v = 0; v < 5; ++v) A[v * n3 + node] = qb[v];
 #pragma unroll
-        for (int b = 0; b < 3; ++b) {
-            A[(1 + b) * SL + v * n3 + node] = fb[b][v];
-            A[(4 + b) * SL + v * n3 + node] = gb[b][v];
-        }
+    for (int a = 0; a < 6; ++a) A[(5 + a) * n3 + node] = tb[a];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) A[(11 + a) * n3 + node] = eb[a];
+    if (wf) {
+#pragma unroll
+        for (int b = 0; b < 3; ++b)
+#pragma unroll
+            for (int v = 0; v < 5; ++v) A[(14 + 5 * b + v) * n3 + node] = gb[b][v];
     }
     __syncthreads();
     if (active) {
         double* rc = rvol + (size_t)cell * SL;
 #pragma unroll
         for (int v = 0; v < 5; ++v) {
-            const float* Fv = A + 1 * SL + v * n3;
-            const float* Gv = A + 2 * SL + v * n3;
-            const float* Hv = A + 3 * SL + v * n3;
+            const float* Fv = A + fx3_slot(5 + v, 0) * n3;
+            const float* Gv = A + fx3_slot(5 + v, 1) * n3;
+            const float* Hv = A + fx3_slot(5 + v, 2) * n3;
             float sx = 0.0f, sy = 0.0f, sz = 0.0f;
 #pragma unroll
             for (int p = 0; p < n; ++p) {
@@ -988,41 +1054,37 @@ k3_predictor_mixed(const double* __restrict__ u, double* __restrict__ rvol, doub
                 sy = fmaf(B.Vx[p][j], Gv[(l * n + p) * n + i], sy);
                 sz = fmaf(B.Vx[p][l], Hv[(p * n + j) * n + i], sz);
             }
-            rc[v * n3 + node] = f32_to_f64(sx * P.inv_h[0] + sy * P.inv_h[1] + sz * P.inv_h[2] + (v == 3 ? sb : 0.0f));
+            rc[v * n3 + node] = f32_to_f64(sx * P.inv_h[0] + sy * P.inv_h[1] + sz * P.inv_h[2] + (v == 3 && P.gravity ? -P.g * qb[0] : 0.0f));
         }
     }
-    const int ic0 = cell % P64.nc[0], ic1 = (cell / P64.nc[0]) % P64.nc[1];
     for (int idx = node; idx < 6 * n2; idx += n3) {
         const int f = idx / n2, m = idx - f * n2;
         const int a = m / n, b = m - a * n;
         const int dir = f >> 1;
-        const float* phi = (f & 1) ? B.phi0 : B.phi1;
-        // the gradient components are read only by slip-wall ghosts: written
-        // for wall faces alone
-        const int icd = dir == 0 ? ic0 : dir == 1 ? ic1 : iz;
-        const int ncd = dir == 0 ? P64.nc[0] : dir == 1 ? P64.nc[1] : P64.nc[2];
-        const int bcd = dir == 0 ? P64.bc[0] : dir == 1 ? P64.bc[1] : P64.bc[2];
-        const bool wallface = bcd == ADG_BC_WALL && ((f & 1) ? icd == 0 : icd == ncd - 1);
-        double rec[kTr3];
+        const bool wallface = wf >> f & 1u;
+        const int at = dir == 0 ? (a * n + b) * n : dir == 1 ? a * n2 + b : a * n + b;
+        const int st = dir == 0 ? 1 : dir == 1 ? n : n2;
+        float phi[n];
 #pragma unroll
-        for (int c = 0; c < 5; ++c) {
-            if (c >= 2 && !wallface) {
+        for (int p = 0; p < n; ++p) phi[p] = (f & 1) ? B.phi0[p] : B.phi1[p];
+        auto ext = [&](const float* S) {
+            float s = 0.0f;
 #pragma unroll
-                for (int v = 0; v < 5; ++v) rec[c * 5 + v] = 0.0;
-                continue;
-            }
-            const int slot = c == 0 ? 0 : c == 1 ? 1 + dir : 2 + c;
+            for (int p = 0; p < n; ++p) s = fmaf(phi[p], S[at + p * st], s);
+            return s;
+        };
+        float rec[5];
 #pragma unroll
-            for (int v = 0; v < 5; ++v) {
-                const float* S = A + slot * SL + v * n3;
-                float s = 0.0f;
+        for (int v = 0; v < 5; ++v) rec[v] = ext(A + v * n3);
+        const float mn = dir == 0 ? rec[1] : dir == 1 ? rec[2] : rec[3];
+        double* tr = trace + ((size_t)cell * 6 + f) * kTr3 * n2 + m;
+        if (active) {
+            tr[5 * n2] = f32_to_f64(mn);
 #pragma unroll
-                for (int p = 0; p < n; ++p) {
-                    const int at = dir == 0 ? (a * n + b) * n + p : dir == 1 ? (a * n + p) * n + b : (p * n + a) * n + b;
-                    s = fmaf(phi[p], S[at], s);
-                }
-                rec[c * 5 + v] = f32_to_f64(s);
-            }
+            for (int c = 0; c < 3; ++c) tr[(6 + c) * n2] = f32_to_f64(ext(A + (5 + fx3_t(c, dir)) * n3));
+            tr[9 * n2] = f32_to_f64(ext(A + (11 + dir) * n3));
+            if (wallface)
+                for (int c = 0; c < 15; ++c) tr[(10 + c) * n2] = f32_to_f64(ext(A + (14 + c) * n3));
         }
         // FP64 base of the face node: the nodal background at the node's height
         // on x- and y-faces, its extrapolation on z-faces
@@ -1048,25 +1110,24 @@ k3_predictor_mixed(const double* __restrict__ u, double* __restrict__ rvol, doub
                 pbf = e[1];
                 zf = (float)(P64.org[2] + (iz + ((f & 1) ? 0 : 1)) * P64.h[2]);
             }
-            const float qp0 = (float)rec[0], qp4 = (float)rec[4];
-            const float m0 = (float)rec[1], m1 = (float)rec[2], m2 = (float)rec[3];
+            const float qp0 = rec[0], qp4 = rec[4];
+            const float m0 = rec[1], m1 = rec[2], m2 = rec[3];
             const float rho = rbf + qp0;
             const float rinv = __frcp_rn(rho);
             const float pp = P.gm1 * (qp4 - 0.5f * (m0 * m0 + m1 * m1 + m2 * m2) * rinv - P.g * zf * qp0);
-            const float mn = dir == 0 ? m0 : dir == 1 ? m1 : m2;
             const float sp = fabsf(mn) * rinv + sqrtf(P.gamma * (pbf + pp) * rinv) +
                              2.0f * P.eta[dir] * P.lamv * rinv;
-            rec[25] = f32_to_f64(sp);
+            if (active) tr[25 * n2] = f32_to_f64(sp);
         }
-        rec[0] += brho;
-        rec[4] += bE;
         if (active) {
-            double* tr = trace + ((size_t)cell * 6 + f) * kTr3 * n2;
-#pragma unroll
-            for (int c = 0; c < kTr3; ++c)
-                if (c < 10 || c == 25 || wallface) tr[c * n2 + m] = rec[c];
+            tr[0] = f32_to_f64(rec[0]) + brho;
+            tr[n2] = f32_to_f64(rec[1]);
+            tr[2 * n2] = f32_to_f64(rec[2]);
+            tr[3 * n2] = f32_to_f64(rec[3]);
+            tr[4 * n2] = f32_to_f64(rec[4]) + bE;
         }
-    }    pdl_trigger();
+    }
+    pdl_trigger();
 }
 
 // nodal values of a scenario: the 3D cosine bubble or the background
