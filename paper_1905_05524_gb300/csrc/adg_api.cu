@@ -402,6 +402,7 @@ int adg_create_mesh(const adg_mesh_desc* d, adg_mesh** out) {
     P.kappa = d->mu * P.cp / d->Pr;
     P.g = d->g;
     P.p0 = d->p0;
+    P.inv_p0 = 1.0 / d->p0;
     P.theta0 = d->theta0;
     P.Rcp = d->R / P.cp;
     P.lamv = std::fmax(4.0 / 3.0, d->gamma / d->Pr) * d->mu;
@@ -958,6 +959,7 @@ extern "C" int adg_step_noalloc(const adg_mesh_desc* d, double* u, size_t count,
     P.kappa = d->mu * P.cp / d->Pr;
     P.g = d->g;
     P.p0 = d->p0;
+    P.inv_p0 = 1.0 / d->p0;
     P.theta0 = d->theta0;
     P.Rcp = d->R / P.cp;
     P.lamv = std::fmax(4.0 / 3.0, d->gamma / d->Pr) * d->mu;

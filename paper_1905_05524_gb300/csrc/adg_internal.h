@@ -34,7 +34,7 @@ struct Basis {
 
 // Physical and mesh constants of one mesh.
 struct Phys {
-    double gamma, gm1, R, invR, mu, kappa, g, cp, p0, theta0, Rcp;
+    double gamma, gm1, R, invR, mu, kappa, g, cp, p0, inv_p0, theta0, Rcp;
     double lamv;              // max(4/3, gamma/Pr) * mu  (viscous eigenvalue * rho)
     double eta_x, eta_y;      // (2N+1) / (h sqrt(pi/2)) per direction
     double hx, hy, inv_hx, inv_hy, x0, y0;

@@ -8,6 +8,7 @@
 //   Eq. 7  momentum flux with p' = p - pbar(z), source -g rho' in the z row
 // Gradients of v, p, T follow from grad Q by the chain rule.
 #pragma once
+#include "adg_fixed.cuh"
 #include "adg_internal.h"
 
 namespace adg {
@@ -86,7 +87,7 @@ __device__ __forceinline__ void steady_source(double x, double y, const Phys& P,
 // Rusanov speed |v.n| + c + 2 eta lambda_v of a face state (normal along x
 // if xdir, else along y), lambda_v = max(4/3, gamma/Pr) mu / rho.
 __device__ __forceinline__ double wave_speed(const double q[4], double z, bool xdir, const Phys& P) {
-    const double rinv = 1.0 / q[0];
+    const double rinv = fx_rcp(q[0]);
     const double u = q[1] * rinv, v = q[2] * rinv;
     const double gz = P.gravity ? P.g * z : 0.0;
     const double p = P.gm1 * (q[3] - 0.5 * (q[1] * u + q[2] * v) - q[0] * gz);

@@ -9,6 +9,7 @@
 // derivative matrix.
 #pragma once
 #include "adg_convert.cuh"
+#include "adg_fixed.cuh"
 #include "adg_internal.h"
 
 namespace adg {
@@ -31,12 +32,20 @@ __device__ __forceinline__ float tv_node_z(int iy, int j, const BasisF& B, const
     return __fadd_rn(P.y0, __fmul_rn(__fadd_rn((float)iy, B.xi[j]), P.hy));
 }
 
+// T (p0/p)^(R/cp), for p within 0.6 p0 .. 1.65 p0 (the lowest 4 km) as
+// T exp(-(R/cp) log(p/p0)): 60 FP64 issue slots against 116 with pow and two
+// divisions (92 and 12 of them; log 30, exp 15), two thirds of the indicator.
+// There |log| < 1/2, so the roundings of the logarithm and of the product
+// reach the result below a quarter of its last place; farther out they would
+// not, and pow stays.
 __device__ __forceinline__ double theta_of(const double q[4], double z, const Phys& P) {
-    const double rinv = __ddiv_rn(1.0, q[0]);
+    const double rinv = fx_rcp(q[0]);
     const double gz = P.gravity ? __dmul_rn(P.g, z) : 0.0;
     const double ke = __dmul_rn(__dmul_rn(0.5, __dadd_rn(__dmul_rn(q[1], q[1]), __dmul_rn(q[2], q[2]))), rinv);
     const double p = __dmul_rn(P.gm1, __dsub_rn(__dsub_rn(q[3], ke), __dmul_rn(q[0], gz)));
     const double T = __dmul_rn(__dmul_rn(p, rinv), P.invR);
+    const double w = __dmul_rn(p, P.inv_p0);
+    if (w > 0.6 && w < 1.65) return __dmul_rn(T, exp(__dmul_rn(-P.Rcp, log(w))));
     return __dmul_rn(T, pow(__ddiv_rn(P.p0, p), P.Rcp));
 }
 
