@@ -443,6 +443,75 @@ struct AmrMixCfg {
     static constexpr int stride = raw + ((16 - raw % 32) + 32) % 32;
 };
 
+// weak volume residual of a leaf's node, one expression for both thread layouts
+__device__ __forceinline__ float amr_rvol(float sx, float sy, float inv_hx, float inv_hy, float S) {
+    return sx * inv_hx + sy * inv_hy + S;
+}
+
+// Face records of a leaf from its time averages A (slots of SLP floats, rows of
+// NP): by the threads loc of the leaf, step threads in all.
+template <int N, int NP>
+__device__ __forceinline__ void amr_mixed_faces(const float* A, double* __restrict__ trace, int cells, int cell, bool active,
+                                                unsigned wf, int loc, int step, double hx, double hy, double yorg,
+                                                const BasisF& B, const PhysF& P, const double* __restrict__ mb64,
+                                                const float* __restrict__ mbf) {
+    constexpr int n = N + 1, RS = n * NP, SLP = 4 * RS;
+    const float eta_x = (2.f * N + 1.f) / ((float)hx * 1.2533141f), eta_y = (2.f * N + 1.f) / ((float)hy * 1.2533141f);
+    for (int idx = loc; idx < 4 * n; idx += step) {
+        const int f = idx / n, m = idx - f * n;
+        const bool xface = f < 2;
+        const float* phi = (f == 0 || f == 2) ? B.phi1 : B.phi0;
+        const bool wall = wf >> f & 1u;
+        float rec[kTraceComps];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            if (c >= 2 && !wall) continue;
+            const int slot = c == 0 ? 0 : c == 1 ? (xface ? 1 : 2) : (c == 2 ? 3 : 4);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                const float* S = A + slot * SLP + v * RS;
+                float s = 0.f;
+#pragma unroll
+                for (int p = 0; p < n; ++p) s = fmaf(phi[p], xface ? S[m * NP + p] : S[p * NP + m], s);
+                rec[c * 4 + v] = s;
+            }
+        }
+        // FP64 base and FP32 speed base of the face node
+        double brho, bE;
+        float rbf, pbf, zf;
+        if (xface) {
+            const size_t rm = (size_t)cell * n + m;
+            brho = mb64[rm * 2];
+            bE = mb64[rm * 2 + 1];
+            rbf = f64_to_f32(brho);
+            pbf = mbf[rm * 3];
+            zf = (float)(yorg + (double)B.xi[m] * hy);
+        } else {
+            const size_t side = (size_t)cell * 2 + (f == 2 ? 0 : 1);
+            const size_t o64 = (size_t)cells * n * 2 + side * 2, o32 = (size_t)cells * n * 3 + side * 2;
+            brho = mb64[o64];
+            bE = mb64[o64 + 1];
+            rbf = mbf[o32];
+            pbf = mbf[o32 + 1];
+            zf = (float)(yorg + (f == 2 ? hy : 0.0));
+        }
+        const float rho = rbf + rec[0];
+        const float rinv = __frcp_rn(rho);
+        const float pp = P.gm1 * (rec[3] - 0.5f * (rec[1] * rec[1] + rec[2] * rec[2]) * rinv - P.g * zf * rec[0]);
+        const float sp = fabsf((xface ? rec[1] : rec[2]) * rinv) + sqrtf(P.gamma * (pbf + pp) * rinv) +
+                         2.f * (xface ? eta_x : eta_y) * P.lamv * rinv;
+        if (active) {
+            double* tr = trace + ((size_t)cell * 4 + f) * kTraceComps * n;
+#pragma unroll
+            for (int c = 0; c < 16; ++c)
+                if (c < 8 || wall) tr[c * n + m] = f32_to_f64(rec[c]);
+            tr[0 * n + m] = brho + f32_to_f64(rec[0]);
+            tr[3 * n + m] = bE + f32_to_f64(rec[3]);
+            tr[16 * n + m] = f32_to_f64(sp);
+        }
+    }
+}
+
 // Per-leaf tables: mb64 [leaves][n][2] (rhobar, Ebar) then [leaves][2 N, S][2]
 // extrapolated (rhobar, Ebar); mbf [leaves][n][3] (pbar, d rhobar/dz,
 // d Ebar/dz) then [leaves][2 N, S][2] (extrapolated rhobar, (gamma-1)(Ebar -
@@ -657,63 +726,82 @@ __device__ __forceinline__ void predictor_amr_mixed_body(const double* __restric
                 sx = fmaf(B.Vx[p][i], A[1 * SL + v * n2 + j * n + p], sx);
                 sy = fmaf(B.Vx[p][j], A[2 * SL + v * n2 + p * n + i], sy);
             }
-            rc[v * n2 + node] = f32_to_f64(sx * inv_hx + sy * inv_hy + Sb[v]);
+            rc[v * n2 + node] = f32_to_f64(amr_rvol(sx, sy, inv_hx, inv_hy, Sb[v]));
         }
     }
-    const float eta_x = (2.f * N + 1.f) / ((float)hx * 1.2533141f), eta_y = (2.f * N + 1.f) / ((float)hy * 1.2533141f);
-    for (int idx = node; idx < 4 * n; idx += n2) {
-        const int f = idx / n, m = idx - f * n;
-        const bool xface = f < 2;
-        const float* phi = (f == 0 || f == 2) ? B.phi1 : B.phi0;
-        const bool wall = wf >> f & 1u;
-        float rec[kTraceComps];
+    amr_mixed_faces<N, n>(A, trace, cells, cell, active, wf, node, n2, hx, hy, yorg, B, P, mb64, mbf);
+}
+
+// Node pairs on the leaves (even n): the uniform meshes' predictor_pairs with
+// the leaf's spacing and background, the outputs of predictor_amr_mixed_body
+// bitwise.
+template <int N, int CPB>
+__device__ __forceinline__ void predictor_amr_mixed_pairs(const double* __restrict__ u, double* __restrict__ rvol,
+                                                          double* __restrict__ trace, int cells, int c0, float dt,
+                                                          const BasisF& B, const PhysF& P,
+                                                          const double* __restrict__ geo, const int* __restrict__ nbr,
+                                                          const double* __restrict__ mb64,
+                                                          const float* __restrict__ mbf, float* smf) {
+    using C = MixCfg2<N, CPB>;
+    constexpr int n = N + 1, n2 = n * n, SL = 4 * n2, TPC = C::tpc;
+    const int cl = threadIdx.x / TPC;
+    const int loc = threadIdx.x - cl * TPC;
+    const int ip = loc / n, j = loc - ip * n, i0 = 2 * ip, nd0 = j * n + i0;
+    const int cell_raw = c0 + cl;
+    const bool active = cell_raw < cells;
+    const int cell = active ? cell_raw : cells - 1;
+    float2* Q2 = reinterpret_cast<float2*>(smf + (size_t)cl * C::stride);
+    unsigned wf = 0;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            if (c >= 2 && !wall) continue;
-            const int slot = c == 0 ? 0 : c == 1 ? (xface ? 1 : 2) : (c == 2 ? 3 : 4);
+    for (int f = 0; f < 4; ++f) wf |= nbr[((size_t)cell * 4 + f) * kNbrInts] == NB_WALL ? 1u << f : 0u;
+    const double* ge = geo + (size_t)cell * kGeo;
+    const double hx = ge[2], hy = ge[3], yorg = ge[1];
+    const float inv_hx = (float)ge[4], inv_hy = (float)ge[5];
+    const float z = (float)(yorg + (double)B.xi[j] * hy);
+    const size_t rowj = (size_t)cell * n + j;
+    const double rb64 = mb64[rowj * 2], Eb64 = mb64[rowj * 2 + 1];
+    const float rb = f64_to_f32(rb64), Eb = f64_to_f32(Eb64);
+    const float pb = mbf[rowj * 3], dzr = mbf[rowj * 3 + 1], dzE = mbf[rowj * 3 + 2];
+    float up[2][4];
+    const float Sm[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    const double* uc = u + (size_t)cell * SL;
 #pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const float* S = A + slot * SL + v * n2;
-                float s = 0.f;
+    for (int a = 0; a < 2; ++a) {
+        up[a][0] = f64_to_f32(__dsub_rn(uc[nd0 + a], rb64));
+        up[a][1] = f64_to_f32(uc[n2 + nd0 + a]);
+        up[a][2] = f64_to_f32(uc[2 * n2 + nd0 + a]);
+        up[a][3] = f64_to_f32(__dsub_rn(uc[3 * n2 + nd0 + a], Eb64));
+    }
+    float Sz[2];
+    predictor_pairs<N, CPB>(Q2, ip, j, up, Sm, z, rb, Eb, pb, dzr, dzE, inv_hx, inv_hy, dt, wf, B, P, Sz);
+    const float* A = reinterpret_cast<const float*>(Q2);
+    if (active) {
+        double* rc = rvol + (size_t)cell * SL;
 #pragma unroll
-                for (int p = 0; p < n; ++p) s = fmaf(phi[p], xface ? S[m * n + p] : S[p * n + m], s);
-                rec[c * 4 + v] = s;
+        for (int v = 0; v < 4; ++v) {
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                float sx = 0.f, sy = 0.f;
+#pragma unroll
+                for (int p = 0; p < n; ++p) {
+                    sx = fmaf(B.Vx[p][i0 + b], A[1 * SL + v * n2 + j * n + p], sx);
+                    sy = fmaf(B.Vx[p][j], A[2 * SL + v * n2 + p * n + i0 + b], sy);
+                }
+                rc[v * n2 + nd0 + b] = f32_to_f64(amr_rvol(sx, sy, inv_hx, inv_hy, v == 2 ? Sz[b] : 0.f));
             }
         }
-        // FP64 base and FP32 speed base of the face node
-        double brho, bE;
-        float rbf, pbf, zf;
-        if (xface) {
-            const size_t rm = (size_t)cell * n + m;
-            brho = mb64[rm * 2];
-            bE = mb64[rm * 2 + 1];
-            rbf = f64_to_f32(brho);
-            pbf = mbf[rm * 3];
-            zf = (float)(yorg + (double)B.xi[m] * hy);
-        } else {
-            const size_t side = (size_t)cell * 2 + (f == 2 ? 0 : 1);
-            const size_t o64 = (size_t)cells * n * 2 + side * 2, o32 = (size_t)cells * n * 3 + side * 2;
-            brho = mb64[o64];
-            bE = mb64[o64 + 1];
-            rbf = mbf[o32];
-            pbf = mbf[o32 + 1];
-            zf = (float)(yorg + (f == 2 ? hy : 0.0));
-        }
-        const float rho = rbf + rec[0];
-        const float rinv = __frcp_rn(rho);
-        const float pp = P.gm1 * (rec[3] - 0.5f * (rec[1] * rec[1] + rec[2] * rec[2]) * rinv - P.g * zf * rec[0]);
-        const float sp = fabsf((xface ? rec[1] : rec[2]) * rinv) + sqrtf(P.gamma * (pbf + pp) * rinv) +
-                         2.f * (xface ? eta_x : eta_y) * P.lamv * rinv;
-        if (active) {
-            double* tr = trace + ((size_t)cell * 4 + f) * kTraceComps * n;
-#pragma unroll
-            for (int c = 0; c < 16; ++c)
-                if (c < 8 || wall) tr[c * n + m] = f32_to_f64(rec[c]);
-            tr[0 * n + m] = brho + f32_to_f64(rec[0]);
-            tr[3 * n + m] = bE + f32_to_f64(rec[3]);
-            tr[16 * n + m] = f32_to_f64(sp);
-        }
     }
+    amr_mixed_faces<N, n>(A, trace, cells, cell, active, wf, loc, TPC, hx, hy, yorg, B, P, mb64, mbf);
+}
+
+template <int N, int CPB>
+__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1) / 2, (MixCfg2<N, CPB>::minb))
+k_predictor_amr_mixed_pairs(const double* __restrict__ u, double* __restrict__ rvol, double* __restrict__ trace, int cells,
+                            float dt, const BasisF B, const PhysF P, const double* __restrict__ geo,
+                            const int* __restrict__ nbr, const double* __restrict__ mb64,
+                            const float* __restrict__ mbf) {
+    extern __shared__ float smf[];
+    predictor_amr_mixed_pairs<N, CPB>(u, rvol, trace, cells, blockIdx.x * CPB, dt, B, P, geo, nbr, mb64, mbf, smf);
 }
 
 template <int N, int CPB>
@@ -1093,18 +1181,40 @@ struct AmrCfg {
     }                                             \
     return fail(ADG_EINVAL, "bad degree");
 
-// Leaves per block of the per-mesh mixed adaptive predictor (the TV
-// statistics of adaptive meshes come from their own kernel, so this need not
-// be tv_cpb).  Measured at N = 5 on the two-bubble tree (1065 leaves, under
-// half a wave): 4 leaves 2.61e9, 2 leaves 2.60e9, 1 leaf 2.43e9 DOF-updates/s.
+// Leaves per block of the per-mesh mixed adaptive predictor with one node per
+// thread (even degrees and degree 1; the TV statistics of adaptive meshes come
+// from their own kernel, so this need not be tv_cpb).
 template <int N>
 constexpr int amr_mixed_cpb() {
     return AmrCfg<N>::cpb;
 }
 
+// Node pairs on the leaves; N = 5, two-bubble tree of 1489 leaves, ten steps and
+// the indicator: 558 us with 3 leaves a block, 568 / 582 / 639 / 660 with 5 / 7 /
+// 4 / 2, 619 with one node per thread and 4 leaves.
+template <int N, int CPB>
+static cudaError_t launch_amr_pairs(adg_mesh* m, float dt, cudaStream_t s) {
+    using C = MixCfg2<N, CPB>;
+    auto kern = k_predictor_amr_mixed_pairs<N, CPB>;
+    const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_pred);
+    if (e != cudaSuccess) return e;
+    kern<<<(m->cells + CPB - 1) / CPB, C::threads, C::smem_pred, s>>>(m->u, m->rvol, m->trace, m->cells, dt, m->Bf, m->Pf,
+                                                                   m->geo, m->nbr, m->mbl64, m->mblf);
+    return cudaGetLastError();
+}
+
 template <int N>
 static int pred_n(adg_mesh* m, double dt, cudaStream_t s) {
     if (m->d.precision == ADG_PREC_MIXED) {
+        if constexpr (N == 3 || N == 5 || N == 7) {  // node pairs, as on uniform meshes
+            using C2 = MixCfg2<N>;
+            if (m->cells > C2::single_cells * sm_count()) {
+                ADG_CK((m->cells <= C2::small_cells * sm_count() ? launch_amr_pairs<N, C2::cpb_small>(m, (float)dt, s)
+                                                                 : launch_amr_pairs<N, C2::cpb>(m, (float)dt, s)),
+                       "amr mixed predictor launch");
+                return ADG_OK;
+            }
+        }
         constexpr int CM = amr_mixed_cpb<N>();
         auto km = k_predictor_amr_mixed<N, CM>;
         const size_t smem = (size_t)CM * AmrMixCfg<N>::stride * sizeof(float);

@@ -116,12 +116,18 @@ __device__ __forceinline__ double fx_rcp(double x) {
     return fma(r0, fma(e, e, e), r0);
 }
 
-// Blocks of a launch that strides over `tiles` tiles: as many rounds as the
-// resident blocks need, the tiles spread evenly over them.
-inline int fx_grid(int tiles, int resident) {
+// SMs of the current device.
+inline int sm_count() {
     int dev = 0, sms = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+// Blocks of a launch that strides over `tiles` tiles: as many rounds as the
+// resident blocks need, the tiles spread evenly over them.
+inline int fx_grid(int tiles, int resident) {
+    const int sms = sm_count();
     const int rounds = (tiles + sms * resident - 1) / (sms * resident);
     return (tiles + rounds - 1) / rounds;
 }

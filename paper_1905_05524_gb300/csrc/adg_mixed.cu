@@ -22,6 +22,7 @@
 
 #include "adg_convert.cuh"
 #include "adg_internal.h"
+#include "adg_fixed.cuh"
 #include "adg_mixed_body.cuh"
 #include "adg_mixed_x2.cuh"
 #include "adg_mixed_point.cuh"
@@ -68,19 +69,28 @@ constexpr int pred_cpb() {
     return N == 6 ? 5 : MixCfg<N>::cpb_default;
 }
 
+template <int N, int CPB>
+static int launch_pairs(const double* u, float* rvol, float* trace, int cells, float dt, const BasisF& B, const PhysF& P,
+                        const MixedBg& bg, cudaStream_t s) {
+    using C = MixCfg2<N, CPB>;
+    auto kern = k_predictor_mixed_x2<N, CPB>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C::smem_pred);
+    if (e != cudaSuccess) return (int)e;
+    kern<<<(cells + CPB - 1) / CPB, C::threads, C::smem_pred, s>>>(u, rvol, trace, cells, dt, B, P, bg);
+    return (int)cudaGetLastError();
+}
+
 template <int N>
 static int launch_pred_mixed(const double* u, float* rvol, float* trace, int cells, float dt,
                              const BasisF& B, const PhysF& P, const MixedBg& bg, cudaStream_t s) {
     // node pairs where a row has an even number of nodes: 2124 against 2405 us
     // per 243x243 launch at N = 7 (N = 1 has rows of one pair)
     if constexpr (N == 3 || N == 5 || N == 7) {
-        using C2 = MixCfg2<N>;
-        auto kern = k_predictor_mixed_x2<N, C2::cpb>;
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)C2::smem_pred);
-        if (e != cudaSuccess) return (int)e;
-        const int blocks = (cells + C2::cpb - 1) / C2::cpb;
-        kern<<<blocks, C2::threads, C2::smem_pred, s>>>(u, rvol, trace, cells, dt, B, P, bg);
-        return (int)cudaGetLastError();
+        using C = MixCfg2<N>;
+        if (cells > C::single_cells * sm_count())
+            return cells <= C::small_cells * sm_count()
+                       ? launch_pairs<N, C::cpb_small>(u, rvol, trace, cells, dt, B, P, bg, s)
+                       : launch_pairs<N, C::cpb>(u, rvol, trace, cells, dt, B, P, bg, s);
     }
     using C = MixCfg<N, pred_cpb<N>()>;
     auto kern = k_predictor_mixed<N, C::cpb>;

@@ -48,70 +48,56 @@ struct MixCfg2 {
     // resident blocks asked of the register allocator: four at N = 3 (128
     // registers, 111.3 us per 243x243 launch; three 113.1), three at N = 5
     // (642 us; four spill, 645), four at N = 7
-    static constexpr int minb = N == 5 ? 3 : N == 3 || N == 7 ? 4 : 1;
+    // Meshes that do not fill the chip run smaller blocks, so that every SM and
+    // sub-partition has some (up to small_cells per SM, all resident at once): a
+    // degree-5 step on 9x9 cells 22.7 -> 19.1 us, on 40x40 36.0 -> 30.9, degree 3
+    // on 81x81 24.7 -> 20.8; degree 5 keeps 255 registers (168 and six blocks:
+    // the two-bubble tree 578 against 558 us).  At degree 7 half the threads take
+    // longer than they save while there are few cells: up to single_cells per SM
+    // the node-per-thread kernel runs (9x9 28 us against 39, 20x20 39 / 41, 40x40
+    // 96 / 80)
+    static constexpr int cpb_small = N == 3 ? 4 : N == 5 ? 3 : 1;
+    static constexpr int small_cells = N == 3 ? 64 : N == 5 ? 12 : 8;
+    static constexpr int single_cells = N == 7 ? 4 : 0;
+    static constexpr int minb = cpb == cpb_small ? small_cells / cpb_small : N == 5 ? 3 : N == 3 || N == 7 ? 4 : 1;
 };
 
+// The sweeps, the final evaluation and the time averages of one cell, from the
+// node pair's state (up), source (Sm), background (rb, Eb, pb and the
+// interpolant's derivatives) and height z to the averages in shared memory:
+// rows of A in slots 0..4 = qbar, Fbar, Gbar, qxbar, qybar (the gradients where
+// wf, the mask of the cell's wall faces, is not zero: they are read on walls
+// only) and the average of the z-momentum source in Sz.  Shared by uniform
+// cells and the leaves of adaptive meshes.
 template <int N, int CPB>
-__device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict__ u, float* __restrict__ rvol,
-                                                        float* __restrict__ trace, int cells, int c0, float dt,
-                                                        const BasisF& B, const PhysF& P, const MixedBg& bg,
-                                                        float* smf) {
+__device__ __forceinline__ void predictor_pairs(float2* Q2, int ip, int j, const float up[2][4], const float Sm[2][4],
+                                                float z, float rb, float Eb, float pb, float dzr, float dzE, float inv_hx,
+                                                float inv_hy, float dt, unsigned wf, const BasisF& B, const PhysF& P,
+                                                float Sz[2]) {
     using C = MixCfg2<N, CPB>;
-    constexpr int n = N + 1, n2 = n * n, SL = 4 * n2, TPC = C::tpc;
+    constexpr int n = N + 1;
     constexpr int NP = n, RS = n * NP, SLP = 4 * RS;  // time-average rows (even n: no padding)
     constexpr int NPAIR = C::npair, RQ = C::rq, PL = n * RQ, PS = 4 * PL;  // slice pairs, row, plane and pair strides (float2)
-    const int cl = threadIdx.x / TPC;
-    const int loc = threadIdx.x - cl * TPC;
-    // column-pair-major: the lanes of one column pair are adjacent, so a
-    // column load is one run of equal addresses (a shared-memory load costs
-    // a wavefront per run of adjacent lanes with equal addresses, at most 16
-    // runs of 8-byte or 8 of 16-byte accesses in one)
-    const int ip = loc / n, j = loc - ip * n, i0 = 2 * ip;
-    const int nd0 = j * n + i0;  // first node of the pair; the second is nd0 + 1
-    const int ns0 = j * RQ + i0;  // its place in a plane of the slice-pair arrays
-    const int cell_raw = c0 + cl;
-    const bool active = cell_raw < cells;
-    const int cell = active ? cell_raw : cells - 1;
-    float2* Q2 = reinterpret_cast<float2*>(smf + (size_t)cl * C::stride);  // [h][v][j][i]
+    constexpr int FS = 3 * PL;  // F and G hold v = 1..3: the mass fluxes are momenta
+    const int i0 = 2 * ip, ns0 = j * RQ + i0;
     float2* F2 = Q2 + NPAIR * PS;
-    constexpr int FS = 3 * PL;            // F and G hold v = 1..3: the mass fluxes are momenta
     float2* G2 = F2 + NPAIR * FS;
     // float4 = the float2 pairs of nodes (a, b) and (a, b+1), b even
     auto ld4 = [](const float2* S, int idx) { return *reinterpret_cast<const float4*>(S + idx); };
     auto st4 = [](float2* S, int idx, float2 a, float2 b) {
         *reinterpret_cast<float4*>(S + idx) = make_float4(a.x, a.y, b.x, b.y);
     };
-    const int ix = cell % P.nx, iy = cell / P.nx;
-    const int row = iy * n + j;
-    const float z = node_coord_f(P.y0, iy, B.xi[j], P.hy);
-    const double rb64 = bg.rb[row], Eb64 = bg.Eb[row];
-    const float rb = f64_to_f32(rb64), Eb = f64_to_f32(Eb64), pb = bg.pb[row];
-    const float dzr = bg.dzr[row], dzE = bg.dzE[row];
-    float up[2][4];
-    const double* uc = u + (size_t)cell * SL;
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-        up[a][0] = f64_to_f32(uc[nd0 + a] - rb64);
-        up[a][1] = f64_to_f32(uc[n2 + nd0 + a]);
-        up[a][2] = f64_to_f32(uc[2 * n2 + nd0 + a]);
-        up[a][3] = f64_to_f32(uc[3 * n2 + nd0 + a] - Eb64);
-    }
 #pragma unroll
     for (int v = 0; v < 4; ++v) st4(Q2, v * PL + ns0, bc2(up[0][v]), bc2(up[1][v]));
-    float Sm[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-    if (P.source == ADG_SRC_STEADY) {
-#pragma unroll
-        for (int a = 0; a < 2; ++a) steady_source_f(node_coord_f(P.x0, ix, B.xi[i0 + a], P.hx), z, P, Sm[a]);
-    }
     __syncthreads();
 
     // the two nodes' rows of D along x and the row's column of D along y, scaled by 1/h
     float dI0[n], dI1[n], dJ[n];
 #pragma unroll
     for (int p = 0; p < n; ++p) {
-        dI0[p] = B.D[i0][p] * P.inv_hx;
-        dI1[p] = B.D[i0 + 1][p] * P.inv_hx;
-        dJ[p] = B.D[j][p] * P.inv_hy;
+        dI0[p] = B.D[i0][p] * inv_hx;
+        dI1[p] = B.D[i0 + 1][p] * inv_hx;
+        dJ[p] = B.D[j][p] * inv_hy;
     }
     // x-contractions of row j for both nodes: one 16-byte load per two terms
     auto xdot2 = [&](const float2* S, float2& s0, float2& s1) {
@@ -269,8 +255,8 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
     }
 
     // final evaluation on the converged iterate and the time averages
-    const unsigned wf = wall_faces(ix, iy, P);  // grad q-bar is read on walls only
-    float qb[2][4], Fb[2][4], Gb[2][4], qxb[2][4], qyb[2][4], Sz[2] = {0.f, 0.f};
+    float qb[2][4], Fb[2][4], Gb[2][4], qxb[2][4], qyb[2][4];
+    Sz[0] = Sz[1] = 0.f;
 #pragma unroll
     for (int b = 0; b < 2; ++b)
 #pragma unroll
@@ -325,6 +311,53 @@ __device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict
         }
     }
     __syncthreads();
+}
+
+template <int N, int CPB>
+__device__ __forceinline__ void predictor_mixed_body_x2(const double* __restrict__ u, float* __restrict__ rvol,
+                                                        float* __restrict__ trace, int cells, int c0, float dt,
+                                                        const BasisF& B, const PhysF& P, const MixedBg& bg,
+                                                        float* smf) {
+    using C = MixCfg2<N, CPB>;
+    constexpr int n = N + 1, n2 = n * n, SL = 4 * n2, TPC = C::tpc;
+    constexpr int NP = n, RS = n * NP, SLP = 4 * RS;  // time-average rows (even n: no padding)
+    const int cl = threadIdx.x / TPC;
+    const int loc = threadIdx.x - cl * TPC;
+    // column-pair-major: the lanes of one column pair are adjacent, so a
+    // column load is one run of equal addresses (a shared-memory load costs
+    // a wavefront per run of adjacent lanes with equal addresses, at most 16
+    // runs of 8-byte or 8 of 16-byte accesses in one)
+    const int ip = loc / n, j = loc - ip * n, i0 = 2 * ip;
+    const int nd0 = j * n + i0;  // first node of the pair; the second is nd0 + 1
+    const int cell_raw = c0 + cl;
+    const bool active = cell_raw < cells;
+    const int cell = active ? cell_raw : cells - 1;
+    float2* Q2 = reinterpret_cast<float2*>(smf + (size_t)cl * C::stride);  // [h][v][j][i]
+    const int ix = cell % P.nx, iy = cell / P.nx;
+    const int row = iy * n + j;
+    const float z = node_coord_f(P.y0, iy, B.xi[j], P.hy);
+    const double rb64 = bg.rb[row], Eb64 = bg.Eb[row];
+    const float rb = f64_to_f32(rb64), Eb = f64_to_f32(Eb64), pb = bg.pb[row];
+    const float dzr = bg.dzr[row], dzE = bg.dzE[row];
+    float up[2][4];
+    const double* uc = u + (size_t)cell * SL;
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+        up[a][0] = f64_to_f32(uc[nd0 + a] - rb64);
+        up[a][1] = f64_to_f32(uc[n2 + nd0 + a]);
+        up[a][2] = f64_to_f32(uc[2 * n2 + nd0 + a]);
+        up[a][3] = f64_to_f32(uc[3 * n2 + nd0 + a] - Eb64);
+    }
+    float Sm[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+    if (P.source == ADG_SRC_STEADY) {
+#pragma unroll
+        for (int a = 0; a < 2; ++a) steady_source_f(node_coord_f(P.x0, ix, B.xi[i0 + a], P.hx), z, P, Sm[a]);
+    }
+    const unsigned wf = wall_faces(ix, iy, P);
+    float Sz[2];
+    predictor_pairs<N, CPB>(Q2, ip, j, up, Sm, z, rb, Eb, pb, dzr, dzE, P.inv_hx, P.inv_hy, dt, wf, B, P, Sz);
+    const float* A = reinterpret_cast<const float*>(Q2);
+    auto st2 = [](float* p, float a, float b) { *reinterpret_cast<float2*>(p) = make_float2(a, b); };
     if (active) {
         float* rc = rvol + (size_t)cell * SL;
 #pragma unroll
