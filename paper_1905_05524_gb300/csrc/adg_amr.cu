@@ -412,6 +412,7 @@ k_predictor_amr(const double* __restrict__ u, double* __restrict__ rvol, double*
                                            bgl[((size_t)cell * C::n + j) * 2], bgl[((size_t)cell * C::n + j) * 2 + 1],
                                            gmask, sm + (size_t)cl * C::words(false), 0.0, ttrace);
     }
+    pdl_trigger();  // the corrector (launched programmatically) may be scheduled
 }
 
 template <int N, bool REC>
@@ -802,6 +803,7 @@ k_predictor_amr_mixed_pairs(const double* __restrict__ u, double* __restrict__ r
                             const float* __restrict__ mbf) {
     extern __shared__ float smf[];
     predictor_amr_mixed_pairs<N, CPB>(u, rvol, trace, cells, blockIdx.x * CPB, dt, B, P, geo, nbr, mb64, mbf, smf);
+    pdl_trigger();
 }
 
 template <int N, int CPB>
@@ -811,6 +813,7 @@ k_predictor_amr_mixed(const double* __restrict__ u, double* __restrict__ rvol, d
                       const int* __restrict__ nbr, const double* __restrict__ mb64, const float* __restrict__ mbf) {
     extern __shared__ float smf[];
     predictor_amr_mixed_body<N, CPB>(u, rvol, trace, cells, blockIdx.x * CPB, dt, B, P, geo, nbr, mb64, mbf, smf);
+    pdl_trigger();
 }
 
 // face data (q-bar and normal flux) of record `rec` of a coarse face evaluated
@@ -1005,10 +1008,10 @@ __device__ __forceinline__ void corrector_amr_body(double* __restrict__ u, const
 
 template <int N, int CPB>
 __global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
-k_corrector_amr(double* __restrict__ u, const double* __restrict__ rvol, const double* __restrict__ trace,
-                int cells, double dt, const Basis B, const Phys P0, const AmrOps O, const double* __restrict__ geo,
+k_corrector_amr(double* __restrict__ u, const double* rvol, const double* trace, int cells, double dt, const Basis B, const Phys P0, const AmrOps O, const double* __restrict__ geo,
                 const int* __restrict__ nbr, const double* __restrict__ bgl) {
-    corrector_amr_body<N, CPB>(u, rvol, trace, cells, blockIdx.x * CPB, dt, B, P0, O, geo, nbr, bgl);
+    pdl_wait();  // the predictor's residual and traces are complete and visible
+    corrector_amr_body<N, CPB>(u, pdl_fresh(rvol), pdl_fresh(trace), cells, blockIdx.x * CPB, dt, B, P0, O, geo, nbr, bgl);
 }
 
 template <int N, int CPB>
@@ -1233,9 +1236,9 @@ int amr_predictor(adg_mesh* m, double dt, void* stream) { AMR_DISPATCH(pred_n, m
 template <int N>
 static int corr_n(adg_mesh* m, double dt, cudaStream_t s) {
     using C = AmrCfg<N>;
-    k_corrector_amr<N, C::cpb><<<(m->cells + C::cpb - 1) / C::cpb, C::threads, 0, s>>>(
-        m->u, m->rvol, m->trace, m->cells, dt, m->B, m->P, tree_of(m)->ops, m->geo, m->nbr, m->bgl);
-    ADG_CK(cudaGetLastError(), "amr corrector launch");
+    ADG_CK(launch_programmatic(k_corrector_amr<N, C::cpb>, (m->cells + C::cpb - 1) / C::cpb, C::threads, s, m->u, m->rvol,
+                               m->trace, m->cells, dt, m->B, m->P, tree_of(m)->ops, m->geo, m->nbr, m->bgl),
+           "amr corrector launch");
     return ADG_OK;
 }
 int amr_corrector(adg_mesh* m, double dt, void* stream) { AMR_DISPATCH(corr_n, m, dt, (cudaStream_t)stream) }

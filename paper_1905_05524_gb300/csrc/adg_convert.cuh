@@ -59,4 +59,20 @@ __device__ __forceinline__ T* pdl_fresh(T* p) {
 }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Launch with that attribute.
+template <typename... K, typename... A>
+inline cudaError_t launch_programmatic(void (*kern)(K...), int grid, int threads, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<A&&>(args)...);
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 }  // namespace adg

@@ -22,6 +22,7 @@
 // whose iterate is constant in time, evaluates the fluxes once, not n times.
 #include <cuda_runtime.h>
 
+#include "adg_convert.cuh"
 #include "adg_internal.h"
 #include "adg_physics.cuh"
 #include "adg_fp64_body.cuh"
@@ -66,6 +67,7 @@ k_predictor_fp64(const double* __restrict__ u, double* __restrict__ rvol,
                                      P.y0 + iy * P.hy, bg.pbar_node[iy * C::n + j], bg.rhobar_node[iy * C::n + j],
                                      edge_faces(ix, iy, P), sm + (size_t)cl * C::words(TSRC), t);
     }
+    pdl_trigger();  // the corrector (launched programmatically) may be scheduled
 }
 
 // Slip-wall ghost of face f (0 E, 1 W, 2 N, 3 S) from the interior trace
@@ -275,10 +277,10 @@ __device__ __forceinline__ void corrector_fp64_body(double* __restrict__ u, cons
 
 template <int N, int CPB, bool TV>
 __global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
-k_corrector_fp64(double* __restrict__ u, const double* __restrict__ rvol,
-                 const double* __restrict__ trace, int cells, double dt, const Basis B,
+k_corrector_fp64(double* __restrict__ u, const double* rvol, const double* trace, int cells, double dt, const Basis B,
                  const Phys P, const Background bg, const TvEpilogue epi, double t) {
-    corrector_fp64_body<N, CPB, TV>(u, rvol, trace, cells, blockIdx.x * CPB, dt, B, P, bg, epi, t);
+    pdl_wait();  // the predictor's residual and traces are complete and visible
+    corrector_fp64_body<N, CPB, TV>(u, pdl_fresh(rvol), pdl_fresh(trace), cells, blockIdx.x * CPB, dt, B, P, bg, epi, t);
 }
 
 // Batched persistent FP64 kernels over uniform instances (tile = instance,
@@ -400,13 +402,14 @@ static int launch_corr(double* u, const double* rvol, const double* trace, int c
                        double t, cudaStream_t s) {
     using C = Fp64Cfg<N>;
     const int blocks = (cells + C::cpb - 1) / C::cpb;
-    if (epi)
-        k_corrector_fp64<N, C::cpb, true>
-            <<<blocks, C::threads, 0, s>>>(u, rvol, trace, cells, dt, B, P, bg, *epi, t);
-    else
-        k_corrector_fp64<N, C::cpb, false>
-            <<<blocks, C::threads, 0, s>>>(u, rvol, trace, cells, dt, B, P, bg, TvEpilogue{}, t);
-    return (int)cudaGetLastError();
+    const TvEpilogue e = epi ? *epi : TvEpilogue{};
+    auto kern = epi ? k_corrector_fp64<N, C::cpb, true> : k_corrector_fp64<N, C::cpb, false>;
+    // strips copy the neighbours' traces in between: an ordinary launch behind those copies
+    if (P.bc_y == ADG_BC_EXCHANGE || P.bc_y == ADG_BC_WALL_EXCHANGE || P.bc_y == ADG_BC_EXCHANGE_WALL) {
+        kern<<<blocks, C::threads, 0, s>>>(u, rvol, trace, cells, dt, B, P, bg, e, t);
+        return (int)cudaGetLastError();
+    }
+    return (int)launch_programmatic(kern, blocks, C::threads, s, u, rvol, trace, cells, dt, B, P, bg, e, t);
 }
 
 int launch_predictor_fp64(int N, const double* u, double* rvol, double* trace, int cells,
