@@ -35,7 +35,7 @@ struct AdjCfg {
     using F = FxCfg<N>;
     static constexpr int n = F::n, n2 = F::n2, n3 = F::n3;
     static constexpr int cpb = F::cpb, tpc = F::tpc, threads = F::threads;
-    static constexpr int resident = N == 5 ? 2 : 4;  // blocks per SM asked of the register allocator
+    static constexpr int resident = 2;  // blocks per SM asked of the register allocator (2 .. 8 within 1%)
     // per cell, in 8-byte words: the limbs of the iterates q^(0) (one time
     // slice) and q^(1..n); a work area (fluxes and residual forward; adjoints
     // of q, of the residual and of the gradients backward); u; D/h and -dt D/h;

@@ -400,15 +400,15 @@ k_predictor_amr(const double* __restrict__ u, double* __restrict__ rvol, double*
     for (int c0 = first + blockIdx.x * C::cpb; c0 < end; c0 += gridDim.x * C::cpb) {
         const bool active = c0 + cl < end;
         const int cell = active ? c0 + cl : end - 1;
-        const double4 ge = *reinterpret_cast<const double4*>(geo + (size_t)cell * kGeo);
-        if (ge.z != P.hx || ge.w != P.hy) {
+        const double* ge = geo + (size_t)cell * kGeo;
+        if (ge[2] != P.hx || ge[3] != P.hy) {
             P = leaf_phys(P0, geo, cell);
             O.make(B, fx_tab<N, false>(sm, cl), tid, P.inv_hx, P.inv_hy);
         }
         unsigned gmask = 0;
 #pragma unroll
         for (int f = 0; f < 4; ++f) gmask |= nbr[((size_t)cell * 4 + f) * kNbrInts] == NB_WALL ? 1u << f : 0u;
-        predictor_fp64_body<N, false, REC>(u, rvol, trace, cell, active, tid, dt, B, P, O, K, ge.x, ge.y,
+        predictor_fp64_body<N, false, REC>(u, rvol, trace, cell, active, tid, dt, B, P, O, K, ge[0], ge[1],
                                            bgl[((size_t)cell * C::n + j) * 2], bgl[((size_t)cell * C::n + j) * 2 + 1],
                                            gmask, sm + (size_t)cl * C::words(false), 0.0, ttrace);
     }
@@ -1007,9 +1007,11 @@ __device__ __forceinline__ void corrector_amr_body(double* __restrict__ u, const
 }
 
 template <int N, int CPB>
-__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
-k_corrector_amr(double* __restrict__ u, const double* rvol, const double* trace, int cells, double dt, const Basis B, const Phys P0, const AmrOps O, const double* __restrict__ geo,
-                const int* __restrict__ nbr, const double* __restrict__ bgl) {
+// (two blocks per SM asked: ten adaptive degree-5 steps and the indicator 519 us, 537 with three or unstated)
+__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1), 2)
+k_corrector_amr(double* __restrict__ u, const double* rvol, const double* trace, int cells, double dt, const Basis B,
+                const Phys P0, const AmrOps O, const double* __restrict__ geo, const int* __restrict__ nbr,
+                const double* __restrict__ bgl) {
     pdl_wait();  // the predictor's residual and traces are complete and visible
     corrector_amr_body<N, CPB>(u, pdl_fresh(rvol), pdl_fresh(trace), cells, blockIdx.x * CPB, dt, B, P0, O, geo, nbr, bgl);
 }
@@ -1024,7 +1026,7 @@ k_corrector_amr_lts(double* __restrict__ u, const double* __restrict__ rvol, con
 }
 
 template <int N, int CPB>
-__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
+__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1), 2)
 k_tv_cells_amr(const double* __restrict__ u, double* __restrict__ tv, double* __restrict__ part, int cells,
                int var, const Basis B, const Phys P0, const double* __restrict__ geo) {
     static_assert(CPB == tv_cpb(N), "the TV statistics combine blocks of tv_cpb(N) cells");
