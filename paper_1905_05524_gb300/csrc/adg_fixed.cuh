@@ -5,7 +5,7 @@
 // cycles on an SM (19 measured with four busy sub-partitions), a 32 x 32 + 64
 // bit integer multiply-add (IMAD.WIDE) per 1.2 cycles.  A dot product of
 // doubles sum_p a_p b_p is therefore formed from integers: all b of a group
-// (one variable of one cell) share a power-of-two scale taken from the group's
+// (one component of one cell) share a power-of-two scale taken from the group's
 // largest magnitude, likewise the a of one matrix row, and both are held as
 // m 2^s with |m| < 2^58 in two limbs m = h 2^29 + l.
 // The products are exact; h h' and h l' + l h' are summed in two 64-bit
@@ -98,6 +98,15 @@ __device__ __forceinline__ double fx_to(long long a, int e) {
     }
     return __hiloint2double((int)(rh | (s & 0x80000000u)), (int)rl);
 }
+
+// Residuals are sums of derivatives, each with the exponents of its own matrix
+// row and data.  fx_row_shift: bits by which a row of exponent ed, absolute sum
+// `row`, lifts a product above 2^57 in units of the product; the derivative then
+// has exponent X = E + ed - 1022 + shift, and its value, moved down by
+// fx_down(shift, ER, X) bits, that of the sum, ER >= X.  Three derivatives and a
+// source (ER above its own) stay below 2^59.
+__device__ __forceinline__ int fx_row_shift(double row, int ed) { return max((int)(fx_mag(row) >> 20) - ed + 1, 0); }
+__device__ __forceinline__ int fx_down(int shift, int ER, int X) { return min(shift + ER - X, 63); }
 
 // 1/x: the hardware FP32 reciprocal of the mantissa, then one third-order
 // step r (1 + e + e^2), e = 1 - x r (Chebyshev's iteration), whose error e^3 is

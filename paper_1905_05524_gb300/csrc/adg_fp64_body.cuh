@@ -32,29 +32,33 @@ struct FxCfg {
     // per cell, in 8-byte words: q (4) and the fluxes (5) of every space-time
     // node, the source of the time-dependent form (4), u, D/hx, D/hy, the
     // steady source (3), the face values of q-bar, the group magnitudes
-    static constexpr int words(bool tsrc) { return (tsrc ? 13 : 9) * n3 + 9 * n2 + 16 * n + 4; }
+    static constexpr int words(bool tsrc) { return (tsrc ? 13 : 9) * n3 + 9 * n2 + 16 * n + 7; }
     static constexpr size_t smem(bool tsrc) { return ((size_t)cpb * words(tsrc) + n2) * 8; }
 };
 
-// D / hx and D / hy of a cell in fixed point, in shared memory: in registers
-// the two rows of a node (24 at degree 5) leave two resident blocks, and the
-// kernel waits on its own dependent chains (1.55 ms on the 81x81 degree-5 mesh).
+// D / hx and D / hy of a cell in fixed point, each with its own exponent (a
+// common one would cost the longer side of a stretched cell the bits of the
+// aspect ratio), in shared memory: in registers the two rows of a node (24 at
+// degree 5) leave two resident blocks, and the kernel waits on its own dependent
+// chains (1.55 ms on the 81x81 degree-5 mesh).
 template <int N>
 struct FxRows {
     const Limbs *dx, *dy;  // [n][n]
-    int ed;                // exponent of the entries
-    int sh;                // |a row of each times a group| < 2^(57 + sh) in units of the product
+    int ex, ey;            // exponents of the entries
+    int shx, shy;          // |a row times a group| < 2^(57 + sh) in units of the product
     // by all threads tid of the cell; readers wait for a barrier
     __device__ __forceinline__ void make(const Basis& B, Limbs* tab, int tid, double inv_hx, double inv_hy) {
         constexpr int n = N + 1, n2 = n * n;
-        ed = fx_exp(fx_mag(B.Dmax * fmax(inv_hx, inv_hy)));
-        sh = (int)(fx_mag(B.Drow * (inv_hx + inv_hy)) >> 20) - ed + 1;
+        ex = fx_exp(fx_mag(B.Dmax * inv_hx));
+        ey = fx_exp(fx_mag(B.Dmax * inv_hy));
+        shx = fx_row_shift(B.Drow * inv_hx, ex);
+        shy = fx_row_shift(B.Drow * inv_hy, ey);
         dx = tab;
         dy = tab + n2;
         for (int a = tid; a < n2; a += FxCfg<N>::tpc) {
             const double d = B.D[a / n][a % n];
-            tab[a] = fx_split_centred(fx_from(d * inv_hx, ed));
-            tab[n2 + a] = fx_split_centred(fx_from(d * inv_hy, ed));
+            tab[a] = fx_split_centred(fx_from(d * inv_hx, ex));
+            tab[n2 + a] = fx_split_centred(fx_from(d * inv_hy, ey));
         }
     }
 };
@@ -118,8 +122,9 @@ __device__ __forceinline__ FxFlux ns_flux5(const double q[4], const double gx[4]
 // own part of this cell's step.
 //
 // Shared memory of the cell: Q[v][k][node] and F[c][k][node] in limbs; the
-// residual takes Q's place once every gradient is formed.  Groups with a common
-// exponent: q by rho, (rho u, rho v), rho E; the fluxes by momentum and energy.
+// residual takes Q's place once every gradient is formed.  Every component of q
+// and of the fluxes has its own exponent (one for the momenta and one for each
+// kind of flux would hold a component to the largest of its kind only).
 template <int N, bool TSRC = false, bool REC = false>
 __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u, double* __restrict__ rvol,
                                                     double* __restrict__ trace, int cell, bool active, int tid, double dt,
@@ -136,7 +141,7 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
     double* US = sm + NS * n3;
     double* SS = US + 6 * n2;
     double* TQ = SS + 3 * n2;
-    uint32_t* mx = reinterpret_cast<uint32_t*>(TQ + 16 * n);  // magnitudes: q (3), fluxes (2)
+    uint32_t* mx = reinterpret_cast<uint32_t*>(TQ + 16 * n);  // magnitudes: q (4), fluxes (5), sources (z-momentum, 0, 1, 3)
     const double z = yorg + B.xi[j] * P.hy;
     const double g = P.gravity ? P.g : 0.0, gz = g * z;
     const double mu23 = (2.0 / 3.0) * P.mu, kR = P.gm1 * P.kappa * P.invR;
@@ -166,23 +171,16 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
             if (tid == 0) mx[slot] = max(mx[slot], m);
         }
     };
-    // magnitude a group must have for the source S to fit the residual's scale
-    auto smag = [&](double S) {
-        const uint32_t h = fx_mag(S);
-        const int e = (int)(h >> 20) - O.ed + 1023 - O.sh;
-        return h >= 0x7ff00000u ? h : (h < 0x100000u || e <= 0) ? 0u : (uint32_t)e << 20;
-    };
     auto push_q = [&]() {
-        push(0, fx_mag(q[0]));
-        push(1, max(max(fx_mag(q[1]), fx_mag(q[2])), has_src ? smag(Sm[0]) : 0u));
-        push(2, fx_mag(q[3]));
+#pragma unroll
+        for (int v = 0; v < 4; ++v) push(v, fx_mag(q[v]));
     };
-    int EQ[3], EF[2];
+    int EQ[4];
     auto store_q = [&](int slice) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) Q[(v * n + slice) * n2 + node] = fx_limbs(q[v], EQ[v == 0 ? 0 : v == 3 ? 2 : 1]);
+        for (int v = 0; v < 4; ++v) Q[(v * n + slice) * n2 + node] = fx_limbs(q[v], EQ[v]);
     };
-    if (tid < 5) mx[tid] = 0;
+    for (int a = tid; a < 13; a += C::tpc) mx[a] = 0;
     __syncthreads();
     if (!TSRC && has_src) {
         Sm[0] = SS[node];
@@ -190,16 +188,21 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
         Sm[3] = SS[2 * n2 + node];
     }
     push_q();
+    if (has_src) {
+        push(10, fx_mag(Sm[0]));
+        push(11, fx_mag(Sm[1]));
+        push(12, fx_mag(Sm[3]));
+    }
     __syncthreads();
 #pragma unroll
-    for (int a = 0; a < 3; ++a) EQ[a] = fx_exp(mx[a]);
+    for (int v = 0; v < 4; ++v) EQ[v] = fx_exp(mx[v]);
     if (id < n2 && on) {
         store_q(0);
 #pragma unroll
         for (int v = 0; v < 4; ++v) US[v * n2 + node] = q[v];
     }
     __syncthreads();
-    if (tid < 3) mx[tid] = 0;
+    if (tid < 4) mx[tid] = 0;
 
     FxFlux f;
     // sweeps 0..n-1 and the final evaluation r = n; in sweep 0 the iterate is u
@@ -208,16 +211,21 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
     for (int r = 0;; ++r) {
         const int ks = r == 0 ? 0 : k;
         const Limbs* Qk = Q + ks * n2;
-        long long R0;  // d(rho u)/dx + d(rho v)/dy
+        // exponents of the residual (fx_sum_exp of the two derivatives and the source)
+        const int X0 = EQ[1] + O.ex - 1022 + O.shx, Y0 = EQ[2] + O.ey - 1022 + O.shy;
+        int ER[4];
+        ER[0] = max(max(X0, Y0), has_src ? fx_exp(mx[10]) + 1 : 0);
+        const int sx0 = fx_down(O.shx, ER[0], X0), sy0 = fx_down(O.shy, ER[0], Y0);
+        long long R[4];  // -dF/dx - dG/dy + S; the mass flux is the momentum
         f = FxFlux{0.0, 0.0, 0.0, 0.0, 0.0};
         if (r == 0 && k > 0) {
-            FxSum a;
+            FxSum a, b;
 #pragma unroll
             for (int p = 0; p < n; ++p) {
                 a.add(O.dx[i * n + p], Qk[n3 + j * n + p]);
-                a.add(O.dy[j * n + p], Qk[2 * n3 + p * n + i]);
+                b.add(O.dy[j * n + p], Qk[2 * n3 + p * n + i]);
             }
-            R0 = a.value();
+            R[0] = -(a.value() >> sx0) - (b.value() >> sy0);
         } else {
             double gx[4], gy[4];
             {
@@ -228,9 +236,9 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
 #pragma unroll
                     for (int v = 0; v < 4; ++v) a[v].add(d, Qk[v * n3 + j * n + p]);
                 }
-                R0 = a[1].value();
+                R[0] = -(a[1].value() >> sx0);
 #pragma unroll
-                for (int v = 0; v < 4; ++v) gx[v] = fx_to(a[v].value(), EQ[v == 0 ? 0 : v == 3 ? 2 : 1] + O.ed - 2102);
+                for (int v = 0; v < 4; ++v) gx[v] = fx_to(a[v].value(), EQ[v] + O.ex - 2102);
             }
             {
                 FxSum a[4];
@@ -240,40 +248,38 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
 #pragma unroll
                     for (int v = 0; v < 4; ++v) a[v].add(d, Qk[v * n3 + p * n + i]);
                 }
-                R0 += a[2].value();
+                R[0] -= a[2].value() >> sy0;
 #pragma unroll
-                for (int v = 0; v < 4; ++v) gy[v] = fx_to(a[v].value(), EQ[v == 0 ? 0 : v == 3 ? 2 : 1] + O.ed - 2102);
+                for (int v = 0; v < 4; ++v) gy[v] = fx_to(a[v].value(), EQ[v] + O.ey - 2102);
             }
             f = ns_flux5(q, gx, gy, g, gz, pbar, P.gm1, P.mu, mu23, kR);
         }
         if (r == n) break;
         double S2 = Sm[2];
         if (P.gravity) S2 = fma(-g, q[0] - rhobar, S2);
-        uint32_t m3 = max(max(max(fx_mag(f.f1), fx_mag(f.xy)), fx_mag(f.g2)), smag(S2)), m4 = max(fx_mag(f.f3), fx_mag(f.g3));
-        if (has_src) {
-            m3 = max(m3, smag(Sm[1]));
-            m4 = max(m4, smag(Sm[3]));
-        }
-        push(3, m3);
-        push(4, m4);
+        const double fl[5] = {f.f1, f.xy, f.f3, f.g2, f.g3};
+#pragma unroll
+        for (int c = 0; c < 5; ++c) push(4 + c, fx_mag(fl[c]));
+        if (has_src || P.gravity) push(9, fx_mag(S2));
         __syncthreads();
-        EF[0] = fx_exp(mx[3]);
-        EF[1] = fx_exp(mx[4]);
+        int EF[5];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) EF[c] = fx_exp(mx[4 + c]);
+        const int ES2 = has_src || P.gravity ? fx_exp(mx[9]) + 1 : 0;
         if (on && (r > 0 || k == 0)) {
-            Limbs* Fk = F + k * n2 + node;
-            Fk[0] = fx_limbs(f.f1, EF[0]);
-            Fk[n3] = fx_limbs(f.xy, EF[0]);
-            Fk[2 * n3] = fx_limbs(f.f3, EF[1]);
-            Fk[3 * n3] = fx_limbs(f.g2, EF[0]);
-            Fk[4 * n3] = fx_limbs(f.g3, EF[1]);
+#pragma unroll
+            for (int c = 0; c < 5; ++c) F[(c * n + k) * n2 + node] = fx_limbs(fl[c], EF[c]);
         }
         __syncthreads();
-        if (tid < 2) mx[3 + tid] = 0;
-        // residual -dF/dx - dG/dy + S, in Q's place
-        const int ER[3] = {EQ[1] + O.ed - 1022 + O.sh, EF[0] + O.ed - 1022 + O.sh, EF[1] + O.ed - 1022 + O.sh};
-        long long R[4];
+        if (tid < 6) mx[4 + tid] = 0;
+        // residual, in Q's place
         {
-            FxSum a[3];
+            const int dX = O.ex - 1022 + O.shx, dY = O.ey - 1022 + O.shy;
+            const int X[3] = {EF[0] + dX, EF[1] + dX, EF[2] + dX}, Y[3] = {EF[1] + dY, EF[3] + dY, EF[4] + dY};
+            ER[1] = max(max(X[0], Y[0]), has_src ? fx_exp(mx[11]) + 1 : 0);
+            ER[2] = max(max(X[1], Y[1]), ES2);
+            ER[3] = max(max(X[2], Y[2]), has_src ? fx_exp(mx[12]) + 1 : 0);
+            FxSum a[3], b[3];
             const Limbs* Fx = F + ks * n2 + j * n;
             const Limbs* Gy = F + ks * n2 + i;
 #pragma unroll
@@ -285,20 +291,20 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
 #pragma unroll
             for (int p = 0; p < n; ++p) {
                 const Limbs d = O.dy[j * n + p];
-                a[0].add(d, Gy[n3 + p * n]);
-                a[1].add(d, Gy[3 * n3 + p * n]);
-                a[2].add(d, Gy[4 * n3 + p * n]);
+                b[0].add(d, Gy[n3 + p * n]);
+                b[1].add(d, Gy[3 * n3 + p * n]);
+                b[2].add(d, Gy[4 * n3 + p * n]);
             }
-            R[0] = -(R0 >> O.sh);
 #pragma unroll
-            for (int v = 0; v < 3; ++v) R[v + 1] = -(a[v].value() >> O.sh);
+            for (int v = 0; v < 3; ++v)
+                R[v + 1] = -(a[v].value() >> fx_down(O.shx, ER[v + 1], X[v])) - (b[v].value() >> fx_down(O.shy, ER[v + 1], Y[v]));
         }
         if (has_src) {
             R[0] += fx_from(Sm[0], ER[0]);
             R[1] += fx_from(Sm[1], ER[1]);
-            R[3] += fx_from(Sm[3], ER[2]);
+            R[3] += fx_from(Sm[3], ER[3]);
         }
-        if (has_src || P.gravity) R[2] += fx_from(S2, ER[1]);
+        if (has_src || P.gravity) R[2] += fx_from(S2, ER[2]);
         if (on) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) Q[(v * n + k) * n2 + node] = fx_split(R[v]);
@@ -315,15 +321,15 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
             }
 #pragma unroll
             for (int v = 0; v < 4; ++v)
-                q[v] = fma(dt, fx_to(a[v].value(), ER[v == 0 ? 0 : v == 3 ? 2 : 1] + B.KwE - 2102), US[v * n2 + node]);
+                q[v] = fma(dt, fx_to(a[v].value(), ER[v] + B.KwE - 2102), US[v * n2 + node]);
         }
         push_q();
         __syncthreads();
 #pragma unroll
-        for (int a = 0; a < 3; ++a) EQ[a] = fx_exp(mx[a]);
+        for (int v = 0; v < 4; ++v) EQ[v] = fx_exp(mx[v]);
         if (on) store_q(k);
         __syncthreads();
-        if (tid < 3) mx[tid] = 0;
+        if (tid < 4) mx[tid] = 0;
     }
 
     // time averages: slots q (4), F1, XY, F3, G2, G3, then the time-dependent source
