@@ -36,12 +36,14 @@ struct AdjCfg {
     static constexpr int n = F::n, n2 = F::n2, n3 = F::n3;
     static constexpr int cpb = F::cpb, tpc = F::tpc, threads = F::threads;
     static constexpr int resident = 2;  // blocks per SM asked of the register allocator (2 .. 8 within 1%)
-    // per cell, in 8-byte words: the limbs of the iterates q^(0) (one time
-    // slice) and q^(1..n); a work area (fluxes and residual forward; adjoints
+    // per cell, in 8-byte words: the limbs of the iterate q^(0) (one time slice);
+    // the iterates q^(1..n), limbs while a sweep contracts them and doubles in
+    // between (so that the reverse works on the states of the forward, not on
+    // their 58-bit images); a work area (fluxes and residual forward; adjoints
     // of q, of the residual and of the gradients backward); u; D/h and -dt D/h;
     // the adjoints of the face records; iterate exponents and group magnitudes
     static constexpr int work = 8 * n3 > 20 * n2 ? 8 * n3 : 20 * n2;
-    static constexpr int words = 4 * n2 + 4 * n * n3 + work + 4 * n2 + 4 * n2 + 64 * n + 2 * (n + 1) + 4;
+    static constexpr int words = 4 * n2 + 4 * n * n3 + work + 4 * n2 + 4 * n2 + 64 * n + 2 * (n + 1) + 13;
     static constexpr size_t smem = ((size_t)cpb * words + n2 + n) * 8;
 };
 
@@ -260,20 +262,23 @@ k_predictor_adj_fp64(const double* __restrict__ u, const double* __restrict__ la
     Limbs* DT = reinterpret_cast<Limbs*>(US + 4 * n2);    // D/hx, D/hy [n][n]
     Limbs* DM = DT + 2 * n2;                              // -dt D/hx, -dt D/hy
     double* FR = US + 8 * n2;                             // adjoints of the face records [4][16][n]
-    int* EX = reinterpret_cast<int*>(FR + 64 * n);        // exponents of the iterates [n + 1][3 (+1)]
+    int* EX = reinterpret_cast<int*>(FR + 64 * n);        // exponents of the iterates [n + 1][4]
+    // magnitudes; forward: q (4), fluxes (5), sources (z-momentum, 0, 1, 3); reverse, from 13: adjoints of the
+    // gradients along x (4) and y (4), of the iterate (4)
     uint32_t* mx = reinterpret_cast<uint32_t*>(EX + 4 * (n + 1));
     Limbs* K = reinterpret_cast<Limbs*>(sm + (size_t)C::cpb * C::words);  // [n][n], then the row sums [n]
     fx_time_table<N>(K, B);
     for (int a = threadIdx.x; a < n; a += blockDim.x) K[n2 + a] = fx_split_centred(fx_from(B.Kw1[a], B.KwE + 3));
-    const double hmax = B.Dmax * fmax(P.inv_hx, P.inv_hy);
-    const int ed = fx_exp(fx_mag(hmax)), em = fx_exp(fx_mag(hmax * dt));
-    const int sh = (int)(fx_mag(B.Drow * (P.inv_hx + P.inv_hy)) >> 20) - ed + 1;
+    const double dmx = B.Dmax * P.inv_hx, dmy = B.Dmax * P.inv_hy;
+    const int ex = fx_exp(fx_mag(dmx)), ey = fx_exp(fx_mag(dmy));
+    const int emx = fx_exp(fx_mag(dmx * dt)), emy = fx_exp(fx_mag(dmy * dt));
+    const int shx = fx_row_shift(B.Drow * P.inv_hx, ex), shy = fx_row_shift(B.Drow * P.inv_hy, ey);
     for (int a = tid; a < n2; a += C::tpc) {
         const double dx = B.D[a / n][a % n] * P.inv_hx, dy = B.D[a / n][a % n] * P.inv_hy;
-        DT[a] = fx_split_centred(fx_from(dx, ed));
-        DT[n2 + a] = fx_split_centred(fx_from(dy, ed));
-        DM[a] = fx_split_centred(fx_from(-dt * dx, em));
-        DM[n2 + a] = fx_split_centred(fx_from(-dt * dy, em));
+        DT[a] = fx_split_centred(fx_from(dx, ex));
+        DT[n2 + a] = fx_split_centred(fx_from(dy, ey));
+        DM[a] = fx_split_centred(fx_from(-dt * dx, emx));
+        DM[n2 + a] = fx_split_centred(fx_from(-dt * dy, emy));
     }
     const int cell_raw = blockIdx.x * C::cpb + cl;
     const bool active = cell_raw < cells;
@@ -297,14 +302,10 @@ k_predictor_adj_fp64(const double* __restrict__ u, const double* __restrict__ la
             if (tid == 0) mx[slot] = max(mx[slot], m);
         }
     };
-    auto smag = [&](double S) {
-        const uint32_t h = fx_mag(S);
-        const int e = (int)(h >> 20) - ed + 1023 - sh;
-        return h >= 0x7ff00000u ? h : (h < 0x100000u || e <= 0) ? 0u : (uint32_t)e << 20;
-    };
-    auto gv = [](int v) { return v == 0 ? 0 : v == 3 ? 2 : 1; };
-    // gradients at this node from the limbs of an iterate's time slice (plane stride ps)
-    auto gradients = [&](const Limbs* Qk, int ps, const int* eq, double gx[4], double gy[4], long long& R0) {
+    // gradients at this node from the limbs of an iterate's time slice (plane stride ps); mx0, my0: the
+    // derivatives of the mass flux as they come
+    auto gradients = [&](const Limbs* Qk, int ps, const int* eq, double gx[4], double gy[4], long long& mx0,
+                         long long& my0) {
         FxSum a[4], b[4];
 #pragma unroll
         for (int p = 0; p < n; ++p) {
@@ -312,80 +313,91 @@ k_predictor_adj_fp64(const double* __restrict__ u, const double* __restrict__ la
 #pragma unroll
             for (int v = 0; v < 4; ++v) a[v].add(d, Qk[v * ps + j * n + p]);
         }
-        R0 = a[1].value();
+        mx0 = a[1].value();
 #pragma unroll
-        for (int v = 0; v < 4; ++v) gx[v] = fx_to(a[v].value(), eq[gv(v)] + ed - 2102);
+        for (int v = 0; v < 4; ++v) gx[v] = fx_to(a[v].value(), eq[v] + ex - 2102);
 #pragma unroll
         for (int p = 0; p < n; ++p) {
             const Limbs d = DT[n2 + j * n + p];
 #pragma unroll
             for (int v = 0; v < 4; ++v) b[v].add(d, Qk[v * ps + p * n + i]);
         }
-        R0 += b[2].value();
+        my0 = b[2].value();
 #pragma unroll
-        for (int v = 0; v < 4; ++v) gy[v] = fx_to(b[v].value(), eq[gv(v)] + ed - 2102);
+        for (int v = 0; v < 4; ++v) gy[v] = fx_to(b[v].value(), eq[v] + ey - 2102);
     };
 
     // ---------------- forward recompute of the iterates (as k_predictor_fp64)
     double q[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) q[v] = u[(size_t)cell * SL + v * n2 + node];
-    if (tid < 8) mx[tid] = 0;
+    for (int a = tid; a < 25; a += C::tpc) mx[a] = 0;
     __syncthreads();
     auto push_q = [&]() {
-        push(0, fx_mag(q[0]));
-        push(1, max(max(fx_mag(q[1]), fx_mag(q[2])), has_src ? smag(Sm[0]) : 0u));
-        push(2, fx_mag(q[3]));
+#pragma unroll
+        for (int v = 0; v < 4; ++v) push(v, fx_mag(q[v]));
     };
     push_q();
+    if (has_src) {
+        push(10, fx_mag(Sm[0]));
+        push(11, fx_mag(Sm[1]));
+        push(12, fx_mag(Sm[3]));
+    }
     __syncthreads();
-    if (tid < 3) EX[tid] = fx_exp(mx[tid]);
+    if (tid < 4) EX[tid] = fx_exp(mx[tid]);
     if (on && k == 0) {
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
-            U0[v * n2 + node] = fx_limbs(q[v], fx_exp(mx[gv(v)]));
+            U0[v * n2 + node] = fx_limbs(q[v], fx_exp(mx[v]));
             US[v * n2 + node] = q[v];
         }
     }
     __syncthreads();
-    if (tid < 3) mx[tid] = 0;
+    if (tid < 4) mx[tid] = 0;
 #pragma unroll 1
     for (int r = 0; r < n; ++r) {
         const int ks = r == 0 ? 0 : k, ps = r == 0 ? n2 : n3;
         const Limbs* Qk = r == 0 ? U0 : IT + (r - 1) * 4 * n3 + k * n2;
-        int eq[3];
+        int eq[4];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) eq[a] = EX[4 * r + a];
+        for (int v = 0; v < 4; ++v) eq[v] = EX[4 * r + v];
         double gx[4], gy[4];
-        long long R0;
-        gradients(Qk, ps, eq, gx, gy, R0);
+        long long R0, R0y;
+        gradients(Qk, ps, eq, gx, gy, R0, R0y);
         FxFlux f{0.0, 0.0, 0.0, 0.0, 0.0};
         if (r > 0 || k == 0) f = ns_flux5(q, gx, gy, g, gz, pbar, P.gm1, P.mu, mu23, kR);
         double S2 = Sm[2];
         if (P.gravity) S2 = fma(-g, q[0] - rhobar, S2);
-        uint32_t m3 = max(max(max(fx_mag(f.f1), fx_mag(f.xy)), fx_mag(f.g2)), smag(S2)), m4 = max(fx_mag(f.f3), fx_mag(f.g3));
-        if (has_src) {
-            m3 = max(m3, smag(Sm[1]));
-            m4 = max(m4, smag(Sm[3]));
-        }
-        push(3, m3);
-        push(4, m4);
+        const double fl[5] = {f.f1, f.xy, f.f3, f.g2, f.g3};
+#pragma unroll
+        for (int c = 0; c < 5; ++c) push(4 + c, fx_mag(fl[c]));
+        if (has_src || P.gravity) push(9, fx_mag(S2));
         __syncthreads();
-        const int EF[2] = {fx_exp(mx[3]), fx_exp(mx[4])};
+        int EF[5], ER[4];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) EF[c] = fx_exp(mx[4 + c]);
+        const int ES2 = has_src || P.gravity ? fx_exp(mx[9]) + 1 : 0;
         if (on && (r > 0 || k == 0)) {
-            Limbs* Fk = W + k * n2 + node;
-            Fk[0] = fx_limbs(f.f1, EF[0]);
-            Fk[n3] = fx_limbs(f.xy, EF[0]);
-            Fk[2 * n3] = fx_limbs(f.f3, EF[1]);
-            Fk[3 * n3] = fx_limbs(f.g2, EF[0]);
-            Fk[4 * n3] = fx_limbs(f.g3, EF[1]);
+#pragma unroll
+            for (int c = 0; c < 5; ++c) W[(c * n + k) * n2 + node] = fx_limbs(fl[c], EF[c]);
+        }
+        if (on && r > 0) {  // every gradient is formed: the iterate itself in place of its limbs
+            double* Qd = reinterpret_cast<double*>(IT + (r - 1) * 4 * n3);
+#pragma unroll
+            for (int v = 0; v < 4; ++v) Qd[(v * n + k) * n2 + node] = q[v];
         }
         __syncthreads();
-        if (tid < 2) mx[3 + tid] = 0;
-        const int ER[3] = {eq[1] + ed - 1022 + sh, EF[0] + ed - 1022 + sh, EF[1] + ed - 1022 + sh};
+        if (tid < 6) mx[4 + tid] = 0;
         Limbs* Rn = IT + r * 4 * n3;  // the next iterate's place holds the residual first
         {
-            FxSum a[3];
+            const int dX = ex - 1022 + shx, dY = ey - 1022 + shy;
+            const int X[4] = {eq[1] + dX, EF[0] + dX, EF[1] + dX, EF[2] + dX};
+            const int Y[4] = {eq[2] + dY, EF[1] + dY, EF[3] + dY, EF[4] + dY};
+            const int ES[4] = {has_src ? fx_exp(mx[10]) + 1 : 0, has_src ? fx_exp(mx[11]) + 1 : 0, ES2,
+                               has_src ? fx_exp(mx[12]) + 1 : 0};
+#pragma unroll
+            for (int v = 0; v < 4; ++v) ER[v] = max(max(X[v], Y[v]), ES[v]);
+            FxSum a[3], b[3];
             const Limbs* Fx = W + ks * n2 + j * n;
             const Limbs* Gy = W + ks * n2 + i;
 #pragma unroll
@@ -397,20 +409,21 @@ k_predictor_adj_fp64(const double* __restrict__ u, const double* __restrict__ la
 #pragma unroll
             for (int p = 0; p < n; ++p) {
                 const Limbs d = DT[n2 + j * n + p];
-                a[0].add(d, Gy[n3 + p * n]);
-                a[1].add(d, Gy[3 * n3 + p * n]);
-                a[2].add(d, Gy[4 * n3 + p * n]);
+                b[0].add(d, Gy[n3 + p * n]);
+                b[1].add(d, Gy[3 * n3 + p * n]);
+                b[2].add(d, Gy[4 * n3 + p * n]);
             }
             long long R[4];
-            R[0] = -(R0 >> sh);
+            R[0] = -(R0 >> fx_down(shx, ER[0], X[0])) - (R0y >> fx_down(shy, ER[0], Y[0]));
 #pragma unroll
-            for (int v = 0; v < 3; ++v) R[v + 1] = -(a[v].value() >> sh);
+            for (int v = 1; v < 4; ++v)
+                R[v] = -(a[v - 1].value() >> fx_down(shx, ER[v], X[v])) - (b[v - 1].value() >> fx_down(shy, ER[v], Y[v]));
             if (has_src) {
                 R[0] += fx_from(Sm[0], ER[0]);
                 R[1] += fx_from(Sm[1], ER[1]);
-                R[3] += fx_from(Sm[3], ER[2]);
+                R[3] += fx_from(Sm[3], ER[3]);
             }
-            if (has_src || P.gravity) R[2] += fx_from(S2, ER[1]);
+            if (has_src || P.gravity) R[2] += fx_from(S2, ER[2]);
             if (on) {
 #pragma unroll
                 for (int v = 0; v < 4; ++v) Rn[(v * n + k) * n2 + node] = fx_split(R[v]);
@@ -426,17 +439,17 @@ k_predictor_adj_fp64(const double* __restrict__ u, const double* __restrict__ la
                 for (int v = 0; v < 4; ++v) a[v].add(d, Rn[(v * n + kk) * n2 + node]);
             }
 #pragma unroll
-            for (int v = 0; v < 4; ++v) q[v] = fma(dt, fx_to(a[v].value(), ER[gv(v)] + B.KwE - 2102), US[v * n2 + node]);
+            for (int v = 0; v < 4; ++v) q[v] = fma(dt, fx_to(a[v].value(), ER[v] + B.KwE - 2102), US[v * n2 + node]);
         }
         push_q();
         __syncthreads();
-        if (tid < 3) EX[4 * (r + 1) + tid] = fx_exp(mx[tid]);
+        if (tid < 4) EX[4 * (r + 1) + tid] = fx_exp(mx[tid]);
         if (on) {
 #pragma unroll
-            for (int v = 0; v < 4; ++v) Rn[(v * n + k) * n2 + node] = fx_limbs(q[v], fx_exp(mx[gv(v)]));
+            for (int v = 0; v < 4; ++v) Rn[(v * n + k) * n2 + node] = fx_limbs(q[v], fx_exp(mx[v]));
         }
         __syncthreads();
-        if (tid < 3) mx[tid] = 0;
+        if (tid < 4) mx[tid] = 0;
     }
 
     // ---------------- reverse of the epilogue
@@ -494,40 +507,44 @@ k_predictor_adj_fp64(const double* __restrict__ u, const double* __restrict__ la
             gyb[v] = wk * Wd[(16 + v) * n2 + node];
         }
         double gx[4], gy[4];
-        long long R0;
-        gradients(IT + (n - 1) * 4 * n3 + k * n2, n3, EX + 4 * n, gx, gy, R0);
+        long long R0, R0y;
+        gradients(IT + (n - 1) * 4 * n3 + k * n2, n3, EX + 4 * n, gx, gy, R0, R0y);
         ns_flux5_adj(q, gx, gy, g, gz, P.gm1, P.mu, mu23, kR, Fb, Gb, wk * dt * lc[2 * n2 + node], qb, gxb, gyb);
     }
     // fold the gradient adjoints back: q_bar(j,p) += (1/h) sum_i' D[i'][p] qx_bar(j,i'); slices: time nodes that hold data
     auto fold = [&](bool mine) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) push(v, mine ? max(fx_mag(gxb[v]), fx_mag(gyb[v])) : 0u);
+        for (int v = 0; v < 4; ++v) {
+            push(13 + v, mine ? fx_mag(gxb[v]) : 0u);
+            push(17 + v, mine ? fx_mag(gyb[v]) : 0u);
+        }
         __syncthreads();
-        int E[4];
+        int E[8];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) E[v] = fx_exp(mx[v]);
+        for (int v = 0; v < 8; ++v) E[v] = fx_exp(mx[13 + v]);
         if (on && mine) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 W[(v * n + k) * n2 + node] = fx_limbs(gxb[v], E[v]);
-                W[((4 + v) * n + k) * n2 + node] = fx_limbs(gyb[v], E[v]);
+                W[((4 + v) * n + k) * n2 + node] = fx_limbs(gyb[v], E[4 + v]);
             }
         }
         __syncthreads();
-        if (tid < 4) mx[tid] = 0;
+        if (tid < 8) mx[13 + tid] = 0;
         if (!mine) return;
-        FxSum a[4];
+        FxSum a[4], b[4];
 #pragma unroll
         for (int p = 0; p < n; ++p) {
             const Limbs dx = DT[p * n + i], dy = DT[n2 + p * n + j];
 #pragma unroll
             for (int v = 0; v < 4; ++v) {
                 a[v].add(dx, W[(v * n + k) * n2 + j * n + p]);
-                a[v].add(dy, W[((4 + v) * n + k) * n2 + p * n + i]);
+                b[v].add(dy, W[((4 + v) * n + k) * n2 + p * n + i]);
             }
         }
 #pragma unroll
-        for (int v = 0; v < 4; ++v) qb[v] += fx_to(a[v].value(), E[v] + ed - 2102);
+        for (int v = 0; v < 4; ++v)
+            qb[v] += fx_to(a[v].value(), E[v] + ex - 2102) + fx_to(b[v].value(), E[4 + v] + ey - 2102);
     };
     fold(true);
 
@@ -539,18 +556,33 @@ k_predictor_adj_fp64(const double* __restrict__ u, const double* __restrict__ la
 #pragma unroll
         for (int v = 0; v < 4; ++v) {
             ub[v] += qb[v];
-            push(4 + v, fx_mag(qb[v]));
+            push(21 + v, fx_mag(qb[v]));
         }
         __syncthreads();  // also: every thread has folded, W is free
         int E[4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) E[v] = fx_exp(mx[4 + v]);
+        for (int v = 0; v < 4; ++v) E[v] = fx_exp(mx[21 + v]);
         if (on) {
 #pragma unroll
             for (int v = 0; v < 4; ++v) W[(v * n + k) * n2 + node] = fx_limbs(qb[v], E[v]);
         }
+        // the state of this sweep's evaluation: the iterate, and its limbs in its place for the gradients
+        const int* eq = EX + 4 * (r - 1);
+        if (r == 1) {
+#pragma unroll
+            for (int v = 0; v < 4; ++v) q[v] = US[v * n2 + node];
+        } else {
+            Limbs* Qr = IT + (r - 2) * 4 * n3 + k * n2 + node;
+#pragma unroll
+            for (int v = 0; v < 4; ++v) q[v] = reinterpret_cast<const double*>(Qr)[v * n3];
+            __syncwarp();  // the lanes that repeat the last node have read it
+            if (on) {
+#pragma unroll
+                for (int v = 0; v < 4; ++v) Qr[v * n3] = fx_limbs(q[v], eq[v]);
+            }
+        }
         __syncthreads();
-        if (tid < 4) mx[4 + tid] = 0;
+        if (tid < 4) mx[21 + tid] = 0;
         double R2 = 0.0;
         if (mine) {
             const int eK = r > 1 ? B.KwE : B.KwE + 3;
@@ -587,21 +619,15 @@ k_predictor_adj_fp64(const double* __restrict__ u, const double* __restrict__ la
                 }
 #pragma unroll
                 for (int v = 0; v < 4; ++v) {
-                    Fb[v] = fx_to(a[v].value(), E[v] + em - 2102);
-                    Gb[v] = fx_to(b[v].value(), E[v] + em - 2102);
+                    Fb[v] = fx_to(a[v].value(), E[v] + emx - 2102);
+                    Gb[v] = fx_to(b[v].value(), E[v] + emy - 2102);
                 }
             }
             const Limbs* Qk = r == 1 ? U0 : IT + (r - 2) * 4 * n3 + k * n2;
             const int ps = r == 1 ? n2 : n3;
-            const int* eq = EX + 4 * (r - 1);
             double gx[4], gy[4];
-            long long R0;
-            gradients(Qk, ps, eq, gx, gy, R0);
-#pragma unroll
-            for (int v = 0; v < 4; ++v) {
-                const Limbs o = Qk[v * ps + node];
-                q[v] = r == 1 ? US[v * n2 + node] : fx_to((long long)o.h * (1ll << 29) + o.l, eq[gv(v)] - 1080);
-            }
+            long long R0, R0y;
+            gradients(Qk, ps, eq, gx, gy, R0, R0y);
             ns_flux5_adj(q, gx, gy, g, gz, P.gm1, P.mu, mu23, kR, Fb, Gb, dt * R2, qb, gxb, gyb);
         }
         fold(mine);

@@ -1,5 +1,5 @@
 """Cells 2^24 times longer along one axis (l) than along the other (s): the FP64
-step keeps the derivatives along the long side to their own
+step and its adjoint keep the derivatives along the long side to their own
 accuracy, not to that of the short side's (2^24 times larger) entries of D / h.
 
 A flow along s, v_s = f(x_s) g(x_l), over uniform density and pressure leaves
@@ -11,7 +11,8 @@ with L the largest row or column sum of |D|, W that of the weak volume term and
 of the lifting, per unit cell length, the two operands of each gradient
 (d(rho v) and v d(rho)) give (2 + 4/3) mu U L W / (h_l h_s), the pressure, which
 the long derivative of the normal flux cancels, p W / h_l.  Two implementations
-differ by at most twice that.
+differ by at most twice that.  The adjoint is the transpose: an adjoint of m_l
+alone gives one of m_s, with (gamma - 1) U for p.
 """
 import numpy as np
 import pytest
@@ -20,6 +21,7 @@ import torch
 from oracle.basis import Basis
 from paper_1905_05524_gb300.solver import Mesh, MeshConfig
 from tests.oracle_bridge import oracle_for
+from tests.test_gpu_adjoint import gpu_adjoint, oracle_adjoint
 
 pytestmark = pytest.mark.gpu
 
@@ -65,4 +67,21 @@ def test_step_2d(degree, long):
     m.set_state(u0.cuda().contiguous())
     m.step(DT)
     check(m.get_state().cpu()[:, 1 + long], o.step(u0, DT)[:, 1 + long], bound(degree, 1.0))
+    m.close()
+
+
+@pytest.mark.parametrize("long", [0, 1])
+@pytest.mark.parametrize("degree", [1, 2, 3, 4, 5])
+def test_adjoint_2d(degree, long):
+    H = [1.0, 1.0]
+    H[long] = LONG
+    cfg = MeshConfig(degree=degree, nx=2, ny=2, Lx=2.0 * H[0], Ly=2.0 * H[1], mu=MU)
+    o = oracle_for(cfg)
+    u0 = flow((o.X, o.Y), long, 1 - long, H, 2)
+    lam = torch.zeros_like(u0)
+    lam[:, 1 + long] = 2.0 * torch.rand(lam[:, 0].shape, generator=torch.Generator().manual_seed(degree),
+                                        dtype=torch.float64) - 1.0
+    m = Mesh(cfg)
+    got = gpu_adjoint(m, DT, u0.cuda().contiguous(), lam.cuda().contiguous()).cpu()
+    check(got[:, 2 - long], oracle_adjoint(o, DT, u0, lam)[:, 2 - long], bound(degree, 0.4 * 1.5))
     m.close()
