@@ -179,8 +179,8 @@ struct Fx3Cfg {
     // degree 4 (13^3) 2134 with 1, 2152 with 2
     static constexpr int resident = N == 1 ? 3 : N == 4 ? 1 : 5;
     // per cell, in 8-byte words: q (5) and the fluxes (9) of every space-time
-    // node, u, D/h, the face values of q-bar, the group magnitudes
-    static constexpr int words = 14 * n4 + 5 * n3 + 3 * n2 + 30 * n2 + 4;
+    // node, u, D/h, the face values of q-bar, the magnitudes
+    static constexpr int words = 14 * n4 + 5 * n3 + 3 * n2 + 30 * n2 + 8;
     static constexpr size_t smem = ((size_t)cpb * words + n2) * 8;
 };
 
@@ -249,13 +249,20 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
     double* US = base + 14 * n4;                // [5][n3]
     Limbs* DT = reinterpret_cast<Limbs*>(US + 5 * n3);  // [3][n][n]
     double* TQ = US + 5 * n3 + 3 * n2;          // [6][5][n2]
-    uint32_t* mx = reinterpret_cast<uint32_t*>(TQ + 30 * n2);
+    uint32_t* mx = reinterpret_cast<uint32_t*>(TQ + 30 * n2);  // magnitudes: q (5), fluxes (9), the source
     Limbs* K = reinterpret_cast<Limbs*>(sm + (size_t)C::cpb * C::words);
     for (int a = threadIdx.x; a < n2; a += blockDim.x) K[a] = Limbs{B.KwH[a / n][a % n], B.KwL[a / n][a % n]};
-    const int ed = fx_exp(fx_mag(B.Dmax * fmax(P.inv_h[0], fmax(P.inv_h[1], P.inv_h[2]))));
-    const int sh = (int)(fx_mag(B.Drow * (P.inv_h[0] + P.inv_h[1] + P.inv_h[2])) >> 20) - ed + 1;
+    int ed[3], sh[3];  // of each direction's entries (FxRows of the 2D predictor)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        ed[b] = fx_exp(fx_mag(B.Dmax * P.inv_h[b]));
+        sh[b] = fx_row_shift(B.Drow * P.inv_h[b], ed[b]);
+    }
     for (int a = tid; a < 3 * n2; a += C::tpc)
-        if (on) DT[a] = fx_split_centred(fx_from(B.D[a % n2 / n][a % n] * P.inv_h[a / n2], ed));
+        if (on) {
+            const int b = a / n2;
+            DT[a] = fx_split_centred(fx_from(B.D[a % n2 / n][a % n] * P.inv_h[b], b == 0 ? ed[0] : b == 1 ? ed[1] : ed[2]));
+        }
     const double gg = P.gravity ? P.g : 0.0, mu23 = (2.0 / 3.0) * P.mu, kR = P.gm1 * P.kappa * P.invR;
 
     // largest magnitude of a group over the cell's threads: a warp reduction and
@@ -289,30 +296,28 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
         double q[5];
 #pragma unroll
         for (int v = 0; v < 5; ++v) q[v] = u[(size_t)cell * SL + v * n3 + node];
-        int EQ[3] = {0, 0, 0}, EF[2];
+        int EQ[5];
         auto push_q = [&]() {
-            push(0, fx_mag(q[0]));
-            push(1, max(max(fx_mag(q[1]), fx_mag(q[2])), fx_mag(q[3])));
-            push(2, fx_mag(q[4]));
+#pragma unroll
+            for (int v = 0; v < 5; ++v) push(v, fx_mag(q[v]));
         };
-        auto eq = [&](int v) { return EQ[v == 0 ? 0 : v == 4 ? 2 : 1]; };
         auto store_q = [&](int slice) {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) Q[(v * n + slice) * n3 + node] = fx_limbs(q[v], eq(v));
+            for (int v = 0; v < 5; ++v) Q[(v * n + slice) * n3 + node] = fx_limbs(q[v], EQ[v]);
         };
-        if (tid < 5) mx[tid] = 0;
+        if (tid < 15) mx[tid] = 0;
         __syncthreads();
         push_q();
         __syncthreads();
 #pragma unroll
-        for (int a = 0; a < 3; ++a) EQ[a] = fx_exp(mx[a]);
+        for (int v = 0; v < 5; ++v) EQ[v] = fx_exp(mx[v]);
         if (id < n3 && on) {
             store_q(0);
 #pragma unroll
             for (int v = 0; v < 5; ++v) US[v * n3 + node] = q[v];
         }
         __syncthreads();
-        if (tid < 3) mx[tid] = 0;
+        if (tid < 5) mx[tid] = 0;
 
         Fx3Flux f;
         // sweeps 0..n-1 and the final evaluation r = n; in sweep 0 the iterate is
@@ -321,22 +326,25 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
         for (int r = 0;; ++r) {
             const int ks = r == 0 ? 0 : k;
             const Limbs* Qk = Q + ks * n3;
-            long long R0;  // divergence of the momentum
+            int ER[5];  // exponents of the residual: the largest of its derivatives' and the source's
+            ER[0] = max(EQ[1] + ed[0] + sh[0], max(EQ[2] + ed[1] + sh[1], EQ[3] + ed[2] + sh[2])) - 1022;
+            long long R[5];  // -div F + S; the mass flux is the momentum
+            R[0] = 0;
 #pragma unroll
             for (int a = 0; a < 6; ++a) f.t[a] = 0.0;
             f.e[0] = f.e[1] = f.e[2] = 0.0;
             if (r == 0 && k > 0) {
-                FxSum a;
 #pragma unroll
-                for (int p = 0; p < n; ++p) {
-                    a.add(Dx[p], Qk[n4 + ox + p]);
-                    a.add(Dy[p], Qk[2 * n4 + oy + p * n]);
-                    a.add(Dz[p], Qk[3 * n4 + oz + p * n2]);
+                for (int b = 0; b < 3; ++b) {
+                    const Limbs* D = b == 0 ? Dx : b == 1 ? Dy : Dz;
+                    const Limbs* L = Qk + (1 + b) * n4 + (b == 0 ? ox : b == 1 ? oy : oz);
+                    FxSum a;
+#pragma unroll
+                    for (int p = 0; p < n; ++p) a.add(D[p], L[p * (b == 0 ? 1 : b == 1 ? n : n2)]);
+                    R[0] -= a.value() >> fx_down(sh[b], ER[0], EQ[1 + b] + ed[b] + sh[b] - 1022);
                 }
-                R0 = a.value();
             } else {
                 double g[3][5];
-                R0 = 0;
 #pragma unroll
                 for (int b = 0; b < 3; ++b) {
                     const Limbs* D = b == 0 ? Dx : b == 1 ? Dy : Dz;
@@ -348,64 +356,57 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
 #pragma unroll
                         for (int v = 0; v < 5; ++v) a[v].add(d, L[v * n4 + p * (b == 0 ? 1 : b == 1 ? n : n2)]);
                     }
-                    R0 += a[1 + b].value();
+                    R[0] -= a[1 + b].value() >> fx_down(sh[b], ER[0], EQ[1 + b] + ed[b] + sh[b] - 1022);
 #pragma unroll
-                    for (int v = 0; v < 5; ++v) g[b][v] = fx_to(a[v].value(), eq(v) + ed - 2102);
+                    for (int v = 0; v < 5; ++v) g[b][v] = fx_to(a[v].value(), EQ[v] + ed[b] - 2102);
                 }
                 f = ns_flux9(q, g, gg, gz, pbar, P.gm1, P.mu, mu23, kR);
             }
             if (r == n) break;
             const double S = P.gravity ? -gg * (q[0] - rhobar) : 0.0;
-            uint32_t m3 = 0, m4 = 0;
-            if (P.gravity) {  // magnitude the momentum group must have for S to fit the residual's scale
-                const uint32_t hs = fx_mag(S);
-                const int e = (int)(hs >> 20) - ed + 1023 - sh;
-                m3 = hs >= 0x7ff00000u ? hs : (hs < 0x100000u || e <= 0) ? 0u : (uint32_t)e << 20;
-            }
+            const double fl[9] = {f.t[0], f.t[1], f.t[2], f.t[3], f.t[4], f.t[5], f.e[0], f.e[1], f.e[2]};
 #pragma unroll
-            for (int a = 0; a < 6; ++a) m3 = max(m3, fx_mag(f.t[a]));
-#pragma unroll
-            for (int a = 0; a < 3; ++a) m4 = max(m4, fx_mag(f.e[a]));
-            push(3, m3);
-            push(4, m4);
+            for (int c = 0; c < 9; ++c) push(5 + c, fx_mag(fl[c]));
+            if (P.gravity) push(14, fx_mag(S));
             __syncthreads();
-            EF[0] = fx_exp(mx[3]);
-            EF[1] = fx_exp(mx[4]);
+            int EF[9];
+#pragma unroll
+            for (int c = 0; c < 9; ++c) EF[c] = fx_exp(mx[5 + c]);
+            const int ES = P.gravity ? fx_exp(mx[14]) + 1 : 0;
             if (on && (r > 0 || k == 0)) {
-                Limbs* Fk = F + k * n3 + node;
 #pragma unroll
-                for (int a = 0; a < 6; ++a) Fk[a * n4] = fx_limbs(f.t[a], EF[0]);
-#pragma unroll
-                for (int a = 0; a < 3; ++a) Fk[(6 + a) * n4] = fx_limbs(f.e[a], EF[1]);
+                for (int c = 0; c < 9; ++c) F[(c * n + k) * n3 + node] = fx_limbs(fl[c], EF[c]);
             }
             __syncthreads();
-            if (tid < 2) mx[3 + tid] = 0;
-            // residual -div F + S, in Q's place
-            const int ER[3] = {EQ[1] + ed - 1022 + sh, EF[0] + ed - 1022 + sh, EF[1] + ed - 1022 + sh};
-            {
+            if (tid < 10) mx[5 + tid] = 0;
+            // residual, in Q's place; component v's flux in direction b
+            auto fc = [](int v, int b) { return v < 4 ? fx3_t(v - 1, b) : 6 + b; };
+#pragma unroll
+            for (int v = 1; v < 5; ++v) {
+                ER[v] = v == 3 ? ES : 0;
+#pragma unroll
+                for (int b = 0; b < 3; ++b) ER[v] = max(ER[v], EF[fc(v, b)] + ed[b] + sh[b] - 1022);
+                R[v] = 0;
+            }
+#pragma unroll
+            for (int b = 0; b < 3; ++b) {
+                const Limbs* D = b == 0 ? Dx : b == 1 ? Dy : Dz;
+                const Limbs* L = F + ks * n3 + (b == 0 ? ox : b == 1 ? oy : oz);
                 FxSum a[4];
 #pragma unroll
-                for (int b = 0; b < 3; ++b) {
-                    const Limbs* D = b == 0 ? Dx : b == 1 ? Dy : Dz;
-                    const Limbs* L = F + ks * n3 + (b == 0 ? ox : b == 1 ? oy : oz);
+                for (int p = 0; p < n; ++p) {
+                    const Limbs d = D[p];
 #pragma unroll
-                    for (int p = 0; p < n; ++p) {
-                        const Limbs d = D[p];
-                        const int o = p * (b == 0 ? 1 : b == 1 ? n : n2);
-#pragma unroll
-                        for (int v = 0; v < 3; ++v) a[v].add(d, L[fx3_t(v, b) * n4 + o]);
-                        a[3].add(d, L[(6 + b) * n4 + o]);
-                    }
+                    for (int v = 1; v < 5; ++v) a[v - 1].add(d, L[fc(v, b) * n4 + p * (b == 0 ? 1 : b == 1 ? n : n2)]);
                 }
-                long long R[5];
-                R[0] = -(R0 >> sh);
 #pragma unroll
-                for (int v = 0; v < 4; ++v) R[v + 1] = -(a[v].value() >> sh);
-                if (P.gravity) R[3] += fx_from(S, ER[1]);
-                if (on) {
+                for (int v = 1; v < 5; ++v)
+                    R[v] -= a[v - 1].value() >> fx_down(sh[b], ER[v], EF[fc(v, b)] + ed[b] + sh[b] - 1022);
+            }
+            if (P.gravity) R[3] += fx_from(S, ER[3]);
+            if (on) {
 #pragma unroll
-                    for (int v = 0; v < 5; ++v) Q[(v * n + k) * n3 + node] = fx_split(R[v]);
-                }
+                for (int v = 0; v < 5; ++v) Q[(v * n + k) * n3 + node] = fx_split(R[v]);
             }
             __syncthreads();
             {  // time contraction: this thread's time node of the next iterate
@@ -418,15 +419,15 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
                 }
 #pragma unroll
                 for (int v = 0; v < 5; ++v)
-                    q[v] = fma(dt, fx_to(a[v].value(), ER[v == 0 ? 0 : v == 4 ? 2 : 1] + B.KwE - 2102), US[v * n3 + node]);
+                    q[v] = fma(dt, fx_to(a[v].value(), ER[v] + B.KwE - 2102), US[v * n3 + node]);
             }
             push_q();
             __syncthreads();
 #pragma unroll
-            for (int a = 0; a < 3; ++a) EQ[a] = fx_exp(mx[a]);
+            for (int v = 0; v < 5; ++v) EQ[v] = fx_exp(mx[v]);
             if (on) store_q(k);
             __syncthreads();
-            if (tid < 3) mx[tid] = 0;
+            if (tid < 5) mx[tid] = 0;
         }
 
         // time averages: slots q (5), t (6), e (3)

@@ -19,8 +19,9 @@ import pytest
 import torch
 
 from oracle.basis import Basis
-from paper_1905_05524_gb300.solver import Mesh, MeshConfig
+from paper_1905_05524_gb300.solver import Mesh, Mesh3, Mesh3Config, MeshConfig
 from tests.oracle_bridge import oracle_for
+from tests.test_gpu_3d import oracle3
 from tests.test_gpu_adjoint import gpu_adjoint, oracle_adjoint
 
 pytestmark = pytest.mark.gpu
@@ -65,6 +66,21 @@ def test_step_2d(degree, long):
     u0 = flow((o.X, o.Y), long, 1 - long, H, 2)
     m = Mesh(cfg)
     m.set_state(u0.cuda().contiguous())
+    m.step(DT)
+    check(m.get_state().cpu()[:, 1 + long], o.step(u0, DT)[:, 1 + long], bound(degree, 1.0))
+    m.close()
+
+
+@pytest.mark.parametrize("long", [0, 1, 2])
+@pytest.mark.parametrize("degree", [1, 2, 3, 4])
+def test_step_3d(degree, long):
+    H = [1.0, 1.0, 1.0]
+    H[long] = LONG
+    cfg = Mesh3Config(degree=degree, nx=2, ny=2, nz=2, Lx=2.0 * H[0], Ly=2.0 * H[1], Lz=2.0 * H[2], mu=MU)
+    o = oracle3(cfg)
+    u0 = flow((o.X, o.Y, o.Z), long, (long + 1) % 3, H, 3)
+    m = Mesh3(cfg)
+    m.set_state(u0)
     m.step(DT)
     check(m.get_state().cpu()[:, 1 + long], o.step(u0, DT)[:, 1 + long], bound(degree, 1.0))
     m.close()
