@@ -33,11 +33,13 @@ __device__ __forceinline__ float tv_node_z(int iy, int j, const BasisF& B, const
 }
 
 // T (p0/p)^(R/cp), for p within 0.6 p0 .. 1.65 p0 (the lowest 4 km) as
-// T exp(-(R/cp) log(p/p0)): 60 FP64 issue slots against 116 with pow and two
+// T exp(-(R/cp) log(p/p0)): 64 FP64 issue slots against 116 with pow and two
 // divisions (92 and 12 of them; log 30, exp 15), two thirds of the indicator.
-// There |log| < 1/2, so the roundings of the logarithm and of the product
-// reach the result below a quarter of its last place; farther out they would
-// not, and pow stays.
+// |log| is at most 0.511 there, so its last place and the product's reach the
+// result times R/cp < 0.3; the rounding of the quotient w is taken out to first
+// order, (p/p0 - w)/w with 1/w ~ 2 - w, which leaves less than that of pow's own
+// argument (tests/test_gpu_device_functions.py: rms and largest error below
+// pow's).  Farther out pow stays.
 __device__ __forceinline__ double theta_of(const double q[4], double z, const Phys& P) {
     const double rinv = fx_rcp(q[0]);
     const double gz = P.gravity ? __dmul_rn(P.g, z) : 0.0;
@@ -45,7 +47,10 @@ __device__ __forceinline__ double theta_of(const double q[4], double z, const Ph
     const double p = __dmul_rn(P.gm1, __dsub_rn(__dsub_rn(q[3], ke), __dmul_rn(q[0], gz)));
     const double T = __dmul_rn(__dmul_rn(p, rinv), P.invR);
     const double w = __dmul_rn(p, P.inv_p0);
-    if (w > 0.6 && w < 1.65) return __dmul_rn(T, exp(__dmul_rn(-P.Rcp, log(w))));
+    if (w > 0.6 && w < 1.65) {
+        const double dw = __dmul_rn(__fma_rn(-P.p0, w, p), P.inv_p0);  // p/p0 - w
+        return __dmul_rn(T, exp(__dmul_rn(-P.Rcp, __fma_rn(dw, __dsub_rn(2.0, w), log(w)))));
+    }
     return __dmul_rn(T, pow(__ddiv_rn(P.p0, p), P.Rcp));
 }
 
