@@ -519,12 +519,6 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
     pdl_trigger();
 }
 
-struct Phys3f {
-    float gamma, gm1, R, invR, mu, kappa, g, lamv, dTdz;
-    float inv_h[3], eta[3];
-    int gravity;
-};
-
 struct Bg3m {
     const double* rb;   // [nz][n] rhobar at nodes (FP64, for the split)
     const double* Eb;   // [nz][n] Ebar = pbar/(gamma-1) + rhobar g z
@@ -798,44 +792,6 @@ struct Cfg3m {
     // 123 / 155 with 1 / 2 / 3 / 5, degree 4 on 13^3 209 / 187 / 187 / 286
     static constexpr int minb = N == 2 ? 4 : N == 3 ? 3 : N == 4 ? 2 : 1;
 };
-
-// Fluxes on perturbations: the FP32 form of ns_flux9.
-struct Fx3FluxF {
-    float t[6], e[3];
-};
-__device__ __forceinline__ Fx3FluxF ns_flux9_pert(const float q[5], const float g[3][5], float gz, float rb, float Eb,
-                                                  float Hb, const Phys3f& P) {
-    const float rho = rb + q[0];
-    const float rinv = rcp_fast(rho);
-    const float v[3] = {q[1] * rinv, q[2] * rinv, q[3] * rinv};
-    const float ke2 = fmaf(q[3], v[2], fmaf(q[2], v[1], q[1] * v[0]));
-    const float pp = P.gm1 * fmaf(-0.5f, ke2, fmaf(-gz, q[0], q[4]));
-    const float H = Hb + (q[4] + pp), eR = (Eb + q[4]) * rinv;
-    float w[3][3];  // w[a][b], rho times the velocity gradient
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b) w[a][b] = fmaf(-v[a], g[b][0], g[b][1 + a]);
-    const float m23 = (2.0f / 3.0f) * P.mu * rinv, mr = -P.mu * rinv, kr = P.gm1 * P.kappa * P.invR * rinv;
-    const float div = w[0][0] + w[1][1] + w[2][2];
-    const float sd[3] = {m23 * fmaf(-3.0f, w[0][0], div), m23 * fmaf(-3.0f, w[1][1], div), m23 * fmaf(-3.0f, w[2][2], div)};
-    const float sxy = mr * (w[0][1] + w[1][0]), sxz = mr * (w[0][2] + w[2][0]), syz = mr * (w[1][2] + w[2][1]);
-    Fx3FluxF f;
-    f.t[0] = fmaf(q[1], v[0], pp + sd[0]);
-    f.t[1] = fmaf(q[1], v[1], sxy);
-    f.t[2] = fmaf(q[1], v[2], sxz);
-    f.t[3] = fmaf(q[2], v[1], pp + sd[1]);
-    f.t[4] = fmaf(q[2], v[2], syz);
-    f.t[5] = fmaf(q[3], v[2], pp + sd[2]);
-    const float so[3][2] = {{sxy, sxz}, {sxy, syz}, {sxz, syz}};
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-        float h = fmaf(-v[2], w[2][b], fmaf(-v[1], w[1][b], fmaf(-v[0], w[0][b], fmaf(-eR, g[b][0], g[b][4]))));
-        if (b == 2) h = fmaf(-P.g, rho, h);
-        f.e[b] = fmaf(-kr, h, fmaf(v[b], H + sd[b], fmaf(v[b == 0 ? 1 : 0], so[b][0], v[b == 2 ? 1 : 2] * so[b][1])));
-    }
-    return f;
-}
 
 template <int N>
 __global__ void __launch_bounds__(Cfg3<N>::threads, Cfg3m<N>::minb)

@@ -2,6 +2,7 @@
 // tests/test_gpu_device_functions.py.
 #include <cuda_runtime.h>
 
+#include "adg_mixed_point.cuh"
 #include "adg_tv_cell.cuh"
 
 using namespace adg;
@@ -23,5 +24,20 @@ extern "C" int dev_theta(const double* p, double* out, int n, double p0, double 
     P.inv_p0 = 1.0 / p0;
     P.Rcp = Rcp;
     k_theta<<<(n + 127) / 128, 128>>>(p, out, n, P);
+    return (int)cudaDeviceSynchronize();
+}
+
+// rho u v of the 3D mixed flux with rho u = rho v = 1 and no viscosity: 1/rho
+__global__ void k_flux3_rcp(const float* rho, float* out, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const Phys3f P = {};
+    const float q[5] = {rho[i], 1.0f, 1.0f, 0.0f, 0.0f};
+    const float g[3][5] = {};
+    out[i] = ns_flux9_pert(q, g, 0.0f, 0.0f, 0.0f, 0.0f, P).t[1];
+}
+
+extern "C" int dev_flux3_rcp(const float* rho, float* out, int n) {
+    k_flux3_rcp<<<(n + 127) / 128, 128>>>(rho, out, n);
     return (int)cudaDeviceSynchronize();
 }

@@ -44,3 +44,16 @@ def test_theta_is_as_accurate_as_pow(dev, lo, hi):
     rms, top = np.sqrt((err ** 2).mean(1)), np.abs(err).max(1)
     print(f"rms {rms}, largest {top}")
     assert rms[0] <= rms[1] and top[0] <= top[1]
+
+
+def test_3d_mixed_flux_divides_by_the_density_correctly_rounded(dev):
+    """1/rho of the 3D mixed flux (rho u v with both momenta 1) is the nearest
+    float, over the densities of gases and far from them."""
+    rng = np.random.default_rng(3)
+    rho = np.concatenate([rng.uniform(0.5, 1.5, 20000), 2.0 ** rng.uniform(-120, 120, 20000)]).astype(np.float32)
+    x = torch.from_numpy(rho).cuda()
+    out = torch.empty_like(x)
+    torch.cuda.synchronize()
+    assert dev.dev_flux3_rcp(_p(x), _p(out), rho.size) == 0
+    # 1/rho in 64 bits rounds to the nearest float unless it lies within 2^-53 of a tie, which 24-bit rho rule out
+    assert np.array_equal(out.cpu().numpy(), (1.0 / rho.astype(np.float64)).astype(np.float32))
