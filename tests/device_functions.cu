@@ -41,3 +41,36 @@ extern "C" int dev_flux3_rcp(const float* rho, float* out, int n) {
     k_flux3_rcp<<<(n + 127) / 128, 128>>>(rho, out, n);
     return (int)cudaDeviceSynchronize();
 }
+
+// adg_fixed.cuh: reciprocal; fixed point from a double and its limbs; double from fixed point
+__global__ void k_rcp(const double* x, double* out, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = fx_rcp(x[i]);
+}
+__global__ void k_from(const double* x, const int* E, long long* m, int* limbs, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    m[i] = fx_from(x[i], E[i]);
+    const Limbs a = fx_split(m[i]), b = fx_split_centred(m[i]);
+    limbs[4 * i] = a.h;
+    limbs[4 * i + 1] = a.l;
+    limbs[4 * i + 2] = b.h;
+    limbs[4 * i + 3] = b.l;
+}
+__global__ void k_to(const long long* a, const int* e, double* out, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = fx_to(a[i], e[i]);
+}
+
+extern "C" int dev_rcp(const double* x, double* out, int n) {
+    k_rcp<<<(n + 127) / 128, 128>>>(x, out, n);
+    return (int)cudaDeviceSynchronize();
+}
+extern "C" int dev_from(const double* x, const int* E, long long* m, int* limbs, int n) {
+    k_from<<<(n + 127) / 128, 128>>>(x, E, m, limbs, n);
+    return (int)cudaDeviceSynchronize();
+}
+extern "C" int dev_to(const long long* a, const int* e, double* out, int n) {
+    k_to<<<(n + 127) / 128, 128>>>(a, e, out, n);
+    return (int)cudaDeviceSynchronize();
+}

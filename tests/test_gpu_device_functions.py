@@ -1,8 +1,10 @@
 """Scalar device functions of the library (tests/device_functions.cu, compiled
 here with the library's flags) against exact values."""
 import ctypes
+import math
 import os
 from decimal import Decimal, localcontext
+from fractions import Fraction
 
 import numpy as np
 import pytest
@@ -57,3 +59,81 @@ def test_3d_mixed_flux_divides_by_the_density_correctly_rounded(dev):
     assert dev.dev_flux3_rcp(_p(x), _p(out), rho.size) == 0
     # 1/rho in 64 bits rounds to the nearest float unless it lies within 2^-53 of a tie, which 24-bit rho rule out
     assert np.array_equal(out.cpu().numpy(), (1.0 / rho.astype(np.float64)).astype(np.float32))
+
+
+def _doubles(rng, exps):
+    """Doubles of the given biased exponents with random and edge mantissas, both signs."""
+    e = np.repeat(np.asarray(exps, dtype=np.uint64), 8)
+    m = rng.integers(0, 1 << 52, e.size, dtype=np.uint64)
+    edge = np.array([0, 1, (1 << 52) - 1, 1 << 51, (1 << 29) - 1, 1 << 29], dtype=np.uint64)
+    k = np.arange(e.size) % 8
+    m = np.where(k < 6, edge[np.minimum(k, 5)], m)
+    s = rng.integers(0, 2, e.size, dtype=np.uint64)
+    return (s << np.uint64(63) | e << np.uint64(52) | m).view(np.float64)
+
+
+def test_reciprocal(dev):
+    """One Newton-like step of third order from 2^-22 leaves 2^-66, so the result
+    is within (1/2 + 2^-12) of its last place; subnormal, huge and special values
+    take the division."""
+    rng = np.random.default_rng(5)
+    x = np.concatenate([_doubles(rng, np.arange(2047)), [0.0, -0.0, np.inf, -np.inf, np.nan], rng.uniform(0.5, 2.0, 20000)])
+    t = torch.from_numpy(x).cuda()
+    out = torch.empty_like(t)
+    torch.cuda.synchronize()
+    assert dev.dev_rcp(_p(t), _p(out), x.size) == 0
+    got = out.cpu().numpy()
+    with np.errstate(divide="ignore", over="ignore"):
+        div = 1.0 / x
+    ex = (x.view(np.uint64) >> np.uint64(52) & np.uint64(0x7FF)).astype(int)
+    far = (ex == 0) | (ex > 2040)
+    assert np.array_equal(got[far], div[far], equal_nan=True)
+    for a, r in zip(x[~far].tolist(), got[~far].tolist()):
+        fr = Fraction(r)
+        assert abs(fr - 1 / Fraction(a)) <= (Fraction(1, 2) + Fraction(1, 4096)) * Fraction(math.ulp(r))
+
+
+def test_fixed_point_from_double(dev):
+    """m = x 2^(1080 - E) cut to an integer below 2^58, and both splits of it."""
+    rng = np.random.default_rng(6)
+    x = _doubles(rng, np.concatenate([[0], np.arange(200, 2047, 3)]))
+    ex = (x.view(np.uint64) >> np.uint64(52) & np.uint64(0x7FF)).astype(int)
+    E = np.maximum(ex + rng.choice([0, 1, 2, 5, 30, 57, 58, 63, 300], x.size), 256).astype(np.int32)
+    tx, tE = torch.from_numpy(x).cuda(), torch.from_numpy(E).cuda()
+    m = torch.empty(x.size, dtype=torch.int64, device="cuda")
+    limbs = torch.empty(x.size, 4, dtype=torch.int32, device="cuda")
+    torch.cuda.synchronize()
+    assert dev.dev_from(_p(tx), _p(tE), _p(m), _p(limbs), x.size) == 0
+    for a, e, k, (h, l, ch, cl) in zip(x.tolist(), E.tolist(), m.cpu().tolist(), limbs.cpu().tolist()):
+        want = abs(Fraction(a)) * Fraction(2) ** (1080 - e) if abs(a) >= 2.0 ** -1022 else 0
+        assert abs(k) == int(want) < 1 << 58 and (k == 0 or (k < 0) == (a < 0))
+        assert h * (1 << 29) + l == k and 0 <= l < 1 << 29
+        assert ch * (1 << 29) + cl == k and abs(cl) <= 1 << 28 and abs(ch) <= 1 << 29
+
+
+def test_double_from_fixed_point(dev):
+    """a 2^e rounds to the nearest double, ties away from zero; NaN above the
+    range, zero below the normal numbers."""
+    rng = np.random.default_rng(8)
+    bits = np.tile(np.arange(1, 63), 60)
+    a = np.array([int(rng.integers(1 << (b - 1), 1 << b)) for b in bits.tolist()])
+    pat = np.arange(a.size) % 6
+    a = np.where(pat == 0, 1 << (bits - 1), np.where(pat == 1, (1 << bits) - 1, a))
+    a = np.where(rng.random(a.size) < 0.5, -a, a)
+    e = rng.integers(-1100, 1050, a.size).astype(np.int32)
+    a, e = np.append(a, [0, 0]), np.append(e, [0, 30000]).astype(np.int32)
+    ta, te = torch.from_numpy(a).cuda(), torch.from_numpy(e).cuda()
+    out = torch.empty(a.size, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    assert dev.dev_to(_p(ta), _p(te), _p(out), a.size) == 0
+    for m, x, r in zip(a.tolist(), e.tolist(), out.cpu().tolist()):
+        top = abs(m).bit_length() + x  # |a 2^e| in [2^(top - 1), 2^top)
+        if (m == 0 and x < 2046) or (m and top - 1 < -1022):
+            assert r == 0.0
+        elif m == 0 or top > 1024:
+            assert math.isnan(r)
+        else:
+            cut = max(abs(m).bit_length() - 53, 0)
+            mag = (abs(m) + (1 << cut >> 1)) >> cut
+            want = Fraction(mag) * Fraction(2) ** (x + cut) * (1 if m > 0 else -1)
+            assert Fraction(r) == want if want < Fraction(2) ** 1024 else math.isinf(r)
