@@ -1006,9 +1006,13 @@ __device__ __forceinline__ void corrector_amr_body(double* __restrict__ u, const
     }
 }
 
+// Two blocks per SM asked at degrees 3 and 5 (us, unstated -> two): ten degree-5
+// steps and the indicator on the two-bubble tree of 1489 leaves 537 -> 519 (three
+// 537), a step on 153 leaves 37.2 -> 35.3 but on 5508 123.5 -> 125.3; degree 3 on
+// 5508 leaves 45.5 -> 43.4.  Degrees 6 and 7 lose (5508 leaves 276.7 -> 279.2,
+// 274.8 -> 275.8), the others are indifferent, as is k_tv_cells_amr.
 template <int N, int CPB>
-// (two blocks per SM asked: ten adaptive degree-5 steps and the indicator 519 us, 537 with three or unstated)
-__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1), 2)
+__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1), N == 3 || N == 5 ? 2 : 1)
 k_corrector_amr(double* __restrict__ u, const double* rvol, const double* trace, int cells, double dt, const Basis B,
                 const Phys P0, const AmrOps O, const double* __restrict__ geo, const int* __restrict__ nbr,
                 const double* __restrict__ bgl) {
@@ -1026,7 +1030,7 @@ k_corrector_amr_lts(double* __restrict__ u, const double* __restrict__ rvol, con
 }
 
 template <int N, int CPB>
-__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1), 2)
+__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1))
 k_tv_cells_amr(const double* __restrict__ u, double* __restrict__ tv, double* __restrict__ part, int cells,
                int var, const Basis B, const Phys P0, const double* __restrict__ geo) {
     static_assert(CPB == tv_cpb(N), "the TV statistics combine blocks of tv_cpb(N) cells");

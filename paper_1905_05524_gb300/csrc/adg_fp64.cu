@@ -275,9 +275,18 @@ __device__ __forceinline__ void corrector_fp64_body(double* __restrict__ u, cons
     }
 }
 
+// Blocks per SM asked of the register allocator, only where several waves gain
+// from it: step with indicator, us, unstated -> six: degree 2 81x81 181 -> 171,
+// degree 5 40x40 381 -> 371, 81x81 1356 -> 1343.  Elsewhere the spills cost more
+// than the occupancy gives: 9x9 cells degree 1 31.2 -> 33.1, 2 35.2 -> 36.9 (step
+// alone), 4 39.3 -> 41.3; degrees 3, 6 and 7 within 1% either way.
+template <int N, bool TV>
+constexpr int corr_resident() {
+    return N == 5 || (N == 2 && TV) ? 6 : 1;
+}
+
 template <int N, int CPB, bool TV>
-// (six blocks per SM asked: 81x81 degree-5 step with indicator 1303 us, 1309 with five, 1317 unstated)
-__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1), 6)
+__global__ void __launch_bounds__(CPB*(N + 1) * (N + 1), (corr_resident<N, TV>()))
 k_corrector_fp64(double* __restrict__ u, const double* rvol, const double* trace, int cells, double dt, const Basis B,
                  const Phys P, const Background bg, const TvEpilogue epi, double t) {
     pdl_wait();  // the predictor's residual and traces are complete and visible
