@@ -175,10 +175,20 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
 #pragma unroll
         for (int v = 0; v < 4; ++v) push(v, fx_mag(q[v]));
     };
-    int EQ[4];
+    // Exponents of q (slots 0..3) and the fluxes (4..8), a phase's magnitudes cleared in the phase after the next
+    // barrier.  From degree 5 on they are formed again wherever they are used: held through a sweep they would spill
+    // (81x81 step, us: degree 5 1281 -> 1272, degree 7 4092 -> 3956; degree 2 with registers to spare 150 -> 148 held).
+    int EE[9];
+    auto take = [&](int first, int end) {
+        if constexpr (N <= 4) {
+#pragma unroll
+            for (int c = first; c < end; ++c) EE[c] = fx_exp(mx[c]);
+        }
+    };
+    auto E = [&](int slot) { return N <= 4 && slot < 9 ? EE[slot] : fx_exp(mx[slot]); };
     auto store_q = [&](int slice) {
 #pragma unroll
-        for (int v = 0; v < 4; ++v) Q[(v * n + slice) * n2 + node] = fx_limbs(q[v], EQ[v]);
+        for (int v = 0; v < 4; ++v) Q[(v * n + slice) * n2 + node] = fx_limbs(q[v], E(v));
     };
     for (int a = tid; a < 13; a += C::tpc) mx[a] = 0;
     __syncthreads();
@@ -194,15 +204,13 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
         push(12, fx_mag(Sm[3]));
     }
     __syncthreads();
-#pragma unroll
-    for (int v = 0; v < 4; ++v) EQ[v] = fx_exp(mx[v]);
+    take(0, 4);
     if (id < n2 && on) {
         store_q(0);
 #pragma unroll
         for (int v = 0; v < 4; ++v) US[v * n2 + node] = q[v];
     }
     __syncthreads();
-    if (tid < 4) mx[tid] = 0;
 
     FxFlux f;
     // sweeps 0..n-1 and the final evaluation r = n; in sweep 0 the iterate is u
@@ -211,11 +219,9 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
     for (int r = 0;; ++r) {
         const int ks = r == 0 ? 0 : k;
         const Limbs* Qk = Q + ks * n2;
-        // exponents of the residual (fx_sum_exp of the two derivatives and the source)
-        const int X0 = EQ[1] + O.ex - 1022 + O.shx, Y0 = EQ[2] + O.ey - 1022 + O.shy;
-        int ER[4];
-        ER[0] = max(max(X0, Y0), has_src ? fx_exp(mx[10]) + 1 : 0);
-        const int sx0 = fx_down(O.shx, ER[0], X0), sy0 = fx_down(O.shy, ER[0], Y0);
+        int ER[4];  // exponents of the residual: the largest of its two derivatives' and the source's
+        const int dX = O.ex - 1022 + O.shx, dY = O.ey - 1022 + O.shy;
+        ER[0] = max(max(E(1) + dX, E(2) + dY), has_src ? E(10) + 1 : 0);
         long long R[4];  // -dF/dx - dG/dy + S; the mass flux is the momentum
         f = FxFlux{0.0, 0.0, 0.0, 0.0, 0.0};
         if (r == 0 && k > 0) {
@@ -225,7 +231,7 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
                 a.add(O.dx[i * n + p], Qk[n3 + j * n + p]);
                 b.add(O.dy[j * n + p], Qk[2 * n3 + p * n + i]);
             }
-            R[0] = -(a.value() >> sx0) - (b.value() >> sy0);
+            R[0] = -(a.value() >> fx_down(O.shx, ER[0], E(1) + dX)) - (b.value() >> fx_down(O.shy, ER[0], E(2) + dY));
         } else {
             double gx[4], gy[4];
             {
@@ -236,9 +242,9 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
 #pragma unroll
                     for (int v = 0; v < 4; ++v) a[v].add(d, Qk[v * n3 + j * n + p]);
                 }
-                R[0] = -(a[1].value() >> sx0);
+                R[0] = -(a[1].value() >> fx_down(O.shx, ER[0], E(1) + dX));
 #pragma unroll
-                for (int v = 0; v < 4; ++v) gx[v] = fx_to(a[v].value(), EQ[v] + O.ex - 2102);
+                for (int v = 0; v < 4; ++v) gx[v] = fx_to(a[v].value(), E(v) + O.ex - 2102);
             }
             {
                 FxSum a[4];
@@ -248,9 +254,9 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
 #pragma unroll
                     for (int v = 0; v < 4; ++v) a[v].add(d, Qk[v * n3 + p * n + i]);
                 }
-                R[0] -= a[2].value() >> sy0;
+                R[0] -= a[2].value() >> fx_down(O.shy, ER[0], E(2) + dY);
 #pragma unroll
-                for (int v = 0; v < 4; ++v) gy[v] = fx_to(a[v].value(), EQ[v] + O.ey - 2102);
+                for (int v = 0; v < 4; ++v) gy[v] = fx_to(a[v].value(), E(v) + O.ey - 2102);
             }
             f = ns_flux5(q, gx, gy, g, gz, pbar, P.gm1, P.mu, mu23, kR);
         }
@@ -262,42 +268,46 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
         for (int c = 0; c < 5; ++c) push(4 + c, fx_mag(fl[c]));
         if (has_src || P.gravity) push(9, fx_mag(S2));
         __syncthreads();
-        int EF[5];
-#pragma unroll
-        for (int c = 0; c < 5; ++c) EF[c] = fx_exp(mx[4 + c]);
-        const int ES2 = has_src || P.gravity ? fx_exp(mx[9]) + 1 : 0;
+        take(4, 9);
+        if (tid < 4) mx[tid] = 0;
         if (on && (r > 0 || k == 0)) {
 #pragma unroll
-            for (int c = 0; c < 5; ++c) F[(c * n + k) * n2 + node] = fx_limbs(fl[c], EF[c]);
+            for (int c = 0; c < 5; ++c) F[(c * n + k) * n2 + node] = fx_limbs(fl[c], E(4 + c));
         }
         __syncthreads();
-        if (tid < 6) mx[4 + tid] = 0;
         // residual, in Q's place
         {
-            const int dX = O.ex - 1022 + O.shx, dY = O.ey - 1022 + O.shy;
-            const int X[3] = {EF[0] + dX, EF[1] + dX, EF[2] + dX}, Y[3] = {EF[1] + dY, EF[3] + dY, EF[4] + dY};
-            ER[1] = max(max(X[0], Y[0]), has_src ? fx_exp(mx[11]) + 1 : 0);
-            ER[2] = max(max(X[1], Y[1]), ES2);
-            ER[3] = max(max(X[2], Y[2]), has_src ? fx_exp(mx[12]) + 1 : 0);
-            FxSum a[3], b[3];
-            const Limbs* Fx = F + ks * n2 + j * n;
-            const Limbs* Gy = F + ks * n2 + i;
+            // fluxes of residual v: F1 XY F3 along x, XY G2 G3 along y
+            auto X = [&](int v) { return E(3 + v) + dX; };
+            auto Y = [&](int v) { return E(v == 1 ? 5 : 5 + v) + dY; };
+            ER[1] = max(max(X(1), Y(1)), has_src ? E(11) + 1 : 0);
+            ER[2] = max(max(X(2), Y(2)), has_src || P.gravity ? E(9) + 1 : 0);
+            ER[3] = max(max(X(3), Y(3)), has_src ? E(12) + 1 : 0);
+            {
+                FxSum a[3];
+                const Limbs* Fx = F + ks * n2 + j * n;
 #pragma unroll
-            for (int p = 0; p < n; ++p) {
-                const Limbs d = O.dx[i * n + p];
+                for (int p = 0; p < n; ++p) {
+                    const Limbs d = O.dx[i * n + p];
 #pragma unroll
-                for (int v = 0; v < 3; ++v) a[v].add(d, Fx[v * n3 + p]);
+                    for (int v = 0; v < 3; ++v) a[v].add(d, Fx[v * n3 + p]);
+                }
+#pragma unroll
+                for (int v = 1; v < 4; ++v) R[v] = -(a[v - 1].value() >> fx_down(O.shx, ER[v], X(v)));
             }
+            {
+                FxSum a[3];
+                const Limbs* Gy = F + ks * n2 + i;
 #pragma unroll
-            for (int p = 0; p < n; ++p) {
-                const Limbs d = O.dy[j * n + p];
-                b[0].add(d, Gy[n3 + p * n]);
-                b[1].add(d, Gy[3 * n3 + p * n]);
-                b[2].add(d, Gy[4 * n3 + p * n]);
+                for (int p = 0; p < n; ++p) {
+                    const Limbs d = O.dy[j * n + p];
+                    a[0].add(d, Gy[n3 + p * n]);
+                    a[1].add(d, Gy[3 * n3 + p * n]);
+                    a[2].add(d, Gy[4 * n3 + p * n]);
+                }
+#pragma unroll
+                for (int v = 1; v < 4; ++v) R[v] -= a[v - 1].value() >> fx_down(O.shy, ER[v], Y(v));
             }
-#pragma unroll
-            for (int v = 0; v < 3; ++v)
-                R[v + 1] = -(a[v].value() >> fx_down(O.shx, ER[v + 1], X[v])) - (b[v].value() >> fx_down(O.shy, ER[v + 1], Y[v]));
         }
         if (has_src) {
             R[0] += fx_from(Sm[0], ER[0]);
@@ -325,11 +335,10 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
         }
         push_q();
         __syncthreads();
-#pragma unroll
-        for (int v = 0; v < 4; ++v) EQ[v] = fx_exp(mx[v]);
+        take(0, 4);
+        if (tid < 6) mx[4 + tid] = 0;
         if (on) store_q(k);
         __syncthreads();
-        if (tid < 4) mx[tid] = 0;
     }
 
     // time averages: slots q (4), F1, XY, F3, G2, G3, then the time-dependent source
