@@ -575,9 +575,9 @@ __device__ __forceinline__ void ns_flux3f(const float q[5], const float g[3][5],
 // MX: the mixed-precision form -- Rusanov flux from the FP64 jump of the
 // face states converted to FP32, flux average and lifting in FP32, the
 // update in FP64 (ghost states stay FP64).
-template <int N, bool MX>
-// blocks per SM: 25^3 degree 2 mixed 157.9 / 154.9 / 153.9 / 156.8 us a step with 2 / 3 / 4 / 5
-__global__ void __launch_bounds__(Cfg3<N>::threads, (MX && N <= 2 ? 4 : 2))
+// MINB: blocks per SM asked of the register allocator (launch3).
+template <int N, bool MX, int MINB>
+__global__ void __launch_bounds__(Cfg3<N>::threads, MINB)
 k3_corrector(double* __restrict__ u, const double* rvol_in, const double* trace_in, int cells, double dt, double t,
               const Basis B, const Phys3 P, const Bg3 bg, const Phys3f Pf) {
     using C = Cfg3<N>;
@@ -1175,8 +1175,13 @@ int launch3(bool pred, double* u, double* rvol, double* trace, int cells, double
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        const cudaError_t e = mixed ? cudaLaunchKernelEx(&cfg, k3_corrector<N, true>, u, rvol, trace, cells, dt, t, B, P, bg, Pf)
-                                    : cudaLaunchKernelEx(&cfg, k3_corrector<N, false>, u, rvol, trace, cells, dt, t, B, P, bg, Pf);
+        // Mixed, degrees 1 and 2: four blocks an SM (25^3 degree-2 bubble, us a step, 157.9 / 154.9 / 153.9 / 156.8
+        // with 2 / 3 / 4 / 5), but two where the analytic field is evaluated on the boundary, whose registers would
+        // spill (25^3 ABC flow 432 / 447 / 498 with 2 / 3 / 4, degree 1 122 / 122 / 135).
+        constexpr int kMany = N <= 2 ? 4 : 2;
+        const bool analytic = P.bc[0] == ADG_BC_ANALYTIC || P.bc[1] == ADG_BC_ANALYTIC || P.bc[2] == ADG_BC_ANALYTIC;
+        auto kern = !mixed ? k3_corrector<N, false, 2> : analytic ? k3_corrector<N, true, 2> : k3_corrector<N, true, kMany>;
+        const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, u, rvol, trace, cells, dt, t, B, P, bg, Pf);
         if (e != cudaSuccess) return (int)e;
     }
     return (int)cudaGetLastError();
