@@ -203,20 +203,23 @@ static int upload_tables(adg_mesh* m) {
         }
         return r;
     };
+    // hx, hy, their reciprocals and the penalties depend on the level alone: divided once a level, not in every leaf
+    // or thread (in the kernels four divisions a thread cost the corrector more than its faces)
+    std::vector<std::array<double, 6>> lev(T->maxl + 1);
+    for (int l = 0; l <= T->maxl; ++l) {
+        const double hx = d->Lx / (d->nx * AmrTree::ipow3(l)), hy = d->Ly / (d->ny * AmrTree::ipow3(l));
+        lev[l] = {hx, hy, 1.0 / hx, 1.0 / hy, (2.0 * m->N + 1.0) / (hx * 1.2533141373155002),  // sqrt(pi/2)
+                  (2.0 * m->N + 1.0) / (hy * 1.2533141373155002)};
+    }
     double hmin = 1e300;
     for (int k = 0; k < L; ++k) {
         const int l = T->leaves[k][0], ix = T->leaves[k][1], iy = T->leaves[k][2];
-        const double hx = d->Lx / (d->nx * AmrTree::ipow3(l)), hy = d->Ly / (d->ny * AmrTree::ipow3(l));
+        const double hx = lev[l][0], hy = lev[l][1];
         hmin = std::fmin(hmin, std::fmin(hx, hy));
         double* g = &geo[(size_t)k * kGeo];
         g[0] = d->x0 + ix * hx;
         g[1] = d->y0 + iy * hy;
-        g[2] = hx;
-        g[3] = hy;
-        g[4] = 1.0 / hx;  // divided once here: four divisions a thread cost the corrector more than its faces
-        g[5] = 1.0 / hy;
-        g[6] = (2.0 * m->N + 1.0) / (hx * 1.2533141373155002);  // sqrt(pi/2)
-        g[7] = (2.0 * m->N + 1.0) / (hy * 1.2533141373155002);
+        std::copy(lev[l].begin(), lev[l].end(), g + 2);
         const std::vector<double>& r = row_of(l, iy, hy);
         for (int j = 0; j < n; ++j) {
             bgl[((size_t)k * n + j) * 2] = r[(size_t)j * 2];
