@@ -17,7 +17,7 @@
 //
 // NaN or infinity anywhere in a group makes every result of the group NaN (an
 // FP64 contraction spreads it to the node's row and column, the following
-// sweeps to the cell).  Groups below 2^-767 count as zero.
+// sweeps to the cell).  Groups below 2^-958 count as zero.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -29,7 +29,9 @@ struct Limbs {
     int h, l;  // m = h 2^29 + l
 };
 
-constexpr int kFxMinExp = 256;      // smallest group exponent (biased as in a double)
+// smallest group exponent (biased as in a double); at least 58, so that zeros and subnormals, whose
+// leading bit fx_from takes for set, shift out
+constexpr int kFxMinExp = 64;
 constexpr int kFxBadExp = 0x4000;   // group exponent of a group with NaN or infinity
 
 // Order of magnitude as an unsigned integer: exponent and 20 bits of mantissa.
