@@ -63,6 +63,7 @@ struct AmrTree {
     // per (level, iy) row: the background tables of upload_tables (they depend
     // on the height only), computed once
     std::unordered_map<long long, std::vector<double>> rows;
+    std::vector<double> geo;  // upload_tables' leaf geometry, rewritten by each call (kept: its pages are touched once)
     AmrOps ops;
 
     static long long key(int l, int ix, int iy) { return ((long long)l << 50) | ((long long)ix << 25) | iy; }
@@ -146,7 +147,9 @@ static int upload_tables(adg_mesh* m) {
     const int L = (int)T->leaves.size(), n = m->n;
     const adg_mesh_desc* d = &m->d;
     const bool mixed = d->precision == ADG_PREC_MIXED;
-    std::vector<double> geo((size_t)L * kGeo), bgl((size_t)L * n * 2 + (size_t)L * 4, 0.0);
+    std::vector<double>& geo = T->geo;
+    geo.resize((size_t)L * kGeo);
+    std::vector<double> bgl((size_t)L * n * 2 + (size_t)L * 4, 0.0);
     std::vector<int> nbr((size_t)L * 4 * kNbrInts);
     std::vector<double> h64(mixed ? (size_t)L * n * 2 + (size_t)L * 4 : 0, 0.0);
     std::vector<float> h32(mixed ? (size_t)L * n * 3 + (size_t)L * 4 : 0, 0.0f);
