@@ -296,28 +296,32 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
         double q[5];
 #pragma unroll
         for (int v = 0; v < 5; ++v) q[v] = u[(size_t)cell * SL + v * n3 + node];
-        int EQ[5];
+        // exponents of q (slots 0..4) and the fluxes (5..13); a phase's magnitudes are cleared in the phase after the
+        // next barrier
+        int E[14] = {};
+        auto take = [&](int first, int end) {
+#pragma unroll
+            for (int c = first; c < end; ++c) E[c] = fx_exp(mx[c]);
+        };
         auto push_q = [&]() {
 #pragma unroll
             for (int v = 0; v < 5; ++v) push(v, fx_mag(q[v]));
         };
         auto store_q = [&](int slice) {
 #pragma unroll
-            for (int v = 0; v < 5; ++v) Q[(v * n + slice) * n3 + node] = fx_limbs(q[v], EQ[v]);
+            for (int v = 0; v < 5; ++v) Q[(v * n + slice) * n3 + node] = fx_limbs(q[v], E[v]);
         };
         if (tid < 15) mx[tid] = 0;
         __syncthreads();
         push_q();
         __syncthreads();
-#pragma unroll
-        for (int v = 0; v < 5; ++v) EQ[v] = fx_exp(mx[v]);
+        take(0, 5);
         if (id < n3 && on) {
             store_q(0);
 #pragma unroll
             for (int v = 0; v < 5; ++v) US[v * n3 + node] = q[v];
         }
         __syncthreads();
-        if (tid < 5) mx[tid] = 0;
 
         Fx3Flux f;
         // sweeps 0..n-1 and the final evaluation r = n; in sweep 0 the iterate is
@@ -327,7 +331,7 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
             const int ks = r == 0 ? 0 : k;
             const Limbs* Qk = Q + ks * n3;
             int ER[5];  // exponents of the residual: the largest of its derivatives' and the source's
-            ER[0] = max(EQ[1] + ed[0] + sh[0], max(EQ[2] + ed[1] + sh[1], EQ[3] + ed[2] + sh[2])) - 1022;
+            ER[0] = max(E[1] + ed[0] + sh[0], max(E[2] + ed[1] + sh[1], E[3] + ed[2] + sh[2])) - 1022;
             long long R[5];  // -div F + S; the mass flux is the momentum
             R[0] = 0;
 #pragma unroll
@@ -341,7 +345,7 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
                     FxSum a;
 #pragma unroll
                     for (int p = 0; p < n; ++p) a.add(D[p], L[p * (b == 0 ? 1 : b == 1 ? n : n2)]);
-                    R[0] -= a.value() >> fx_down(sh[b], ER[0], EQ[1 + b] + ed[b] + sh[b] - 1022);
+                    R[0] -= a.value() >> fx_down(sh[b], ER[0], E[1 + b] + ed[b] + sh[b] - 1022);
                 }
             } else {
                 double g[3][5];
@@ -356,9 +360,9 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
 #pragma unroll
                         for (int v = 0; v < 5; ++v) a[v].add(d, L[v * n4 + p * (b == 0 ? 1 : b == 1 ? n : n2)]);
                     }
-                    R[0] -= a[1 + b].value() >> fx_down(sh[b], ER[0], EQ[1 + b] + ed[b] + sh[b] - 1022);
+                    R[0] -= a[1 + b].value() >> fx_down(sh[b], ER[0], E[1 + b] + ed[b] + sh[b] - 1022);
 #pragma unroll
-                    for (int v = 0; v < 5; ++v) g[b][v] = fx_to(a[v].value(), EQ[v] + ed[b] - 2102);
+                    for (int v = 0; v < 5; ++v) g[b][v] = fx_to(a[v].value(), E[v] + ed[b] - 2102);
                 }
                 f = ns_flux9(q, g, gg, gz, pbar, P.gm1, P.mu, mu23, kR);
             }
@@ -369,23 +373,20 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
             for (int c = 0; c < 9; ++c) push(5 + c, fx_mag(fl[c]));
             if (P.gravity) push(14, fx_mag(S));
             __syncthreads();
-            int EF[9];
-#pragma unroll
-            for (int c = 0; c < 9; ++c) EF[c] = fx_exp(mx[5 + c]);
-            const int ES = P.gravity ? fx_exp(mx[14]) + 1 : 0;
+            take(5, 14);
+            if (tid < 5) mx[tid] = 0;
             if (on && (r > 0 || k == 0)) {
 #pragma unroll
-                for (int c = 0; c < 9; ++c) F[(c * n + k) * n3 + node] = fx_limbs(fl[c], EF[c]);
+                for (int c = 0; c < 9; ++c) F[(c * n + k) * n3 + node] = fx_limbs(fl[c], E[5 + c]);
             }
             __syncthreads();
-            if (tid < 10) mx[5 + tid] = 0;
             // residual, in Q's place; component v's flux in direction b
             auto fc = [](int v, int b) { return v < 4 ? fx3_t(v - 1, b) : 6 + b; };
 #pragma unroll
             for (int v = 1; v < 5; ++v) {
-                ER[v] = v == 3 ? ES : 0;
+                ER[v] = v == 3 && P.gravity ? fx_exp(mx[14]) + 1 : 0;
 #pragma unroll
-                for (int b = 0; b < 3; ++b) ER[v] = max(ER[v], EF[fc(v, b)] + ed[b] + sh[b] - 1022);
+                for (int b = 0; b < 3; ++b) ER[v] = max(ER[v], E[5 + fc(v, b)] + ed[b] + sh[b] - 1022);
                 R[v] = 0;
             }
 #pragma unroll
@@ -401,7 +402,7 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
                 }
 #pragma unroll
                 for (int v = 1; v < 5; ++v)
-                    R[v] -= a[v - 1].value() >> fx_down(sh[b], ER[v], EF[fc(v, b)] + ed[b] + sh[b] - 1022);
+                    R[v] -= a[v - 1].value() >> fx_down(sh[b], ER[v], E[5 + fc(v, b)] + ed[b] + sh[b] - 1022);
             }
             if (P.gravity) R[3] += fx_from(S, ER[3]);
             if (on) {
@@ -423,11 +424,10 @@ k3_predictor(const double* __restrict__ u, double* __restrict__ rvol, double* __
             }
             push_q();
             __syncthreads();
-#pragma unroll
-            for (int v = 0; v < 5; ++v) EQ[v] = fx_exp(mx[v]);
+            take(0, 5);
+            if (tid < 10) mx[5 + tid] = 0;
             if (on) store_q(k);
             __syncthreads();
-            if (tid < 5) mx[tid] = 0;
         }
 
         // time averages: slots q (5), t (6), e (3)
