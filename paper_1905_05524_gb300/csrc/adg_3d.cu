@@ -175,8 +175,8 @@ struct Fx3Cfg {
     static constexpr int cpb = N == 1 ? 8 : N == 2 ? 3 : 1;
     static constexpr int threads = (cpb * tpc + 31) / 32 * 32;
     // blocks per SM asked of the register allocator; us a step at 3 / 4 / 5 / 6: degree 1 (41^3 cells)
-    // 1098 / 1126 / 1144 / 1140, 2 (25^3) 1297 / 1281 / 1255 / 1301, 3 (17^3) 1299 / 1342 / 1279 / 1327;
-    // degree 4 (13^3) 2134 with 1, 2152 with 2
+    // 1121 / 1155 / 1153 / 1167, 2 (25^3) 1327 / 1299 / 1274 / 1322, 3 (17^3) 1328 / 1374 / 1308 / 1352;
+    // degree 4 (13^3) 2158 with 1 or 2, 2415 with 3
     static constexpr int resident = N == 1 ? 3 : N == 4 ? 1 : 5;
     // per cell, in 8-byte words: q (5) and the fluxes (9) of every space-time
     // node, u, D/h, the face values of q-bar, the magnitudes
@@ -787,9 +787,9 @@ struct Cfg3m {
     // nine fluxes of one slice, or the 29 averages (q', fluxes, grad q)
     static constexpr int fields = 5 * (N + 1) + 9 > 29 ? 5 * (N + 1) + 9 : 29;
     static constexpr size_t smem = (size_t)Cfg3<N>::cpb * fields * Cfg3<N>::n3 * sizeof(float);
-    // resident blocks asked of the register allocator (us a step): degree 2 on
-    // 25^3 cells 159 with 1, 3 or 4 and 177 with 5, degree 3 on 17^3 144 / 122 /
-    // 123 / 155 with 1 / 2 / 3 / 5, degree 4 on 13^3 209 / 187 / 187 / 286
+    // resident blocks asked of the register allocator (us a step with 1 / 2 / 3 / 4
+    // / 5): degree 2 on 25^3 cells 164 / 165 / 161 / 162 / 169, degree 3 on 17^3 155
+    // / 130 / 127 / 136 / 153, degree 4 on 13^3 188 / 190 / 191 / 203 / 243
     static constexpr int minb = N == 2 ? 4 : N == 3 ? 3 : N == 4 ? 2 : 1;
 };
 
@@ -888,8 +888,8 @@ k3_predictor_mixed(const double* __restrict__ u, double* __restrict__ rvol, doub
     }
     // Sweeps 2..n.  Degrees <= 2 accumulate the time contraction slice by
     // slice (the same order as a row-by-row sum), degree 1 with a rolled loop
-    // (142.0 against 145.5 us a step on 41^3 cells unrolled; degree 2 159.3
-    // rolled, 157.0 unrolled on 25^3); degrees 3 and 4 keep the residuals of all
+    // (152.5 against 154.9 us a step on 41^3 cells unrolled; degree 2 165.1
+    // rolled, 161.7 unrolled on 25^3); degrees 3 and 4 keep the residuals of all
     // slices in registers.
     constexpr int kSliceUnroll = N == 1 ? 1 : n;
 #pragma unroll 1

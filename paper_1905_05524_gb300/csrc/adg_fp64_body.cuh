@@ -25,9 +25,11 @@ struct FxCfg {
     // Blocks per SM asked of the register allocator.  The phases of a block
     // alternate between the FP64 and the integer pipe, so blocks in other
     // phases keep both busy: spilling registers for them pays.  Measured (us a
-    // launch, 81x81 cells): degree 5 1555 / 1263 / 1212 / 1200 / 1109 with 2 / 3
-    // / 4 / 5 / 8 blocks, degree 6 2569 / 2402 / 2197 / 2156 with 2 / 3 / 4 / 5,
-    // degree 7 4308 / 3886 / 3569 with 2 / 3 / 4; flat between 4 and 10 below.
+    // step, 81x81 cells): degree 5 1447 / 1376 / 1293 / 1286 / 1309 / 1273 with 2
+    // / 3 / 4 / 5 / 6 / 8 blocks, degree 6 2746 / 2552 / 2303 / 2340 with 2 / 3 / 4
+    // / 5 (five, for meshes of four to five blocks an SM: 27x27 284 against 345),
+    // degree 7 4496 / 4094 / 3965 with 2 / 3 / 4; degree 4 651 / 608 / 613 / 667
+    // with 3 / 4 / 5 / 6; within 5% from 3 to 10 below.
     static constexpr int resident = N == 1 ? 5 : N <= 4 ? 4 : N == 5 ? 8 : N == 6 ? 5 : 4;
     // per cell, in 8-byte words: q (4) and the fluxes (5) of every space-time
     // node, the source of the time-dependent form (4), u, D/hx, D/hy, the
@@ -178,7 +180,7 @@ __device__ __forceinline__ void predictor_fp64_body(const double* __restrict__ u
     // Exponents of q (slots 0..3) and the fluxes (4..8), a phase's magnitudes cleared in the phase after the next
     // barrier.  From degree 5 on they are formed again wherever they are used: held through a sweep they would spill
     // (81x81 step, us: degree 5 1281 -> 1272, degree 7 4092 -> 3956; degree 2 with registers to spare 150 -> 148 held).
-    int EE[9];
+    int EE[9] = {};
     auto take = [&](int first, int end) {
         if constexpr (N <= 4) {
 #pragma unroll

@@ -46,8 +46,12 @@ struct MixCfg2 {
     static constexpr int stride = raw + ((bank_off - raw % 32) + 32) % 32;  // a multiple of 4 floats
     static constexpr size_t smem_pred = (size_t)cpb * stride * sizeof(float);
     // resident blocks asked of the register allocator: four at N = 3 (128
-    // registers, 111.3 us per 243x243 launch; three 113.1), three at N = 5
-    // (642 us; four spill, 645), four at N = 7
+    // registers, 111.3 us per 243x243 launch; three 113.1), four at N = 7, three at
+    // N = 5, of whose blocks (60.5 KB) no fourth fits in shared memory.  More
+    // resident cells there cost more in spills than they hide: us a step on 60x60 /
+    // 81x81 / 243x243 cells 57.6 / 92.5 / 689 with three blocks of seven (168
+    // registers), 53.7 / 98.5 / 735 with four of six, 57.6 / 95.0 / 763 with five of
+    // five, 57.7 / 94.5 / 701 with three of seven at 128 registers
     // Meshes that do not fill the chip run smaller blocks, so that every SM and
     // sub-partition has some (up to small_cells per SM, all resident at once): a
     // degree-5 step on 9x9 cells 22.7 -> 19.1 us, on 40x40 36.0 -> 30.9, degree 3
