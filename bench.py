@@ -109,10 +109,10 @@ PREDICTOR_SOURCES = {
               "adg_internal.h"],
 }
 PREDICTOR_COUNTERS = {
-    "fp64": {"sha256": "fb06b3cfea322b0ca98a9ad4bca5aff9309306e186570cf75ada98a969e7d974",
-             "traffic": 17412608 + 156965632, "smem_frac": None},
-    "mixed": {"sha256": "b0628117c291aebe00fc07d72ffd668268acca3db774cf33c5cd318de257b8a2",
-              "traffic": 7679744 + 2048, "smem_frac": 0.672},
+    "fp64": {"sha256": "750d7af0f925a361d23a8f54012ab8f4e387eb6b58e8b645cea7a39a54a6d8f0",
+             "traffic": 17373440 + 160926976, "smem_frac": None},
+    "mixed": {"sha256": "5fca4f23fe911158708744da6bd1c8ab2ad2379c3a8de041bb0a88f5db38c07d",
+              "traffic": 7678464 + 3072, "smem_frac": 0.672},
 }
 
 
